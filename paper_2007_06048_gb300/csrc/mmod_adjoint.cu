@@ -30,11 +30,13 @@
 //     reversed step in two more volumes; the fewest replayed steps for S slots;
 //   segments with S >= nt and FP32 storage keeps g^n of every step (nt + 2
 //     volumes, written by the first sweep): no replay.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include <algorithm>
 #include <cfloat>
+#include <cstdint>
 #include <cstring>
 
 #include "mmod_handle.h"
@@ -56,75 +58,161 @@ __device__ __forceinline__ __half to_store<__half>(float v) { return __float2hal
 __device__ __forceinline__ float from_store(__nv_bfloat16 v) { return __bfloat162float(v); }
 __device__ __forceinline__ float from_store(__half v) { return __half2float(v); }
 
-// One CTA per plane: scale = max(max |u| over the plane, FLT_MIN), stored =
-// u / scale.
+__device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b) {
+    return (uint32_t)__bfloat16_as_ushort(a) | (uint32_t)__bfloat16_as_ushort(b) << 16;
+}
+__device__ __forceinline__ uint32_t pack2(__half a, __half b) {
+    return (uint32_t)__half_as_ushort(a) | (uint32_t)__half_as_ushort(b) << 16;
+}
+__device__ __forceinline__ uint32_t pack2(short a, short b) {
+    return (uint32_t)(unsigned short)a | (uint32_t)(unsigned short)b << 16;
+}
 template <class T>
-__global__ void compress_kernel(const float *__restrict__ u, long long plane, T *__restrict__ out,
-                                float *__restrict__ scale) {
-    const long long base = (long long)blockIdx.x * plane;
+__device__ __forceinline__ T stored_half(uint32_t w);
+template <>
+__device__ __forceinline__ __nv_bfloat16 stored_half<__nv_bfloat16>(uint32_t w) {
+    return __ushort_as_bfloat16((unsigned short)w);
+}
+template <>
+__device__ __forceinline__ __half stored_half<__half>(uint32_t w) { return __ushort_as_half((unsigned short)w); }
+template <>
+__device__ __forceinline__ short stored_half<short>(uint32_t w) { return (short)(unsigned short)w; }
+
+// The two volumes of a checkpoint (u^{a-1}, u^a), handled by one launch
+// (blockIdx.y selects the volume): each is a few microseconds of traffic, so
+// separate launches would cost as much as the work.
+template <class T>
+struct CkptPair {
+    float *u[2];
+    T *q[2];
+    float *scale[2];
+};
+
+// Scale = max(max |u| over the plane, FLT_MIN), stored = u / scale.  A cluster
+// of kPlaneCtas CTAs serves one plane: each takes the maximum of its share,
+// the shares meet through distributed shared memory, and the second pass
+// reads the plane again from L2.  Bound by memory; one CTA per plane left most
+// of the chip idle (a 133 x 144 x 120 volume is 120 planes of 92 KB).  That
+// form took 17.7 us per volume there and 15.4 us to restore it, with 4-byte
+// accesses; with clusters, 32 bytes per thread and access and one launch per
+// state, the gradient of that box (200 steps, binomial schedule, 10 BF16
+// slots) went from 24.4 to 18.5 ms.  Padded rows
+// are a multiple of 32 floats, so groups of 8 values tile a plane exactly and
+// start on 16-byte boundaries.
+constexpr int kPlaneCtas = 8;
+
+template <class T>
+__global__ void __cluster_dims__(kPlaneCtas, 1, 1) __launch_bounds__(256)
+    compress_kernel(const CkptPair<T> p, long long plane) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int k = blockIdx.x / kPlaneCtas, rank = blockIdx.x % kPlaneCtas, vol = blockIdx.y;
+    const float4 *u = reinterpret_cast<const float4 *>(p.u[vol] + (long long)k * plane);
+    const long long groups = plane >> 3;
+    const int first = rank * 256 + threadIdx.x;
     float m = 0.0f;
-    for (long long q = threadIdx.x; q < plane; q += blockDim.x) m = fmaxf(m, fabsf(u[base + q]));
-    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    __shared__ float part[32];
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        m = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.0f;
-        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-        if (threadIdx.x == 0) part[0] = m;
+#pragma unroll 4
+    for (long long g = first; g < groups; g += kPlaneCtas * 256) {
+        const float4 a = u[2 * g], b = u[2 * g + 1];
+        m = fmaxf(m, fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w))),
+                           fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fmaxf(fabsf(b.z), fabsf(b.w)))));
     }
-    __syncthreads();
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    __shared__ float part[8];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+    cluster.sync();
+    m = *cluster.map_shared_rank(&part[threadIdx.x & 7], (threadIdx.x >> 3) & (kPlaneCtas - 1));
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    __shared__ float half_max[2];   // a warp holds the shares of four CTAs: warps 0 and 1 cover all eight
+    if (threadIdx.x < 64 && (threadIdx.x & 31) == 0) half_max[threadIdx.x >> 5] = m;
+    cluster.sync();   // also: no CTA leaves while another still reads its shares
     // A plane that holds only zeros and subnormals (the leading edge of a
     // wave, far planes early in a run) gets the smallest normal scale, so
     // 1/scale stays finite.
-    const float s = fmaxf(part[0], FLT_MIN);
-    if (threadIdx.x == 0) scale[blockIdx.x] = s;
+    const float s = fmaxf(fmaxf(half_max[0], half_max[1]), FLT_MIN);
+    if (first == 0) p.scale[vol][k] = s;
     const float inv = 1.0f / s;
-    for (long long q = threadIdx.x; q < plane; q += blockDim.x) out[base + q] = to_store<T>(u[base + q] * inv);
+    uint4 *out = reinterpret_cast<uint4 *>(p.q[vol] + (long long)k * plane);
+#pragma unroll 2
+    for (long long g = first; g < groups; g += kPlaneCtas * 256) {
+        const float4 a = u[2 * g], b = u[2 * g + 1];
+        out[g] = make_uint4(pack2(to_store<T>(a.x * inv), to_store<T>(a.y * inv)),
+                            pack2(to_store<T>(a.z * inv), to_store<T>(a.w * inv)),
+                            pack2(to_store<T>(b.x * inv), to_store<T>(b.y * inv)),
+                            pack2(to_store<T>(b.z * inv), to_store<T>(b.w * inv)));
+    }
 }
 
 template <class T>
-__global__ void decompress_kernel(const T *__restrict__ in, const float *__restrict__ scale, long long plane,
-                                  float *__restrict__ u) {
-    const long long base = (long long)blockIdx.x * plane;
-    const float s = scale[blockIdx.x];
-    for (long long q = threadIdx.x; q < plane; q += blockDim.x) u[base + q] = from_store(in[base + q]) * s;
+__global__ void __launch_bounds__(256) decompress_kernel(const CkptPair<T> p, long long plane, int ctas) {
+    const int k = blockIdx.x / ctas, vol = blockIdx.y;   // ctas CTAs per plane
+    const uint4 *in = reinterpret_cast<const uint4 *>(p.q[vol] + (long long)k * plane);
+    float4 *u = reinterpret_cast<float4 *>(p.u[vol] + (long long)k * plane);
+    const float s = p.scale[vol][k];
+    const long long groups = plane >> 3;
+#pragma unroll 2
+    for (long long g = (long long)(blockIdx.x % ctas) * 256 + threadIdx.x; g < groups; g += (long long)ctas * 256) {
+        const uint4 v = in[g];
+        float4 a, b;
+        a.x = from_store(stored_half<T>(v.x)) * s; a.y = from_store(stored_half<T>(v.x >> 16)) * s;
+        a.z = from_store(stored_half<T>(v.y)) * s; a.w = from_store(stored_half<T>(v.y >> 16)) * s;
+        b.x = from_store(stored_half<T>(v.z)) * s; b.y = from_store(stored_half<T>(v.z >> 16)) * s;
+        b.z = from_store(stored_half<T>(v.w)) * s; b.w = from_store(stored_half<T>(v.w >> 16)) * s;
+        u[2 * g] = a;
+        u[2 * g + 1] = b;
+    }
 }
 
 // Block floating point (MMOD_CKPT_BFP16): per block of 32 consecutive x
 // values of a padded row (rows are padded to 32, so blocks never straddle
 // rows), scale s = max |u| over the block and q = round(u * 32767 / s) as
 // int16; u is restored as q * (s / 32767), within s / 65534 of the stored
-// value.  One warp per block, grid-stride over the volume's blocks.
+// value.  Four threads per block, eight values each (16-byte accesses).
 constexpr int kBfpBlock = 32;
 constexpr float kBfpMax = 32767.0f;
 
-__global__ void compress_bfp_kernel(const float *__restrict__ u, long long nblocks, short *__restrict__ out,
-                                    float *__restrict__ scale) {
-    const int lane = threadIdx.x & 31;
-    const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long b = warp0; b < nblocks; b += nwarps) {
-        const float v = u[b * kBfpBlock + lane];
-        float m = fabsf(v);
-        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-        int q = 0;
-        if (m > 0.0f) q = max(-32767, min(32767, __float2int_rn(v * (kBfpMax / m))));
-        out[b * kBfpBlock + lane] = (short)q;
-        if (lane == 0) scale[b] = m;
+__device__ __forceinline__ short bfp_value(float v, float m) {
+    return m > 0.0f ? (short)max(-32767, min(32767, __float2int_rn(v * (kBfpMax / m)))) : (short)0;
+}
+
+__global__ void __launch_bounds__(256) compress_bfp_kernel(const CkptPair<short> p, long long nblocks) {
+    const float4 *u = reinterpret_cast<const float4 *>(p.u[blockIdx.y]);
+    uint4 *out = reinterpret_cast<uint4 *>(p.q[blockIdx.y]);
+    const long long groups = 4 * nblocks, stride = (long long)gridDim.x * 256;
+    // a warp's lanes leave the loop together: its base is a multiple of 32
+    for (long long base = (long long)blockIdx.x * 256 + (threadIdx.x & ~31); base < groups; base += stride) {
+        const long long g = base + (threadIdx.x & 31);
+        const bool in = g < groups;
+        const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f), a = in ? u[2 * g] : z, b = in ? u[2 * g + 1] : z;
+        float m = fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w))),
+                        fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fmaxf(fabsf(b.z), fabsf(b.w))));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        if (!in) continue;
+        out[g] = make_uint4(pack2(bfp_value(a.x, m), bfp_value(a.y, m)), pack2(bfp_value(a.z, m), bfp_value(a.w, m)),
+                            pack2(bfp_value(b.x, m), bfp_value(b.y, m)), pack2(bfp_value(b.z, m), bfp_value(b.w, m)));
+        if ((g & 3) == 0) p.scale[blockIdx.y][g >> 2] = m;
     }
 }
 
-__global__ void decompress_bfp_kernel(const short *__restrict__ in, const float *__restrict__ scale, long long nblocks,
-                                      float *__restrict__ u) {
-    const int lane = threadIdx.x & 31;
-    const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long b = warp0; b < nblocks; b += nwarps)
-        u[b * kBfpBlock + lane] = (float)in[b * kBfpBlock + lane] * (scale[b] / kBfpMax);
+__global__ void __launch_bounds__(256) decompress_bfp_kernel(const CkptPair<short> p, long long nblocks) {
+    const uint4 *in = reinterpret_cast<const uint4 *>(p.q[blockIdx.y]);
+    float4 *u = reinterpret_cast<float4 *>(p.u[blockIdx.y]);
+    const long long groups = 4 * nblocks, stride = (long long)gridDim.x * 256;
+    for (long long g = (long long)blockIdx.x * 256 + threadIdx.x; g < groups; g += stride) {
+        const float f = p.scale[blockIdx.y][g >> 2] / kBfpMax;
+        const uint4 v = in[g];
+        float4 a, b;
+        a.x = (float)stored_half<short>(v.x) * f; a.y = (float)stored_half<short>(v.x >> 16) * f;
+        a.z = (float)stored_half<short>(v.y) * f; a.w = (float)stored_half<short>(v.y >> 16) * f;
+        b.x = (float)stored_half<short>(v.z) * f; b.y = (float)stored_half<short>(v.z >> 16) * f;
+        b.z = (float)stored_half<short>(v.w) * f; b.w = (float)stored_half<short>(v.w >> 16) * f;
+        u[2 * g] = a;
+        u[2 * g + 1] = b;
+    }
 }
 
-int bfp_grid(long long nblocks) { return (int)std::min<long long>((nblocks + 7) / 8, 152LL * 16); }
+int bfp_grid(long long nblocks) { return (int)std::min<long long>((nblocks + 63) / 64, 152LL * 8); }
 
 size_t ckpt_elem_bytes(int dtype) { return dtype == MMOD_CKPT_FP32 ? 4 : 2; }
 
@@ -135,39 +223,59 @@ size_t ckpt_scales(const mmod_handle *h, int dtype) {
     return dtype == MMOD_CKPT_FP32 ? 0 : (size_t)h->cfg.nz;
 }
 
-// Save the volume u as checkpoint volume slot (FP32: copy; 16-bit: compress).
-cudaError_t save_volume(mmod_handle *h, const float *u, int slot, cudaStream_t s) {
+template <class T>
+CkptPair<T> ckpt_pair(mmod_handle *h, int slot, float *u_prev, float *u_cur) {
     auto &gw = h->gw;
-    const size_t eb = ckpt_elem_bytes(gw.dtype);
-    char *dst = static_cast<char *>(gw.ckpt) + (size_t)slot * h->vol * eb;
-    if (gw.dtype == MMOD_CKPT_FP32)
-        return cudaMemcpyAsync(dst, u, sizeof(float) * (size_t)h->vol, cudaMemcpyDeviceToDevice, s);
-    float *sc = gw.ckpt_scale + (size_t)slot * ckpt_scales(h, gw.dtype);
-    if (gw.dtype == MMOD_CKPT_BFP16) {
+    CkptPair<T> p;
+    p.u[0] = u_prev;
+    p.u[1] = u_cur;
+    for (int i = 0; i < 2; ++i) {
+        p.q[i] = static_cast<T *>(gw.ckpt) + (size_t)(2 * slot + i) * h->vol;
+        p.scale[i] = gw.ckpt_scale ? gw.ckpt_scale + (size_t)(2 * slot + i) * ckpt_scales(h, gw.dtype) : nullptr;
+    }
+    return p;
+}
+
+// Save the state (u^{a-1}, u^a) into checkpoint slot (FP32: copies; 16-bit: compress).
+cudaError_t save_state(mmod_handle *h, int slot, float *u_prev, float *u_cur, cudaStream_t s) {
+    const int dtype = h->gw.dtype;
+    const size_t vb = sizeof(float) * (size_t)h->vol;
+    const dim3 grid(kPlaneCtas * h->cfg.nz, 2);
+    if (dtype == MMOD_CKPT_FP32) {
+        const auto p = ckpt_pair<float>(h, slot, u_prev, u_cur);
+        for (int i = 0; i < 2; ++i)
+            if (cudaError_t e = cudaMemcpyAsync(p.q[i], p.u[i], vb, cudaMemcpyDeviceToDevice, s)) return e;
+        return cudaSuccess;
+    }
+    if (dtype == MMOD_CKPT_BFP16) {
         const long long nb = h->vol / kBfpBlock;
-        compress_bfp_kernel<<<bfp_grid(nb), 256, 0, s>>>(u, nb, reinterpret_cast<short *>(dst), sc);
-    } else if (gw.dtype == MMOD_CKPT_BF16)
-        compress_kernel<__nv_bfloat16><<<h->cfg.nz, 256, 0, s>>>(u, h->plane, reinterpret_cast<__nv_bfloat16 *>(dst), sc);
+        compress_bfp_kernel<<<dim3(bfp_grid(nb), 2), 256, 0, s>>>(ckpt_pair<short>(h, slot, u_prev, u_cur), nb);
+    } else if (dtype == MMOD_CKPT_BF16)
+        compress_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(ckpt_pair<__nv_bfloat16>(h, slot, u_prev, u_cur), h->plane);
     else
-        compress_kernel<__half><<<h->cfg.nz, 256, 0, s>>>(u, h->plane, reinterpret_cast<__half *>(dst), sc);
+        compress_kernel<__half><<<grid, 256, 0, s>>>(ckpt_pair<__half>(h, slot, u_prev, u_cur), h->plane);
     return cudaGetLastError();
 }
 
-cudaError_t restore_volume(mmod_handle *h, int slot, float *u, cudaStream_t s) {
-    auto &gw = h->gw;
-    const size_t eb = ckpt_elem_bytes(gw.dtype);
-    const char *src = static_cast<const char *>(gw.ckpt) + (size_t)slot * h->vol * eb;
-    if (gw.dtype == MMOD_CKPT_FP32)
-        return cudaMemcpyAsync(u, src, sizeof(float) * (size_t)h->vol, cudaMemcpyDeviceToDevice, s);
-    const float *sc = gw.ckpt_scale + (size_t)slot * ckpt_scales(h, gw.dtype);
-    if (gw.dtype == MMOD_CKPT_BFP16) {
+cudaError_t restore_state(mmod_handle *h, int slot, float *u_prev, float *u_cur, cudaStream_t s) {
+    const int dtype = h->gw.dtype;
+    const size_t vb = sizeof(float) * (size_t)h->vol;
+    const int per = (int)std::min<long long>((h->plane / 8 + 511) / 512, 8);   // CTAs per plane
+    const dim3 grid(per * h->cfg.nz, 2);
+    if (dtype == MMOD_CKPT_FP32) {
+        const auto p = ckpt_pair<float>(h, slot, u_prev, u_cur);
+        for (int i = 0; i < 2; ++i)
+            if (cudaError_t e = cudaMemcpyAsync(p.u[i], p.q[i], vb, cudaMemcpyDeviceToDevice, s)) return e;
+        return cudaSuccess;
+    }
+    if (dtype == MMOD_CKPT_BFP16) {
         const long long nb = h->vol / kBfpBlock;
-        decompress_bfp_kernel<<<bfp_grid(nb), 256, 0, s>>>(reinterpret_cast<const short *>(src), sc, nb, u);
-    } else if (gw.dtype == MMOD_CKPT_BF16)
-        decompress_kernel<__nv_bfloat16><<<h->cfg.nz, 256, 0, s>>>(reinterpret_cast<const __nv_bfloat16 *>(src), sc,
-                                                                    h->plane, u);
+        decompress_bfp_kernel<<<dim3(bfp_grid(nb), 2), 256, 0, s>>>(ckpt_pair<short>(h, slot, u_prev, u_cur), nb);
+    } else if (dtype == MMOD_CKPT_BF16)
+        decompress_kernel<__nv_bfloat16>
+            <<<grid, 256, 0, s>>>(ckpt_pair<__nv_bfloat16>(h, slot, u_prev, u_cur), h->plane, per);
     else
-        decompress_kernel<__half><<<h->cfg.nz, 256, 0, s>>>(reinterpret_cast<const __half *>(src), sc, h->plane, u);
+        decompress_kernel<__half><<<grid, 256, 0, s>>>(ckpt_pair<__half>(h, slot, u_prev, u_cur), h->plane, per);
     return cudaGetLastError();
 }
 
@@ -437,16 +545,14 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
                     for (int n = act.a; n < act.b; ++n) MMOD_CK(h, fwd_step_in_place(n));
                     break;
                 case MMOD_REV_SAVE:   // state of step b: u^{b-1} in u[b & 1], u^b in u[(b + 1) & 1]
-                    MMOD_CK(h, save_volume(h, h->u[act.b & 1], 2 * act.a, s));
-                    MMOD_CK(h, save_volume(h, h->u[(act.b + 1) & 1], 2 * act.a + 1, s));
+                    MMOD_CK(h, save_state(h, act.a, h->u[act.b & 1], h->u[(act.b + 1) & 1], s));
                     break;
                 case MMOD_REV_RESTORE:
                     if (act.a < 0) {
                         MMOD_CK(h, cudaMemsetAsync(h->u[0], 0, vb, s));
                         MMOD_CK(h, cudaMemsetAsync(h->u[1], 0, vb, s));
                     } else {
-                        MMOD_CK(h, restore_volume(h, 2 * act.a, h->u[act.b & 1], s));
-                        MMOD_CK(h, restore_volume(h, 2 * act.a + 1, h->u[(act.b + 1) & 1], s));
+                        MMOD_CK(h, restore_state(h, act.a, h->u[act.b & 1], h->u[(act.b + 1) & 1], s));
                     }
                     break;
                 case MMOD_REV_REVERSE: {   // g^n from the working state, then the adjoint step and its term
@@ -480,10 +586,8 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
         for (int sg = 0; sg < nseg; ++sg) {
             const int a0 = sg * seglen, b0 = std::min(nt, a0 + seglen);
             const bool last = keep_last && sg == nseg - 1;
-            if (!last) {   // at step a0: u^{a0-1} in u[a0 & 1], u^{a0} in u[(a0 + 1) & 1]
-                MMOD_CK(h, save_volume(h, h->u[a0 & 1], 2 * sg, s));
-                MMOD_CK(h, save_volume(h, h->u[(a0 + 1) & 1], 2 * sg + 1, s));
-            }
+            if (!last)   // at step a0: u^{a0-1} in u[a0 & 1], u^{a0} in u[(a0 + 1) & 1]
+                MMOD_CK(h, save_state(h, sg, h->u[a0 & 1], h->u[(a0 + 1) & 1], s));
             for (int n = a0; n < b0; ++n) {
                 fa.gout = last ? gw.seg[2 + n - a0] : nullptr;
                 const cudaError_t e = fwd_step_in_place(n);
@@ -499,8 +603,7 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
         for (int sg = nseg - 1; sg >= 0; --sg) {
             const int a0 = sg * seglen, b0 = std::min(nt, a0 + seglen);
             if (!(keep_last && sg == nseg - 1)) {
-                MMOD_CK(h, restore_volume(h, 2 * sg, gw.seg[0], s));
-                MMOD_CK(h, restore_volume(h, 2 * sg + 1, gw.seg[1], s));
+                MMOD_CK(h, restore_state(h, sg, gw.seg[0], gw.seg[1], s));
                 for (int n = a0; n < b0; ++n) {   // seg[2 + n - a0] receives g^n
                     const int j = n - a0;
                     MMOD_CK(h, fwd_step_g(n, j & 1, (j + 1) & 1, gw.seg[2 + j]));
