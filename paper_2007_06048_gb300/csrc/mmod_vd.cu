@@ -316,18 +316,24 @@ __device__ __forceinline__ float2 relax2(float2 x, float2 c, float2 d, float2 ep
 
 __device__ __forceinline__ float2 undamped2(float2 x, float2 c, float2 d) { return __ffma2_rn(c, d, x); }
 
-// CPML of two x-adjacent points (skipped where G = 0 or outside the grid).
-__device__ __forceinline__ float2 cpml_pair(float *mem, const float *B, const float *G, int i0, int i1, int n,
-                                            bool in0, bool in1, float2 d) {
-    if (in0) {
-        const float g0 = G[min(i0, n - 1)];
-        if (g0 != 0.0f) d.x = cpml_mem(mem, B[min(i0, n - 1)], g0, d.x);
-    }
-    if (in1) {
-        const float g1 = G[min(i1, n - 1)];
-        if (g1 != 0.0f) d.y = cpml_mem(mem + 1, B[min(i1, n - 1)], g1, d.y);
-    }
-    return d;
+// CPML of a thread's points.  The memory variable of one axis is kept one
+// plane ahead in registers: a plane's rows consume their values and at once
+// request the next plane's, so the loads have a whole plane to arrive (the
+// first form loaded G, then, if it was not 0, the memory variable, right where
+// each was needed: three dependent trips to memory per row and plane, 5x the
+// time of the damped kernels).  G and B of the two columns and the rows are
+// kept in registers for the whole z range; on columns outside the grid G is 0.
+struct Memory {
+    float2 gx, bx;           // axis x: the thread's two columns
+    float gy[RY], by[RY];    // axis y: its rows
+    float2 mx[RY], my[RY], mz[RY];
+};
+
+// Per component exactly cpml_mem where G != 0, nothing where G = 0.
+__device__ __forceinline__ float2 cpml_pair(float2 &m, float2 B, float2 G, float2 d) {
+    const float2 nm = __ffma2_rn(B, m, __fmul2_rn(G, d)), dm = __fadd2_rn(d, nm);
+    m = make_float2(G.x != 0.0f ? nm.x : m.x, G.y != 0.0f ? nm.y : m.y);
+    return make_float2(G.x != 0.0f ? dm.x : d.x, G.y != 0.0f ? dm.y : d.y);
 }
 
 __device__ __forceinline__ void store_pair(float *dst, float2 v, bool in0, bool in1) {
@@ -335,6 +341,51 @@ __device__ __forceinline__ void store_pair(float *dst, float2 v, bool in0, bool 
         *reinterpret_cast<float2 *>(dst) = v;
     else if (in0)
         dst[0] = v.x;
+}
+
+// The memory variables of row r (grid row y) of plane k, gz = G of the z axis on
+// that plane; 0 where the axis has none.
+__device__ __forceinline__ void memory_load(Memory &m, int r, float *const (&vol)[3], long long o, float gz, bool in0) {
+    m.mx[r] = m.my[r] = m.mz[r] = make_float2(0.0f, 0.0f);
+    if (in0 && (m.gx.x != 0.0f || m.gx.y != 0.0f)) m.mx[r] = *reinterpret_cast<const float2 *>(vol[0] + o);
+    if (in0 && m.gy[r] != 0.0f) m.my[r] = *reinterpret_cast<const float2 *>(vol[1] + o);
+    if (in0 && gz != 0.0f) m.mz[r] = *reinterpret_cast<const float2 *>(vol[2] + o);
+}
+
+// G, B of the thread's columns (x, x + 1) and rows (y ..), and the memory
+// variables of its points on plane z0.
+__device__ __forceinline__ void memory_init(Memory &m, const VdArgs &a, const float *const (&G)[3],
+                                            const float *const (&B)[3], float *const (&vol)[3], int x, int y, int z0) {
+    m.gx = make_float2(x < a.nx ? G[0][x] : 0.0f, x + 1 < a.nx ? G[0][x + 1] : 0.0f);
+    m.bx = make_float2(x < a.nx ? B[0][x] : 0.0f, x + 1 < a.nx ? B[0][x + 1] : 0.0f);
+#pragma unroll
+    for (int r = 0; r < RY; ++r) {
+        m.gy[r] = y + r < a.ny ? G[1][y + r] : 0.0f;
+        m.by[r] = y + r < a.ny ? B[1][y + r] : 0.0f;
+        memory_load(m, r, vol, (long long)z0 * a.plane + (long long)(y + r) * a.nxp + x, G[2][z0],
+                    x < a.nx && y + r < a.ny);
+    }
+}
+
+// Updates row r's memory variables with the differences dx, dy, dz of its
+// points, stores them and adds them to the differences; then requests the
+// next plane's (gz1 = G of the z axis there; o + plane).
+__device__ __forceinline__ void memory_update(Memory &m, int r, float *const (&vol)[3], long long o, long long plane,
+                                              float gz, float bz, float gz1, bool in0, bool in1, float2 &dx,
+                                              float2 &dy, float2 &dz) {
+    if (m.gx.x != 0.0f || m.gx.y != 0.0f) {
+        dx = cpml_pair(m.mx[r], m.bx, m.gx, dx);
+        store_pair(vol[0] + o, m.mx[r], in0, in1);
+    }
+    if (m.gy[r] != 0.0f) {
+        dy = cpml_pair(m.my[r], bc2(m.by[r]), bc2(m.gy[r]), dy);
+        store_pair(vol[1] + o, m.my[r], in0, in1);
+    }
+    if (gz != 0.0f) {
+        dz = cpml_pair(m.mz[r], bc2(bz), bc2(gz), dz);
+        store_pair(vol[2] + o, m.mz[r], in0, in1);
+    }
+    memory_load(m, r, vol, o + plane, gz1, in0);
 }
 
 // ---------------------------------------------------------------------------
@@ -368,8 +419,14 @@ __device__ __forceinline__ void v_read_q(const VCtx &c, int seq, float2 (&dst)[R
 }
 
 template <int J, bool C>
-__device__ __forceinline__ bool v_plane(const VdArgs &a, const VCtx &c, int t, float2 (&q)[kVQ][RY]) {
+__device__ __forceinline__ bool v_plane(const VdArgs &a, const VCtx &c, int t, float2 (&q)[kVQ][RY], Memory &m) {
     const int k = c.z0 + t;
+    float gz = 0.0f, bz_ = 0.0f, gz1 = 0.0f;   // CPML of the z axis on this plane and the next of the range
+    if (C) {
+        gz = a.Gh[2][k];
+        bz_ = a.Bh[2][k];
+        gz1 = t + 1 < c.T ? a.Gh[2][k + 1] : 0.0f;
+    }
     if (!(mbar_wait(&c.bar_p[(t + 7) % VNSP], ((t + 7) / VNSP) & 1, c.abort_flag, a.err) &&
           mbar_wait(&c.bar_o[t % VNSO], (t / VNSO) & 1, c.abort_flag, a.err) &&
           mbar_wait(&c.bar_b[t % VNSB], (t / VNSB) & 1, c.abort_flag, a.err) &&
@@ -431,9 +488,8 @@ __device__ __forceinline__ bool v_plane(const VdArgs &a, const VCtx &c, int t, f
             ny_ = relax2(vy, bhy, dy, ey);
             nz_ = relax2(vz, bhz, dz, ez);
         } else if (C) {
-            const float2 ddx = cpml_pair(a.psi[0] + o, a.Bh[0], a.Gh[0], c.x, c.x + 1, a.nx, in0, in1, dx);
-            const float2 ddy = cpml_pair(a.psi[1] + o, a.Bh[1], a.Gh[1], y, y, a.ny, in0, in1, dy);
-            const float2 ddz = cpml_pair(a.psi[2] + o, a.Bh[2], a.Gh[2], k, k, a.nz, in0, in1, dz);
+            float2 ddx = dx, ddy = dy, ddz = dz;
+            memory_update(m, r, a.psi, o, t + 1 < c.T ? a.plane : 0, gz, bz_, gz1, in0, in1, ddx, ddy, ddz);
             nx_ = undamped2(vx, bhx, ddx);
             ny_ = undamped2(vy, bhy, ddy);
             nz_ = undamped2(vz, bhz, ddz);
@@ -531,6 +587,8 @@ __global__ void __launch_bounds__(NT, 2)
         c.lay_xy[r] = lay_x || y < a.nbl || y >= a.ny - 1 - a.nbl;
     }
 
+    Memory m;
+    if (C) memory_init(m, a, a.Gh, a.Bh, a.psi, c.x, y0 + RY * c.warp, z0);
     float2 q[kVQ][RY];
     bool ok = true;
     for (int s = 0; s < 2 * kRadius - 1 && ok; ++s) {
@@ -558,7 +616,7 @@ __global__ void __launch_bounds__(NT, 2)
     // end of step t: the centre tile (seq t+3), the own tile and b plane k are free
 #define VD_VSTEP(J)                                                                   \
     if (t + (J) < T) {                                                                \
-        v_plane<(J), C>(a, c, t + (J), q);                                               \
+        v_plane<(J), C>(a, c, t + (J), q, m);                                             \
         __syncthreads();                                                              \
         if (*c.abort_flag) break;                                                     \
         if (tid == 0) {                                                               \
@@ -599,9 +657,12 @@ __global__ void __launch_bounds__(NT, 2)
 // group (kPU = 8: slots modulo 8, no shifts).  The pressure kernel's code is
 // small enough at 8 (240^3: 101.8 against 101.4 Gpoint-updates/s at 4).
 // ---------------------------------------------------------------------------
-constexpr int kPU = 8;
-constexpr int kPQ = kPU == 8 ? 8 : 2 * kRadius - 1 + kPU;
-__host__ __device__ constexpr int pq(int J, int i) { return kPU == 8 ? (J + i) % 8 : J + i; }
+template <bool C>
+constexpr int kPU = C ? 4 : 8;   // the CPML kernel's planes hold more code
+template <bool C>
+constexpr int kPQ = kPU<C> == 8 ? 8 : 2 * kRadius - 1 + kPU<C>;
+template <bool C>
+__host__ __device__ constexpr int pq(int J, int i) { return kPU<C> == 8 ? (J + i) % 8 : J + i; }
 struct PCtx {
     float *ring_c, *ring_z;
     uint64_t *bar_c, *bar_z;
@@ -620,12 +681,18 @@ __device__ __forceinline__ void p_read_q(const PCtx &c, int seq, float2 (&dst)[R
 }
 
 template <int J, bool C>
-__device__ __forceinline__ bool p_plane(const VdArgs &a, const PCtx &c, int t, float2 (&q)[kPQ][RY]) {
+__device__ __forceinline__ bool p_plane(const VdArgs &a, const PCtx &c, int t, float2 (&q)[kPQ<C>][RY], Memory &m) {
     const int k = c.z0 + t;
+    float gz = 0.0f, bz = 0.0f, gz1 = 0.0f;   // CPML of the z axis on this plane and the next of the range
+    if (C) {
+        gz = a.Gg[2][k];
+        bz = a.Bg[2][k];
+        gz1 = t + 1 < c.T ? a.Gg[2][k + 1] : 0.0f;
+    }
     if (!(mbar_wait(&c.bar_z[(t + 7) % PNSZ], ((t + 7) / PNSZ) & 1, c.abort_flag, a.err) &&
           mbar_wait(&c.bar_c[t % PNSC], (t / PNSC) & 1, c.abort_flag, a.err)))
         return false;
-    p_read_q(c, t + 7, q[pq(J, 7)]);
+    p_read_q(c, t + 7, q[pq<C>(J, 7)]);
     const float *base = c.ring_c + (t % PNSC) * P_SLOT_C;
     const float *tvx = base, *tvy = base + P_VX, *tp = base + P_VX + P_VY, *tk = tp + OWN;
     const bool zl = !C && (k < a.nbl || k > a.nz - 1 - a.nbl);
@@ -649,14 +716,12 @@ __device__ __forceinline__ bool p_plane(const VdArgs &a, const PCtx &c, int t, f
         float2 dy = stag_diff2(a.w[1], yc[r + 4], yc[r + 3], yc[r + 5], yc[r + 2], yc[r + 6], yc[r + 1], yc[r + 7],
                                yc[r + 0]);
         // D-_z: planes k+m-1 and k-m -> queue entries 3+m and 4-m
-        float2 dz = stag_diff2(a.w[2], q[pq(J, 4)][r], q[pq(J, 3)][r], q[pq(J, 5)][r], q[pq(J, 2)][r],
-                               q[pq(J, 6)][r], q[pq(J, 1)][r], q[pq(J, 7)][r], q[pq(J, 0)][r]);
+        float2 dz = stag_diff2(a.w[2], q[pq<C>(J, 4)][r], q[pq<C>(J, 3)][r], q[pq<C>(J, 5)][r], q[pq<C>(J, 2)][r],
+                               q[pq<C>(J, 6)][r], q[pq<C>(J, 1)][r], q[pq<C>(J, 7)][r], q[pq<C>(J, 0)][r]);
         const bool in0 = c.in0 && y < a.ny, in1 = c.in1 && y < a.ny;
         const long long o = (long long)k * a.plane + (long long)y * a.nxp + c.x;
         if (C) {
-            dx = cpml_pair(a.phi[0] + o, a.Bg[0], a.Gg[0], c.x, c.x + 1, a.nx, in0, in1, dx);
-            dy = cpml_pair(a.phi[1] + o, a.Bg[1], a.Gg[1], y, y, a.ny, in0, in1, dy);
-            dz = cpml_pair(a.phi[2] + o, a.Bg[2], a.Gg[2], k, k, a.nz, in0, in1, dz);
+            memory_update(m, r, a.phi, o, t + 1 < c.T ? a.plane : 0, gz, bz, gz1, in0, in1, dx, dy, dz);
         }
         const float2 div = __fadd2_rn(__fadd2_rn(dx, dy), dz);
         const float2 po = *reinterpret_cast<const float2 *>(tp + yl * TX + c.xl);
@@ -751,7 +816,9 @@ __global__ void __launch_bounds__(NT, 2)
         c.lay_xy[r] = lay_x || y < a.nbl || y > a.ny - 1 - a.nbl;
     }
 
-    float2 q[kPQ][RY];
+    Memory m;
+    if (C) memory_init(m, a, a.Gg, a.Bg, a.phi, c.x, y0 + RY * c.warp, z0);
+    float2 q[kPQ<C>][RY];
     bool ok = true;
     for (int s = 0; s < 2 * kRadius - 1 && ok; ++s) {
         ok = mbar_wait(&c.bar_z[s % PNSZ], (s / PNSZ) & 1, c.abort_flag, a.err);
@@ -769,7 +836,7 @@ __global__ void __launch_bounds__(NT, 2)
     // end of step t: the vz tile read into the queue (seq t+7) and the centre slot are free
 #define VD_PSTEP(J)                                                                   \
     if (t + (J) < T) {                                                                \
-        p_plane<(J), C>(a, c, t + (J), q);                                               \
+        p_plane<(J), C>(a, c, t + (J), q, m);                                             \
         __syncthreads();                                                              \
         if (*c.abort_flag) break;                                                     \
         if (tid == 0) {                                                               \
@@ -779,15 +846,15 @@ __global__ void __launch_bounds__(NT, 2)
     }
     if (!*c.abort_flag) {
 #pragma unroll 1
-        for (int t = 0; t < T; t += kPU) {
+        for (int t = 0; t < T; t += kPU<C>) {
             VD_PSTEP(0) VD_PSTEP(1) VD_PSTEP(2) VD_PSTEP(3)
-            if constexpr (kPU == 8) {
+            if constexpr (kPU<C> == 8) {
                 VD_PSTEP(4) VD_PSTEP(5) VD_PSTEP(6) VD_PSTEP(7)
             } else {
 #pragma unroll
                 for (int i = 0; i < 2 * kRadius - 1; ++i) {
 #pragma unroll
-                    for (int r = 0; r < RY; ++r) q[i][r] = q[i + kPU][r];
+                    for (int r = 0; r < RY; ++r) q[i][r] = q[i + kPU<C>][r];
                 }
             }
         }
