@@ -287,17 +287,16 @@ mmod_status ensure_grad_work(mmod_handle *h, int nslot, int nwork, int dtype) {
     free_grad_work(h);
     const size_t vb = sizeof(float) * (size_t)h->vol;
     gw.seg.assign(nwork, nullptr);
-    gw.seg_cur.resize(nwork);
-    gw.seg_prev.resize(nwork);
+    gw.seg_map.resize(nwork);
     for (int i = 0; i < nwork; ++i) {
         MMOD_CK(h, cudaMalloc(&gw.seg[i], vb));
         MMOD_CK(h, cudaMemset(gw.seg[i], 0, vb));
-        if (h->tma_ok && !encode_maps(h->cfg, h->nxp, gw.seg[i], &gw.seg_cur[i], &gw.seg_prev[i]))
+        if (h->tma_ok && !encode_maps(h->cfg, h->nxp, gw.seg[i], &gw.seg_map[i]))
             return fail(h, MMOD_ERR_CUDA, "tensor map encoding failed for a work volume");
     }
     for (int b = 0; b < 2; ++b) {
         MMOD_CK(h, cudaMalloc(&gw.psi[b], vb));
-        if (h->tma_ok && !encode_maps(h->cfg, h->nxp, gw.psi[b], &gw.psi_cur[b], &gw.psi_prev[b]))
+        if (h->tma_ok && !encode_maps(h->cfg, h->nxp, gw.psi[b], &gw.psi_map[b]))
             return fail(h, MMOD_ERR_CUDA, "tensor map encoding failed for an adjoint buffer");
     }
     MMOD_CK(h, cudaMalloc(&gw.gradc, vb));
@@ -356,8 +355,7 @@ void free_grad_work(mmod_handle *h) {
     for (float *p : gw.seg)
         if (p) cudaFree(p);
     gw.seg.clear();
-    gw.seg_cur.clear();
-    gw.seg_prev.clear();
+    gw.seg_map.clear();
     for (float *&p : gw.psi) {
         if (p) cudaFree(p);
         p = nullptr;
@@ -465,7 +463,7 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
         fa.ucur = h->u[(n + 1) & 1];
         fa.uprev = h->u[n & 1];
         fa.uout = h->u[n & 1];
-        return enqueue_step(h, fa, &h->cur_map[(n + 1) & 1], &h->prev_map[n & 1], tma, nullptr, s, &launches);
+        return enqueue_step(h, fa, h->u_map[(n + 1) & 1], h->u_map[n & 1], tma, nullptr, s, &launches);
     };
     // forward step n of a replay in the work volumes w0, w1 (u^{n-1} in w0,
     // u^n in w1, u^{n+1} over u^{n-1}), also writing g^n into gout
@@ -475,8 +473,7 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
         fa.uprev = gw.seg[w0];
         fa.uout = gw.seg[w0];
         fa.gout = gout;
-        const cudaError_t e = enqueue_step(h, fa, tma ? &gw.seg_cur[w1] : nullptr, tma ? &gw.seg_prev[w0] : nullptr,
-                                           tma, nullptr, s, &launches);
+        const cudaError_t e = enqueue_step(h, fa, gw.seg_map[w1], gw.seg_map[w0], tma, nullptr, s, &launches);
         fa.gout = nullptr;
         return e;
     };
@@ -489,8 +486,7 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
         aa.ucur = gw.psi[(m + 1) & 1];
         aa.uprev = gw.psi[m & 1];
         aa.uout = gw.psi[m & 1];
-        return enqueue_step(h, aa, tma ? &gw.psi_cur[(m + 1) & 1] : nullptr, tma ? &gw.psi_prev[m & 1] : nullptr,
-                            tma, nullptr, s, &launches);
+        return enqueue_step(h, aa, gw.psi_map[(m + 1) & 1], gw.psi_map[m & 1], tma, nullptr, s, &launches);
     };
     // imaging terms of forward steps n (and n - 1 when ns = 2) from g[t] =
     // g^{n-t}, after their adjoint steps: psi^{n+1} in psi[(nt-1-n) & 1],
@@ -562,7 +558,7 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
                     fa.uprev = h->u[n & 1];
                     fa.uout = unext;
                     fa.gout = gn;
-                    const cudaError_t e = enqueue_step(h, fa, &h->cur_map[(n + 1) & 1], &h->prev_map[n & 1], tma,
+                    const cudaError_t e = enqueue_step(h, fa, h->u_map[(n + 1) & 1], h->u_map[n & 1], tma,
                                                        nullptr, s, &launches);
                     fa.gout = nullptr;
                     MMOD_CK(h, e);

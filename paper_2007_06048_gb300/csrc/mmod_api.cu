@@ -391,11 +391,11 @@ StepArgs base_args(mmod_handle *h, const Geometry &geo, const float *wavelet) {
 // Enqueue one step of a run on stream s.  Plain path: step kernel, then the
 // injection kernel, then (if plain_gather_dst) the receivers of u^{n+1}.
 // TMA path: one kernel (injection inside; receivers of u^n go to a.traces).
-cudaError_t enqueue_step(mmod_handle *h, const StepArgs &a, const CUtensorMap *cur, const CUtensorMap *prev,
-                         bool tma, float *plain_gather_dst, cudaStream_t s, long long *count) {
+cudaError_t enqueue_step(mmod_handle *h, const StepArgs &a, const VolMaps &cur, const VolMaps &prev, bool tma,
+                         float *plain_gather_dst, cudaStream_t s, long long *count) {
     cudaError_t e;
     if (tma) {
-        e = launch_step_tma(a, cur, prev, &h->c_map, a.gout ? g_plan(h) : active_plan(h), s);
+        e = launch_step_tma(a, cur, prev, h->c_map, a.gout ? g_plan(h) : active_plan(h), s);
         ++*count;
         return e;
     }
@@ -449,7 +449,7 @@ static mmod_status enqueue_loop(mmod_handle *h, const Geometry &geo, const float
             a.uprev = h->u[n & 1];
             a.uout = h->u[n & 1];
             a.traces = (n >= 1 && tr && ng > 0) ? tr + (long long)(n - 1) * ng : nullptr;
-            MMOD_CK(h, enqueue_step(h, a, &h->cur_map[(n + 1) & 1], &h->prev_map[n & 1], tma, nullptr, s, count));
+            MMOD_CK(h, enqueue_step(h, a, h->u_map[(n + 1) & 1], h->u_map[n & 1], tma, nullptr, s, count));
             int passes = 0;
             MMOD_CK(h, launch_cpml_layers(cp, &h->cpml_tiles, (n + 1) & 1, a.ucur, a.uout, s, &passes));
             *count += passes;
@@ -476,7 +476,7 @@ static mmod_status enqueue_loop(mmod_handle *h, const Geometry &geo, const float
         a.uprev = h->u[n & 1];
         a.uout = h->u[n & 1];
         a.traces = (n >= 1 && tr && ng > 0) ? tr + (long long)(n - 1) * ng : nullptr;
-        MMOD_CK(h, enqueue_step(h, a, &h->cur_map[(n + 1) & 1], &h->prev_map[n & 1], tma,
+        MMOD_CK(h, enqueue_step(h, a, h->u_map[(n + 1) & 1], h->u_map[n & 1], tma,
                                 (tr && ng > 0) ? tr + (long long)n * ng : nullptr, s, count));
         MMOD_CK(h, mark(tma ? n : n + 1));   // the TMA kernel of step n gathers row n - 1
     }
@@ -523,8 +523,8 @@ mmod_status run_loop_graph(mmod_handle *h, GraphSlot &g, const Geometry &geo, co
         pa.u[1] = h->u[1];
         TmaMaps maps;
         for (int b = 0; b < 2; ++b) {
-            maps.cur[b] = h->cur_map[b];
-            maps.prev[b] = h->prev_map[b];
+            maps.cur[b] = h->u_map[b].halo;
+            maps.prev[b] = h->u_map[b].own;
         }
         maps.c = h->c_map;
         MMOD_CK(h, launch_step_tma_persistent(a, maps, plan, pa, pgrid, s));
@@ -672,7 +672,7 @@ MMOD_API mmod_status mmod_create(const mmod_config *cfg, int device, mmod_handle
     *h->err_host = 0;
     CKC(cudaHostGetDevicePointer(&h->err_dev, h->err_host, 0));
     if (is_cpml(h)) make_cpml_tiles(cpml_args(h), h->u, &h->cpml_tiles);   // axes it cannot tile keep the march
-    h->tma_ok = make_tma_plan(h->cfg, h->nxp, h->u, h->c, h->cur_map, h->prev_map, &h->c_map, h->plans);
+    h->tma_ok = make_tma_plan(h->cfg, h->nxp, h->u, h->c, h->u_map, &h->c_map, h->plans);
     if (h->tma_ok) {   // counters of the persistent kernel, sized for the plan with the most units
         for (int v = 0; v < tma_variant_count(); ++v)
             h->ncounters = std::max<long long>(h->ncounters, (long long)h->plans[v].tiles_x * h->plans[v].tiles_y *

@@ -177,7 +177,7 @@ mmod_status enqueue_tune_steps(mmod_handle *h, int steps, cudaStream_t s) {
         a.ucur = h->u[(n + 1) & 1];
         a.uprev = h->u[n & 1];
         a.uout = h->u[n & 1];
-        MMOD_CK(h, enqueue_step(h, a, &h->cur_map[(n + 1) & 1], &h->prev_map[n & 1], true, nullptr, s, &count));
+        MMOD_CK(h, enqueue_step(h, a, h->u_map[(n + 1) & 1], h->u_map[n & 1], true, nullptr, s, &count));
     }
     h->state_pending = false;
     h->ran = false;
@@ -223,8 +223,8 @@ MMOD_API mmod_status mmod_batch_create(mmod_handle *const *shots, int nshots, mm
         d.rec_idx = h->fwd.g_idx;
         d.rec_boff = h->fwd.g_off;
         for (int k = 0; k < 2; ++k) {
-            d.cur[k] = h->cur_map[k];
-            d.prev[k] = h->prev_map[k];
+            d.cur[k] = h->u_map[k].halo;
+            d.prev[k] = h->u_map[k].own;
             d.u[k] = h->u[k];
         }
         d.cmap = h->c_map;

@@ -114,15 +114,16 @@ struct mmod_handle {
     long long ncounters = 0;
     int ckpt_scheme = MMOD_SCHEME_SEGMENTS;   // MMOD_OPT_CKPT_SCHEME
     bool tma_ok = false;
-    CUtensorMap cur_map[2], prev_map[2], c_map;
+    mmod::VolMaps u_map[2];             // tensor maps of u[0], u[1]
+    CUtensorMap c_map;
 
     // gradient work space (lazy, sized for the last checkpoint layout)
     struct GradWork {
         int nslot = 0, nwork = 0, dtype = -1;
         std::vector<float *> seg;           // nwork padded FP32 work volumes
-        std::vector<CUtensorMap> seg_cur, seg_prev;
+        std::vector<mmod::VolMaps> seg_map;
         float *psi[2] = {nullptr, nullptr};
-        CUtensorMap psi_cur[2], psi_prev[2];
+        mmod::VolMaps psi_map[2];
         float *gradc = nullptr;             // padded FP32 sum of psi^{n+1} g^n
         void *ckpt = nullptr;               // nslot * 2 volumes (FP32 or 16-bit)
         float *ckpt_scale = nullptr;        // 16-bit storage: per-plane (BF16, FP16) or per-32-value
@@ -168,8 +169,8 @@ const TmaPlan &active_plan(const mmod_handle *h);
 StepArgs base_args(mmod_handle *h, const Geometry &geo, const float *wavelet);
 // Enqueues one step (plain path: step, injection, optional gather of
 // u^{n+1} into plain_gather_dst; TMA path: one kernel).
-cudaError_t enqueue_step(mmod_handle *h, const StepArgs &a, const CUtensorMap *cur, const CUtensorMap *prev,
-                         bool tma, float *plain_gather_dst, cudaStream_t s, long long *count);
+cudaError_t enqueue_step(mmod_handle *h, const StepArgs &a, const VolMaps &cur, const VolMaps &prev, bool tma,
+                         float *plain_gather_dst, cudaStream_t s, long long *count);
 // The nt-step loop of a run from u[0], u[1] with geometry geo, captured into
 // the graph slot g on first use and replayed.
 mmod_status run_loop_graph(mmod_handle *h, GraphSlot &g, const Geometry &geo, const float *wav, float *tr,

@@ -203,8 +203,12 @@ cudaError_t launch_step_tma_batch_persistent(int variant, const ShotDesc *shots,
                                              cudaStream_t s);
 // CTAs of the persistent batch kernel of variant v that fit at once (0: none).
 int batch_persistent_grid(int variant, int units);
-cudaError_t launch_step_tma(const StepArgs &a, const CUtensorMap *cur_map,
-                            const CUtensorMap *prev_map, const CUtensorMap *c_map,
+struct VolMaps;
+// One launch's tensor maps: u^n as halo and as tile box, u^{n-1} and c.
+struct StepMaps {
+    CUtensorMap halo, own, prev, c;
+};
+cudaError_t launch_step_tma(const StepArgs &a, const VolMaps &cur, const VolMaps &prev, const CUtensorMap &c_map,
                             const TmaPlan &plan, cudaStream_t s);
 
 // Persistent run: one cooperative launch advances steps n0 .. n1-1.  CTAs

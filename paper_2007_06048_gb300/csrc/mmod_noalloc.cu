@@ -306,9 +306,10 @@ extern "C" __attribute__((visibility("default"))) mmod_status mmod_forward_noall
     // ---- time loop: u^{-1} = u^0 = 0, one step kernel per step
     CKS(cudaMemsetAsync(u[0], 0, sizeof(float) * vol, s));
     CKS(cudaMemsetAsync(u[1], 0, sizeof(float) * vol, s));
-    CUtensorMap cur_map[2], prev_map[2], c_map;
+    VolMaps u_map[2];
+    CUtensorMap c_map;
     TmaPlan plans[kMaxTmaVariants];
-    const bool tma = make_tma_plan(c, nxp, u, cvol, cur_map, prev_map, &c_map, plans);
+    const bool tma = make_tma_plan(c, nxp, u, cvol, u_map, &c_map, plans);
     StepArgs a{};
     a.nx = c.nx; a.ny = c.ny; a.nz = c.nz; a.nxp = nxp; a.plane = plane; a.nbl = c.nbl; a.nt = c.nt;
     for (int m = 0; m < kRadius; ++m) {
@@ -338,7 +339,7 @@ extern "C" __attribute__((visibility("default"))) mmod_status mmod_forward_noall
         a.uout = u[n & 1];
         if (tma) {
             a.traces = (n >= 1 && want_tr) ? traces + (long long)(n - 1) * c.nrec : nullptr;
-            CKS(launch_step_tma(a, &cur_map[(n + 1) & 1], &prev_map[n & 1], &c_map, plans[kTmaDefaultVariant], s));
+            CKS(launch_step_tma(a, u_map[(n + 1) & 1], u_map[n & 1], c_map, plans[kTmaDefaultVariant], s));
         } else {
             a.traces = nullptr;
             CKS(launch_step_simple(a, s));

@@ -44,6 +44,7 @@ constexpr int HX = TX + 2 * kRadius;   // 72: halo tile width
 
 template <int TY_, int RY_, int U_, int NSU_ = 8, int NSC_ = 4, int MINB_ = 1>
 struct Shape {
+    static constexpr bool kStaged = false;
     static constexpr int MINB = MINB_;              // resident CTAs per SM the registers are capped for
     // the batch and persistent kernels always keep two CTAs per SM resident
     static constexpr int MINB2 = MINB_ > 2 ? MINB_ : 2;
@@ -58,7 +59,8 @@ struct Shape {
     static constexpr int HY = TY + 2 * kRadius;
     static constexpr int CUR = HX * HY;             // floats per u^n slot
     static constexpr int PC = TX * TY;              // floats per u^{n-1} or c slot
-    static constexpr int SMEM = (NSU * CUR + NSC * 2 * PC) * 4 + (NSU + NSC) * 8 + 16;
+    static constexpr int ABORT_OFF = (NSU * CUR + NSC * 2 * PC) * 4 + (NSU + NSC) * 8;   // then the claim words
+    static constexpr int SMEM = ABORT_OFF + 16;
     static_assert(TY % RY == 0, "rows per thread must divide the tile height");
     static_assert(NSU >= 6 && NSU <= 8 && NSC >= 2, "ring depth outside the fill / release schedule");
 };
@@ -470,14 +472,30 @@ __device__ __forceinline__ void step_tma_body(const StepArgs &a, const StepVar &
     }
 }
 
+}  // namespace
+}  // namespace mmod
+
+#include "step_staged.cuh"
+
+namespace mmod {
+namespace {
+
+template <class S, class Dep, bool G = false>
+__device__ __forceinline__ void step_body(const StepArgs &a, const StepVar &v, const CUtensorMap *halo_map,
+                                          const CUtensorMap *own_map, const CUtensorMap *prev_map,
+                                          const CUtensorMap *c_map, const Geom &g, int bid, int nbid, const Dep &dep) {
+    if constexpr (S::kStaged)
+        step_staged_body<S, Dep, G>(a, v, halo_map, own_map, prev_map, c_map, g, bid, nbid, dep);
+    else
+        step_tma_body<S, Dep, G>(a, v, halo_map, prev_map, c_map, g, bid, nbid, dep);
+}
+
 // G: also write g^n = L u^n + s^n into a.gout (the gradient's imaging factor).
 template <class S, bool G = false>
 __global__ void __launch_bounds__(S::NT, S::MINB)
-    step_tma_kernel(const StepArgs a, const __grid_constant__ CUtensorMap cur_map,
-                    const __grid_constant__ CUtensorMap prev_map, const __grid_constant__ CUtensorMap c_map,
-                    const Geom g) {
-    step_tma_body<S, PdlDep, G>(a, StepVar{a.n, a.uout, a.ucur, a.traces}, &cur_map, &prev_map, &c_map, g,
-                                blockIdx.x, gridDim.x, PdlDep{a.pdl});
+    step_tma_kernel(const StepArgs a, const __grid_constant__ StepMaps maps, const Geom g) {
+    step_body<S, PdlDep, G>(a, StepVar{a.n, a.uout, a.ucur, a.traces}, &maps.halo, &maps.own, &maps.prev, &maps.c, g,
+                            blockIdx.x, gridDim.x, PdlDep{a.pdl});
 }
 
 // Work-claiming step (StepArgs::claim set): at most one wave of CTAs covers
@@ -507,18 +525,15 @@ struct ClaimDep {
 
 template <class S, bool G = false>
 __global__ void __launch_bounds__(S::NT, S::MINB2)
-    step_tma_claim_kernel(const StepArgs a, const __grid_constant__ CUtensorMap cur_map,
-                          const __grid_constant__ CUtensorMap prev_map, const __grid_constant__ CUtensorMap c_map,
-                          const Geom g, int units) {
+    step_tma_claim_kernel(const StepArgs a, const __grid_constant__ StepMaps maps, const Geom g, int units) {
     extern __shared__ __align__(128) unsigned char smem[];
     // the body's abort flag and, next to it, the claimed unit
-    int *abort_flag = reinterpret_cast<int *>(smem + (S::NSU * S::CUR + S::NSC * 2 * S::PC) * 4 +
-                                              (S::NSU + S::NSC) * 8);
+    int *abort_flag = reinterpret_cast<int *>(smem + S::ABORT_OFF);
     int *next = abort_flag + 1;
     bool first = true;
     for (int unit = blockIdx.x; unit < units;) {
-        step_tma_body<S, ClaimDep, G>(a, StepVar{a.n, a.uout, a.ucur, a.traces}, &cur_map, &prev_map, &c_map, g,
-                                      unit, units, ClaimDep{a.pdl, first});
+        step_body<S, ClaimDep, G>(a, StepVar{a.n, a.uout, a.ucur, a.traces}, &maps.halo, &maps.own, &maps.prev,
+                                  &maps.c, g, unit, units, ClaimDep{a.pdl, first});
         first = false;
         __syncthreads();
         if (*abort_flag) break;   // the body drained its copies
@@ -572,8 +587,8 @@ __global__ void __launch_bounds__(S::NT, S::MINB2)
         sa.traces = (n >= 1 && d->traces && sa.nrec > 0) ? d->traces + (long long)(n - 1) * sa.nrec : nullptr;
     }
     __syncthreads();
-    step_tma_body<S>(sa, StepVar{sa.n, sa.uout, sa.ucur, sa.traces}, &d->cur[(n + 1) & 1], &d->prev[n & 1],
-                     &d->cmap, d->geom, __ldg(cta_local + blockIdx.x), d->nblocks, PdlDep{sa.pdl});
+    step_body<S>(sa, StepVar{sa.n, sa.uout, sa.ucur, sa.traces}, &d->cur[(n + 1) & 1], &d->prev[(n + 1) & 1],
+                 &d->prev[n & 1], &d->cmap, d->geom, __ldg(cta_local + blockIdx.x), d->nblocks, PdlDep{sa.pdl});
 }
 
 // Persistent run (PersistArgs): steps n0 .. n1-1 in one cooperative launch,
@@ -593,7 +608,7 @@ __global__ void __launch_bounds__(S::NT, S::MINB2)
     step_tma_persistent_kernel(const StepArgs a, const __grid_constant__ TmaMaps maps, const Geom g,
                                const PersistArgs pa) {
     extern __shared__ __align__(128) unsigned char smem[];
-    unsigned char *reserved = smem + (S::NSU * S::CUR + S::NSC * 2 * S::PC) * 4 + (S::NSU + S::NSC) * 8;
+    unsigned char *reserved = smem + S::ABORT_OFF;
     const int *abort_flag = reinterpret_cast<const int *>(reserved);
     unsigned long long *claimed = claimed_item(reserved);
     const unsigned long long total = (unsigned long long)(pa.n1 - pa.n0) * pa.units;
@@ -606,8 +621,8 @@ __global__ void __launch_bounds__(S::NT, S::MINB2)
         if (item >= total) break;
         const int n = pa.n0 + (int)(item / pa.units), unit = (int)(item % pa.units);
         float *uout = pa.u[n & 1];
-        step_tma_body<S>(a, StepVar{n, uout, nullptr, nullptr}, &maps.cur[(n + 1) & 1], &maps.prev[n & 1], &maps.c,
-                         g, unit, pa.units, NeighborDep{pa.counters, unit, n, g, first});
+        step_body<S>(a, StepVar{n, uout, nullptr, nullptr}, &maps.cur[(n + 1) & 1], &maps.prev[(n + 1) & 1],
+                     &maps.prev[n & 1], &maps.c, g, unit, pa.units, NeighborDep{pa.counters, unit, n, g, first});
         first = false;
         __syncthreads();
         if (*abort_flag) return;   // the body drained its copies; waiters give up on the error word
@@ -647,7 +662,7 @@ __global__ void __launch_bounds__(S::NT, S::MINB2)
     step_tma_batch_persistent_kernel(const ShotDesc *__restrict__ shots, const BatchPersistArgs pa) {
     extern __shared__ __align__(128) unsigned char smem[];
     StepArgs &sa = *reinterpret_cast<StepArgs *>(smem + batch_args_offset<S>());
-    unsigned char *reserved = smem + (S::NSU * S::CUR + S::NSC * 2 * S::PC) * 4 + (S::NSU + S::NSC) * 8;
+    unsigned char *reserved = smem + S::ABORT_OFF;
     const int *abort_flag = reinterpret_cast<const int *>(reserved);
     unsigned long long *claimed = claimed_item(reserved);
     const unsigned long long total = (unsigned long long)(pa.n1 - pa.n0) * pa.units;
@@ -669,8 +684,9 @@ __global__ void __launch_bounds__(S::NT, S::MINB2)
         __syncthreads();
         float *uout = d->u[n & 1];
         int *counters = pa.counters + __ldg(pa.counter_base + shot);
-        step_tma_body<S>(sa, StepVar{n, uout, nullptr, nullptr}, &d->cur[(n + 1) & 1], &d->prev[n & 1], &d->cmap,
-                         d->geom, local, d->nblocks, NeighborDep{counters, local, n, d->geom, first});
+        step_body<S>(sa, StepVar{n, uout, nullptr, nullptr}, &d->cur[(n + 1) & 1], &d->prev[(n + 1) & 1],
+                     &d->prev[n & 1], &d->cmap, d->geom, local, d->nblocks,
+                     NeighborDep{counters, local, n, d->geom, first});
         first = false;
         __syncthreads();
         if (*abort_flag) return;   // the body drained its copies; waiters give up on the error word
@@ -735,7 +751,7 @@ constexpr int kTY = 16;
 static_assert(kTY == kInjTileY && TX == kInjTileX, "injection buckets must match the kernel's tiles");
 using V22_1 = Shape<kTY, 2, 1>;
 using V22_2 = Shape<kTY, 2, 2>;
-using V22_4 = Shape<kTY, 2, 4>;
+using V22_4 = Staged<TX, kTY, HX>;
 using V24_1 = Shape<kTY, 4, 1>;
 using V24_2 = Shape<kTY, 4, 2>;
 using V24_2s = Shape<kTY, 4, 2, 6, 2>;
@@ -788,16 +804,14 @@ bool encode_box(CUtensorMap *map, const float *base, int nx, int ny, int nz, int
     return encode(map, base, c, nxp, bx, by);
 }
 
-bool encode_maps(const mmod_config &cfg, int nxp, const float *buf, CUtensorMap *cur, CUtensorMap *prev) {
-    return encode(cur, buf, cfg, nxp, HX, kTY + 2 * kRadius) && encode(prev, buf, cfg, nxp, TX, kTY);
+bool encode_maps(const mmod_config &cfg, int nxp, const float *buf, VolMaps *m) {
+    return encode(&m->halo, buf, cfg, nxp, HX, kTY + 2 * kRadius) && encode(&m->own, buf, cfg, nxp, TX, kTY);
 }
 
-bool make_tma_plan(const mmod_config &cfg, int nxp, float *const u[2], const float *c, CUtensorMap cur_map[2],
-                   CUtensorMap prev_map[2], CUtensorMap *c_map, TmaPlan plans[]) {
-    for (int b = 0; b < 2; ++b) {
-        if (!encode(&cur_map[b], u[b], cfg, nxp, HX, kTY + 2 * kRadius)) return false;
-        if (!encode(&prev_map[b], u[b], cfg, nxp, TX, kTY)) return false;
-    }
+bool make_tma_plan(const mmod_config &cfg, int nxp, float *const u[2], const float *c, VolMaps u_map[2],
+                   CUtensorMap *c_map, TmaPlan plans[]) {
+    for (int b = 0; b < 2; ++b)
+        if (!encode_maps(cfg, nxp, u[b], &u_map[b])) return false;
     if (!encode(c_map, c, cfg, nxp, TX, kTY)) return false;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -872,8 +886,9 @@ bool claim_geom(const TmaPlan &plan, int nz, Geom *g, int *units, int *grid) {
     return true;
 }
 
-cudaError_t launch_step_tma(const StepArgs &a, const CUtensorMap *cur_map, const CUtensorMap *prev_map,
-                            const CUtensorMap *c_map, const TmaPlan &plan, cudaStream_t s) {
+cudaError_t launch_step_tma(const StepArgs &a, const VolMaps &cur, const VolMaps &prev, const CUtensorMap &c_map,
+                            const TmaPlan &plan, cudaStream_t s) {
+    const StepMaps maps{cur.halo, cur.own, prev.own, c_map};
     Geom cg;
     int units = 0, cgrid = 0;
     const bool claim = a.claim && claim_geom(plan, a.nz, &cg, &units, &cgrid);
@@ -891,8 +906,8 @@ cudaError_t launch_step_tma(const StepArgs &a, const CUtensorMap *cur_map, const
         lc.numAttrs = a.pdl ? 1 : 0;
         const Geom g{plan.tiles_x, plan.tiles_y, plan.zchunks, plan.zlen};
         const cudaError_t e =
-            claim ? cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_4, true>, a, *cur_map, *prev_map, *c_map, cg, units)
-                  : cudaLaunchKernelEx(&lc, step_tma_kernel<V22_4, true>, a, *cur_map, *prev_map, *c_map, g);
+            claim ? cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_4, true>, a, maps, cg, units)
+                  : cudaLaunchKernelEx(&lc, step_tma_kernel<V22_4, true>, a, maps, g);
         if (e != cudaSuccess) return e;
         return cudaGetLastError();
     }
@@ -909,9 +924,9 @@ cudaError_t launch_step_tma(const StepArgs &a, const CUtensorMap *cur_map, const
         lc.numAttrs = a.pdl ? 1 : 0;
         cudaError_t e;
         switch (plan.variant) {
-            case 1: e = cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_2>, a, *cur_map, *prev_map, *c_map, cg, units); break;
-            case 2: e = cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_4>, a, *cur_map, *prev_map, *c_map, cg, units); break;
-            case 6: e = cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_4s>, a, *cur_map, *prev_map, *c_map, cg, units); break;
+            case 1: e = cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_2>, a, maps, cg, units); break;
+            case 2: e = cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_4>, a, maps, cg, units); break;
+            case 6: e = cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_4s>, a, maps, cg, units); break;
             default: return cudaErrorInvalidValue;
         }
         if (e != cudaSuccess) return e;
@@ -928,7 +943,7 @@ cudaError_t launch_step_tma(const StepArgs &a, const CUtensorMap *cur_map, const
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = a.pdl ? 1 : 0;
-#define MMOD_LAUNCH(V) cudaLaunchKernelEx(&lc, step_tma_kernel<V>, a, *cur_map, *prev_map, *c_map, g)
+#define MMOD_LAUNCH(V) cudaLaunchKernelEx(&lc, step_tma_kernel<V>, a, maps, g)
     switch (plan.variant) {
         case 0: MMOD_LAUNCH(V22_1); break;
         case 1: MMOD_LAUNCH(V22_2); break;

@@ -1,0 +1,320 @@
+// The step kernel's plane pipeline in staged form (included by
+// mmod_step_tma.cu, which documents the decomposition and the arithmetic).
+//
+// A CTA owns a TX x TY tile and marches down T planes from z0; each thread
+// owns 2 (x) x 2 (y) points.  What differs from the ring form of
+// mmod_step_tma.cu:
+//   * One mbarrier per stage: stage t % 4 carries everything plane t needs that
+//     is not on chip yet, i.e. the halo tile of u^n at z0 + t + 4, and u^{n-1}
+//     and c at z0 + t.  A plane costs one wait instead of two, and with the
+//     plane loop unrolled by 4 every shared-memory offset and the barrier are
+//     constants; the eight halo slots alternate between two halves, so a group
+//     of four planes reads its leading planes from one half and its centre
+//     planes from the other.
+//   * All the first planes are requested at once.  The planes z0-4 .. z0-1 are
+//     only ever z neighbours of the thread's own points: they come as tile
+//     boxes without x-y halo into a region of their own (TX x TY instead of
+//     PITCH x (TY + 8) floats), so the eight halo slots hold z0 .. z0+7 from the
+//     start and the leading planes of the first group do not wait for a slot
+//     (one memory latency less per launch).
+//   * A thread's own centre values come from its z queue, not from shared
+//     memory again (4 of 24 loads per plane), and the damping terms are formed
+//     only on damped planes (e = 0 elsewhere, where the multiply-add and the
+//     factor are exact identities).
+// Bound by DRAM on large grids and by the pipeline's latencies on one-wave
+// grids.  us per step, ring form -> staged: 64^3 4.47 -> 3.83, 128^3 8.68 ->
+// 7.89, 200^3 34.98 -> 32.35, 240^3 41.96 -> 41.20, 512^3 337.0 -> 325.5 (6.60
+// TB/s); 110 registers instead of 120.
+// PITCH, the halo tile's row pitch, is chosen so that a half-warp whose lanes
+// span two row pairs reads 16 different bank pairs: 2 PITCH = TX (mod 32).
+#pragma once
+
+namespace mmod {
+namespace {
+
+template <int TX_, int TY_, int PITCH_, int MINB_ = 2>
+struct Staged {
+    static constexpr bool kStaged = true;
+    static constexpr int TX = TX_, TY = TY_, PITCH = PITCH_, HY = TY_ + 2 * kRadius;
+    static constexpr int RY = 2, U = 4, NSU = 8;
+    static constexpr int QD = 2 * kRadius + U;           // z queue: 8 planes and one group
+    static constexpr int LX = TX / 2, NT = LX * (TY / RY);
+    static constexpr int MINB = MINB_, MINB2 = MINB_ > 2 ? MINB_ : 2;
+    static constexpr int CUR = PITCH * HY;               // floats of a halo slot
+    static constexpr int OWN = TX * TY;                  // floats of a tile box
+    static constexpr int OWN_S = (OWN + 31) / 32 * 32;   // its slot, 128-byte aligned
+    static constexpr int CUR_S = (CUR + 31) / 32 * 32;
+    static constexpr int RINGS = NSU * CUR_S + 4 * OWN_S + U * 2 * OWN_S;   // floats
+    static constexpr int ABORT_OFF = RINGS * 4 + (U + 1) * 8;               // abort flag, then the claim words
+    static constexpr int SMEM = ABORT_OFF + 16;
+    static constexpr unsigned STAGE_BYTES = (CUR + 2 * OWN) * 4;
+    static constexpr unsigned FIRST_BYTES = (4 * CUR + 4 * OWN) * 4;
+    static_assert(TX % 4 == 0 && TY % RY == 0 && PITCH % 4 == 0 && PITCH >= TX + 2 * kRadius, "16-byte boxes");
+    static_assert(NT <= 256 && SMEM <= 113 * 1024, "two CTAs per SM");
+};
+
+struct StagedCtx {
+    float *col;          // the thread's column in halo slot 0 (row 2 py, column 2 px)
+    float *pc;           // the thread's point in the first u^{n-1} tile
+    uint64_t *full;      // U stage barriers
+    int *abort_flag;
+    int z0;
+    bool xy_damped;
+    bool full0, full1, part0, part1;   // row 0 / 1: both columns, or only the first, inside the grid
+};
+
+// One plane: step t of the range, J = t % 4, half = (t / 4) & 1.  out / gout:
+// the thread's point of row 0 on this plane.
+template <class S, int J, bool G>
+__device__ __forceinline__ void staged_plane(const StepArgs &a, const StagedCtx &c, int k, unsigned half,
+                                             const float *ctr_half, const float *lead_half,
+                                             float2 (&q)[S::QD][S::RY], const Wts &w, float2 exr,
+                                             const float (&eyr)[S::RY], float *out, float *gout) {
+    const bool damped = c.xy_damped || k < a.nbl || k > a.nz - 1 - a.nbl;
+    const float ez = damped ? __ldg(a.ez + k) : 0.0f;
+    if (!mbar_wait(&c.full[J], half, c.abort_flag, a.err)) return;
+    // the leading plane k + 4 enters the queue
+    const float *lead = lead_half + J * S::CUR_S + kRadius * S::PITCH + kRadius;
+#pragma unroll
+    for (int r = 0; r < S::RY; ++r) q[J + 2 * kRadius][r] = *reinterpret_cast<const float2 *>(lead + r * S::PITCH);
+    // y neighbours: rows 2 py .. 2 py + 9 of the centre plane; the thread's own two rows are in the queue
+    const float *ctr = ctr_half + J * S::CUR_S;
+    float2 yc[S::RY + 2 * kRadius];
+#pragma unroll
+    for (int rr = 0; rr < S::RY + 2 * kRadius; ++rr)
+        yc[rr] = rr >= kRadius && rr < kRadius + S::RY
+                     ? q[J + kRadius][rr >= kRadius && rr < kRadius + S::RY ? rr - kRadius : 0]
+                     : *reinterpret_cast<const float2 *>(ctr + rr * S::PITCH + kRadius);
+    const float *upp = c.pc + J * 2 * S::OWN_S;
+#pragma unroll
+    for (int r = 0; r < S::RY; ++r) {
+        const float *row = ctr + (kRadius + r) * S::PITCH;
+        const float2 p = q[J + kRadius][r];
+        const float2 x0 = *reinterpret_cast<const float2 *>(row), x1 = *reinterpret_cast<const float2 *>(row + 2);
+        const float2 x3 = *reinterpret_cast<const float2 *>(row + 6), x4 = *reinterpret_cast<const float2 *>(row + 8);
+        const float2 two_p = __fadd2_rn(p, p);
+        const float2 ntp = neg2(two_p);
+        // x: offsets 1 and 3 do not form aligned pairs, so they run scalar
+        float2 lx;
+        lx.x = pair_first(w.x1, p.y, x1.y, two_p.x);
+        lx.y = pair_first(w.x1, x3.x, p.x, two_p.y);
+        lx = pair_acc2(lx, w.x2, x3, x1, ntp);
+        lx.x = pair_acc(lx.x, w.x3, x3.y, x0.y, two_p.x);
+        lx.y = pair_acc(lx.y, w.x3, x4.x, x1.x, two_p.y);
+        lx = pair_acc2(lx, w.x4, x4, x0, ntp);
+        float2 ly = pair_first2(w.y[0], yc[kRadius + r + 1], yc[kRadius + r - 1], ntp);
+        float2 lz = pair_first2(w.z[0], q[J + kRadius + 1][r], q[J + kRadius - 1][r], ntp);
+#pragma unroll
+        for (int m = 2; m <= kRadius; ++m) {
+            ly = pair_acc2(ly, w.y[m - 1], yc[kRadius + r + m], yc[kRadius + r - m], ntp);
+            lz = pair_acc2(lz, w.z[m - 1], q[J + kRadius + m][r], q[J + kRadius - m][r], ntp);
+        }
+        const float2 lap = __fadd2_rn(__fadd2_rn(lx, ly), lz);
+        const float2 pp = *reinterpret_cast<const float2 *>(upp + r * S::TX);
+        const float2 cc = *reinterpret_cast<const float2 *>(upp + S::OWN_S + r * S::TX);
+        float2 num = __fadd2_rn(two_p, neg2(pp));
+        if (damped) {   // e = (e_x + e_y) + e_z
+            const float2 e = __fadd2_rn(__fadd2_rn(exr, bcast(eyr[r])), bcast(ez));
+            num = __ffma2_rn(cc, lap, __ffma2_rn(e, pp, num));
+            num = __fmul2_rn(num, make_float2(damp_factor(e.x), damp_factor(e.y)));
+        } else {
+            num = __ffma2_rn(cc, lap, num);
+        }
+        if (a.fs && k == 0) num = make_float2(0.0f, 0.0f);   // p = 0 on a free surface
+        float *dst = out + (r ? a.nxp : 0);
+        if (r ? c.full1 : c.full0)
+            *reinterpret_cast<float2 *>(dst) = num;
+        else if (r ? c.part1 : c.part0)
+            dst[0] = num.x;
+        if constexpr (G) {   // g^n = L u^n (sources added after the z range), 0 on a free surface
+            const float2 gv = (a.fs && k == 0) ? make_float2(0.0f, 0.0f) : lap;
+            float *gd = gout + (r ? a.nxp : 0);
+            if (r ? c.full1 : c.full0)
+                *reinterpret_cast<float2 *>(gd) = gv;
+            else if (r ? c.part1 : c.part0)
+                gd[0] = gv.x;
+        }
+    }
+}
+
+// The work of one CTA: block `bid` of the `nbid` blocks of one grid.
+// halo_map: u^n, PITCH x HY box; own_map: u^n, prev_map: u^{n-1}, c_map: c, TX x TY boxes.
+template <class S, class Dep, bool G = false>
+__device__ __forceinline__ void step_staged_body(const StepArgs &a, const StepVar &v, const CUtensorMap *halo_map,
+                                                 const CUtensorMap *own_map, const CUtensorMap *prev_map,
+                                                 const CUtensorMap *c_map, const Geom &g, int bid, int nbid,
+                                                 const Dep &dep) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    float *const ring = reinterpret_cast<float *>(smem);
+    float *const first = ring + S::NSU * S::CUR_S;       // planes z0-4 .. z0-1, tile boxes
+    float *const pc = first + 4 * S::OWN_S;              // stage j: u^{n-1}, then c
+    StagedCtx c;
+    c.full = reinterpret_cast<uint64_t *>(pc + S::U * 2 * S::OWN_S);
+    uint64_t *const init = c.full + S::U;
+    c.abort_flag = reinterpret_cast<int *>(smem + S::ABORT_OFF);
+    const int tid = threadIdx.x;
+    int b = bid;
+    const int tx = b % g.tiles_x;
+    b /= g.tiles_x;
+    const int ty = b % g.tiles_y;
+    const int x0 = tx * S::TX, y0 = ty * S::TY, z0 = b / g.tiles_y * g.zlen;
+    c.z0 = z0;
+    const int T = min(a.nz - z0, g.zlen);
+
+    auto load_pc = [&](int t) {   // u^{n-1} and c of plane t into its stage
+        float *dst = pc + t % S::U * 2 * S::OWN_S;
+        tma_load_3d(dst, prev_map, x0, y0, z0 + t, &c.full[t % S::U]);
+        tma_load_3d(dst + S::OWN_S, c_map, x0, y0, z0 + t, &c.full[t % S::U]);
+    };
+    auto load_halo = [&](int p, uint64_t *bar) {   // u^n at z0 + p
+        tma_load_3d(ring + p % S::NSU * S::CUR_S, halo_map, x0 - kRadius, y0 - kRadius, z0 + p, bar);
+    };
+    if (tid == 0) {
+        if (dep.reinit()) {   // the previous unit consumed every copy it issued
+            for (int s = 0; s <= S::U; ++s) mbar_inval(&c.full[s]);
+        }
+        for (int s = 0; s <= S::U; ++s) mbar_init(&c.full[s], 1);
+        *c.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if constexpr (Dep::kProxyFence) __syncthreads();   // the flag is 0 before any waiter may set it
+    // c and u^{n-1} first where the dependency allows it (PdlDep), then wait, then u^n
+    const bool early = dep.early();
+    if (early && tid == 0) {
+        if constexpr (Dep::kProxyFence) fence_proxy_async_global();
+        for (int t = 0; t < S::U && t < T; ++t) {
+            mbar_expect_tx(&c.full[t], S::STAGE_BYTES);
+            load_pc(t);
+        }
+    }
+    dep.wait(tid, c.abort_flag, a.err);
+    __syncthreads();
+    const bool dep_ok = !*c.abort_flag;
+    if (tid == 0 && dep_ok) {
+        if constexpr (Dep::kProxyFence) fence_proxy_async_global();
+        mbar_expect_tx(init, S::FIRST_BYTES);
+        for (int p = 0; p < kRadius; ++p) {
+            int z = z0 - kRadius + p;
+            if (a.fs && z < 0) z = -z;   // plane -m is the odd image of plane m (negated when read)
+            tma_load_3d(first + p * S::OWN_S, own_map, x0, y0, z, init);
+        }
+        for (int p = 0; p < kRadius; ++p) load_halo(p, init);
+        for (int t = 0; t < S::U && t < T; ++t) {
+            if (!early) {
+                mbar_expect_tx(&c.full[t], S::STAGE_BYTES);
+                load_pc(t);
+            }
+            load_halo(t + kRadius, &c.full[t]);
+        }
+    }
+    int armed = dep_ok ? min(S::U, T) : 0;   // planes whose stage has been filled
+    // receivers of the previous step (u^n, read-only during this launch)
+    if (v.traces) {
+        for (int r = bid * S::NT + tid; r < a.nrec; r += nbid * S::NT)
+            v.traces[r] = v.ucur[__ldg(a.rec_off + r)];
+    }
+
+    Wts w;
+    w.x1 = a.w.x[0];
+    w.x2 = bcast(a.w.x[1]);
+    w.x3 = a.w.x[2];
+    w.x4 = bcast(a.w.x[3]);
+#pragma unroll
+    for (int m = 0; m < kRadius; ++m) {
+        w.y[m] = bcast(a.w.y[m]);
+        w.z[m] = bcast(a.w.z[m]);
+    }
+    const int px = tid % S::LX, py = tid / S::LX;
+    const int x = x0 + 2 * px, y = y0 + S::RY * py;
+    c.col = ring + S::RY * py * S::PITCH + 2 * px;
+    c.pc = pc + S::RY * py * S::TX + 2 * px;
+    float2 exr;
+    exr.x = x < a.nx ? __ldg(a.ex + x) : 0.0f;
+    exr.y = x + 1 < a.nx ? __ldg(a.ex + x + 1) : 0.0f;
+    const float eyr[S::RY] = {y < a.ny ? __ldg(a.ey + y) : 0.0f, y + 1 < a.ny ? __ldg(a.ey + y + 1) : 0.0f};
+    c.full0 = y < a.ny && x + 1 < a.nx;
+    c.full1 = y + 1 < a.ny && x + 1 < a.nx;
+    c.part0 = y < a.ny && x + 1 == a.nx;
+    c.part1 = y + 1 < a.ny && x + 1 == a.nx;
+    c.xy_damped = x0 < a.nbl || x0 + S::TX - 1 > a.nx - 1 - a.nbl || y0 < a.nbl ||
+                  y0 + S::TY - 1 > a.ny - 1 - a.nbl;
+    const long long off = (long long)z0 * a.plane + (long long)y * a.nxp + x;
+    float *out = v.uout + off;
+    float *gout = G ? a.gout + off : nullptr;
+
+    float2 q[S::QD][S::RY];
+    if (dep_ok && mbar_wait(init, 0, c.abort_flag, a.err)) {
+        const float *own = first + S::RY * py * S::TX + 2 * px;
+        const float *ctr = c.col + kRadius * S::PITCH + kRadius;
+#pragma unroll
+        for (int i = 0; i < kRadius; ++i) {
+#pragma unroll
+            for (int r = 0; r < S::RY; ++r) {
+                q[i][r] = *reinterpret_cast<const float2 *>(own + i * S::OWN_S + r * S::TX);
+                q[kRadius + i][r] = *reinterpret_cast<const float2 *>(ctr + i * S::CUR_S + r * S::PITCH);
+            }
+        }
+        if (a.fs && z0 < kRadius) {   // queue planes above k = 0 hold the images: negate
+#pragma unroll
+            for (int i = 0; i < kRadius; ++i)
+                if (i < kRadius - z0) {
+#pragma unroll
+                    for (int r = 0; r < S::RY; ++r) q[i][r] = neg2(q[i][r]);
+                }
+        }
+    }
+    // Plane t done by every thread: its centre slot and its u^{n-1} / c tiles
+    // are free and take plane t + 4's data.
+#define MMOD_STAGED(J)                                                                                              \
+    if (t + (J) < T) {                                                                                              \
+        staged_plane<S, (J), G>(a, c, z0 + t + (J), half, c.col + half * (4 * S::CUR_S),                            \
+                                c.col + (half ^ 1) * (4 * S::CUR_S), q, w, exr, eyr, out, gout);                    \
+        out += a.plane;                                                                                             \
+        if constexpr (G) gout += a.plane;                                                                           \
+        __syncthreads();                                                                                            \
+        if (tid == 0 && t + (J) + S::U < T && !*c.abort_flag) {                                                     \
+            mbar_expect_tx(&c.full[J], S::STAGE_BYTES);                                                             \
+            tma_load_3d(ring + (half * 4 + (J)) * S::CUR_S, halo_map, x0 - kRadius, y0 - kRadius,                   \
+                        z0 + t + (J) + 2 * S::U, &c.full[J]);                                                       \
+            tma_load_3d(pc + (J) * 2 * S::OWN_S, prev_map, x0, y0, z0 + t + (J) + S::U, &c.full[J]);                \
+            tma_load_3d(pc + (J) * 2 * S::OWN_S + S::OWN_S, c_map, x0, y0, z0 + t + (J) + S::U, &c.full[J]);        \
+            armed = t + (J) + S::U + 1;                                                                             \
+        }                                                                                                           \
+    }
+    unsigned half = 0;
+#pragma unroll 1
+    for (int t = 0; t < T; t += S::U, half ^= 1) {
+        if (*c.abort_flag) break;
+        MMOD_STAGED(0)
+        MMOD_STAGED(1)
+        MMOD_STAGED(2)
+        MMOD_STAGED(3)
+#pragma unroll
+        for (int i = 0; i < 2 * kRadius; ++i)
+#pragma unroll
+            for (int r = 0; r < S::RY; ++r) q[i][r] = q[i + S::U][r];
+    }
+#undef MMOD_STAGED
+    // Sources of this CTA's tile and planes: nothing in this launch reads the
+    // u^{n+1} it writes, so they are added once the whole z range is stored
+    // (the block barrier makes every thread's stores visible).  The points of
+    // one tile over planes [z0, z0 + T) are one run of the table.
+    __syncthreads();
+    if (!*c.abort_flag && a.inj.npts > 0) {
+        const long long bucket = ((long long)ty * a.inj.tiles_x + tx) * a.nz + z0;
+        const int lo = __ldg(a.inj.tile_start + bucket), hi = __ldg(a.inj.tile_start + bucket + T);
+        inject_points(a, v.uout, v.n, lo, hi, tid, S::NT);
+        if constexpr (G) inject_g_points(a, v.n, lo, hi, tid, S::NT);
+    }
+    // After a give-up, wait (bounded) for the copies this CTA still has in
+    // flight (the first planes and the latest phase of every stage) before its
+    // shared memory is released.
+    if (*c.abort_flag && tid == 0 && dep_ok) {
+        mbar_drain(init, 0);
+        for (int t = max(0, armed - S::U); t < armed; ++t) mbar_drain(&c.full[t % S::U], (t / S::U) & 1);
+    }
+}
+
+}  // namespace
+}  // namespace mmod
