@@ -279,11 +279,23 @@ cudaError_t restore_state(mmod_handle *h, int slot, float *u_prev, float *u_cur,
     return cudaGetLastError();
 }
 
+// Tensor maps of the work volumes for the run's tile shape.
+mmod_status encode_grad_maps(mmod_handle *h, int shape) {
+    auto &gw = h->gw;
+    if (gw.shape == shape || !h->tma_ok) return MMOD_OK;
+    bool ok = true;
+    for (int i = 0; i < gw.nwork; ++i) ok = ok && encode_maps(h->cfg, h->nxp, gw.seg[i], shape, &gw.seg_map[i]);
+    for (int b = 0; b < 2; ++b) ok = ok && encode_maps(h->cfg, h->nxp, gw.psi[b], shape, &gw.psi_map[b]);
+    if (!ok) return fail(h, MMOD_ERR_CUDA, "tensor map encoding failed for a work volume");
+    gw.shape = shape;
+    return MMOD_OK;
+}
+
 // Allocate (or keep) the gradient work space: nslot checkpoints of two
 // volumes, nwork FP32 work volumes (with tensor maps), psi, grad_c.
-mmod_status ensure_grad_work(mmod_handle *h, int nslot, int nwork, int dtype) {
+mmod_status ensure_grad_work(mmod_handle *h, int nslot, int nwork, int dtype, int shape) {
     auto &gw = h->gw;
-    if (gw.nslot == nslot && gw.nwork == nwork && gw.dtype == dtype) return MMOD_OK;
+    if (gw.nslot == nslot && gw.nwork == nwork && gw.dtype == dtype) return encode_grad_maps(h, shape);
     free_grad_work(h);
     const size_t vb = sizeof(float) * (size_t)h->vol;
     gw.seg.assign(nwork, nullptr);
@@ -291,14 +303,8 @@ mmod_status ensure_grad_work(mmod_handle *h, int nslot, int nwork, int dtype) {
     for (int i = 0; i < nwork; ++i) {
         MMOD_CK(h, cudaMalloc(&gw.seg[i], vb));
         MMOD_CK(h, cudaMemset(gw.seg[i], 0, vb));
-        if (h->tma_ok && !encode_maps(h->cfg, h->nxp, gw.seg[i], &gw.seg_map[i]))
-            return fail(h, MMOD_ERR_CUDA, "tensor map encoding failed for a work volume");
     }
-    for (int b = 0; b < 2; ++b) {
-        MMOD_CK(h, cudaMalloc(&gw.psi[b], vb));
-        if (h->tma_ok && !encode_maps(h->cfg, h->nxp, gw.psi[b], &gw.psi_map[b]))
-            return fail(h, MMOD_ERR_CUDA, "tensor map encoding failed for an adjoint buffer");
-    }
+    for (int b = 0; b < 2; ++b) MMOD_CK(h, cudaMalloc(&gw.psi[b], vb));
     MMOD_CK(h, cudaMalloc(&gw.gradc, vb));
     gw.ckpt_bytes = (size_t)nslot * 2 * (size_t)h->vol * ckpt_elem_bytes(dtype);
     if (nslot > 0) MMOD_CK(h, cudaMalloc(&gw.ckpt, gw.ckpt_bytes));
@@ -307,7 +313,7 @@ mmod_status ensure_grad_work(mmod_handle *h, int nslot, int nwork, int dtype) {
     gw.nslot = nslot;
     gw.nwork = nwork;
     gw.dtype = dtype;
-    return MMOD_OK;
+    return encode_grad_maps(h, shape);
 }
 
 // Checkpoint layout of a gradient call: slots and FP32 work volumes.
@@ -367,7 +373,7 @@ void free_grad_work(mmod_handle *h) {
     gw.ckpt = nullptr;
     gw.ckpt_scale = nullptr;
     gw.nslot = gw.nwork = 0;
-    gw.dtype = -1;
+    gw.dtype = gw.shape = -1;
     gw.ckpt_bytes = 0;
 }
 
@@ -435,7 +441,10 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
     const int nt = c.nt;
     int nslot = 0, nwork = 0, seglen = 0;
     grad_layout(h, ckpt_count, ckpt_dtype, &nslot, &nwork, &seglen);
-    if (mmod_status st = ensure_grad_work(h, nslot, nwork, ckpt_dtype)) return st;
+    const int shape = active_shape(h);
+    if (mmod_status st = ensure_shape(h, shape)) return st;
+    if (mmod_status st = ensure_grad_work(h, nslot, nwork, ckpt_dtype, shape)) return st;
+    const VolMaps *u_map = h->shapes[shape].u;
     auto &gw = h->gw;
     const bool tma = use_tma(h);
     long long launches = 0;
@@ -451,10 +460,10 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
     MMOD_CK(h, cudaMemsetAsync(h->u[0], 0, vb, s));
     MMOD_CK(h, cudaMemsetAsync(h->u[1], 0, vb, s));
     h->state_pending = false;
-    StepArgs fa = base_args(h, h->fwd, dwav);
+    StepArgs fa = base_args(h, h->fwd, dwav, shape);
     fa.nrec = 0;   // no receivers in the gradient's forward sweeps
     fa.inv_cell = (float)(1.0 / (c.hx * c.hy * c.hz));
-    StepArgs aa = base_args(h, h->adj, h->st_adjw);
+    StepArgs aa = base_args(h, h->adj, h->st_adjw, shape);
     aa.nrec = 0;
     // forward step n in place on the handle's buffers: u^{n-1} in u[n & 1],
     // u^n in u[(n + 1) & 1], u^{n+1} over u^{n-1}
@@ -463,7 +472,7 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
         fa.ucur = h->u[(n + 1) & 1];
         fa.uprev = h->u[n & 1];
         fa.uout = h->u[n & 1];
-        return enqueue_step(h, fa, h->u_map[(n + 1) & 1], h->u_map[n & 1], tma, nullptr, s, &launches);
+        return enqueue_step(h, fa, u_map[(n + 1) & 1], u_map[n & 1], tma, nullptr, s, &launches);
     };
     // forward step n of a replay in the work volumes w0, w1 (u^{n-1} in w0,
     // u^n in w1, u^{n+1} over u^{n-1}), also writing g^n into gout
@@ -558,7 +567,7 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
                     fa.uprev = h->u[n & 1];
                     fa.uout = unext;
                     fa.gout = gn;
-                    const cudaError_t e = enqueue_step(h, fa, h->u_map[(n + 1) & 1], h->u_map[n & 1], tma,
+                    const cudaError_t e = enqueue_step(h, fa, u_map[(n + 1) & 1], u_map[n & 1], tma,
                                                        nullptr, s, &launches);
                     fa.gout = nullptr;
                     MMOD_CK(h, e);

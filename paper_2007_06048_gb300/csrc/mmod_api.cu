@@ -67,10 +67,9 @@ std::string validate(const mmod_config *c, mmod_status *st) {
 }
 
 void free_inj(DevInj &t) {
-    for (int *p : {t.tile_start, t.pt_i, t.pt_j, t.pt_k, t.pt_first, t.src_row, t.src_i, t.src_j, t.src_k})
+    for (int *p : {t.tile_start, t.pt_i, t.pt_j, t.pt_k, t.pt_first, t.src_row})
         if (p) cudaFree(p);
     if (t.pt_off) cudaFree(t.pt_off);
-    if (t.src_scale) cudaFree(t.src_scale);
     t = DevInj();
 }
 
@@ -86,9 +85,11 @@ void free_all(mmod_handle *h) {
     for (float *p : {h->u[0], h->u[1], h->c, h->eta, h->vel_copy, h->st_vol, h->st_wav, h->st_tr, h->st_adjw,
                      h->st_adjg, h->st_adjo})
         if (p) cudaFree(p);
-    free_inj(h->fwd.inj);
-    free_inj(h->adj.inj);
     for (Geometry *g : {&h->fwd, &h->adj}) {
+        for (DevInj &t : g->inj) free_inj(t);
+        for (int *p : {g->si, g->sj, g->sk})
+            if (p) cudaFree(p);
+        if (g->scale) cudaFree(g->scale);
         if (g->gather_off) cudaFree(g->gather_off);
         if (g->g_start) cudaFree(g->g_start);
         if (g->g_idx) cudaFree(g->g_idx);
@@ -121,62 +122,95 @@ cudaError_t upload(T **dst, const std::vector<T> &v) {
     return cudaMemcpy(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice);
 }
 
+// Indices 0 .. n-1 in stable ascending order of key (>= 0): radix sort, 16
+// bits per pass (a million receivers in a few milliseconds).
+std::vector<int> order_by_key(const std::vector<long long> &key) {
+    const int n = (int)key.size();
+    std::vector<int> order(n), tmp(n);
+    std::iota(order.begin(), order.end(), 0);
+    if (n < 4096) {
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return key[a] < key[b]; });
+        return order;
+    }
+    const long long top = *std::max_element(key.begin(), key.end());
+    std::vector<int> count(65537);
+    for (int shift = 0; shift < 63 && (top >> shift) > 0; shift += 16) {
+        std::fill(count.begin(), count.end(), 0);
+        for (int q = 0; q < n; ++q) ++count[((key[q] >> shift) & 0xffff) + 1];
+        for (int d = 0; d < 65536; ++d) count[d + 1] += count[d];
+        for (int q = 0; q < n; ++q) tmp[count[(key[order[q]] >> shift) & 0xffff]++] = order[q];
+        order.swap(tmp);
+    }
+    return order;
+}
+
 // Injection table of the positions pos[n][3]: sources grouped by grid point
 // (stable order), points sorted by (tile, plane, j, i) and bucketed per
-// (64 x 16 tile, plane).  src_row = index of the position in pos.
-cudaError_t build_inj(const mmod_config &c, long long plane, int nxp, const int *pos, int n, DevInj *t) {
-    t->tiles_x = (c.nx + kInjTileX - 1) / kInjTileX;
-    t->tiles_y = (c.ny + kInjTileY - 1) / kInjTileY;
+// (tile of the shape, plane).  src_row = index of the position in pos.
+cudaError_t build_inj(const mmod_config &c, long long plane, int nxp, const int *pos, int n, const TmaShape &sh,
+                      DevInj *t) {
+    t->tiles_x = (c.nx + sh.tx - 1) / sh.tx;
+    t->tiles_y = (c.ny + sh.ty - 1) / sh.ty;
     const long long tiles = (long long)t->tiles_x * t->tiles_y;
-    auto bucket = [&](int s) {
-        const int *p = pos + 3 * s;
-        return ((long long)(p[1] / kInjTileY) * t->tiles_x + p[0] / kInjTileX) * c.nz + p[2];
-    };
-    // with a free surface, positions on the plane k = 0 inject nothing
-    std::vector<int> order;
-    for (int q = 0; q < n; ++q)
-        if (!(c.free_surface && pos[3 * q + 2] == 0)) order.push_back(q);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        const long long ba = bucket(a), bb = bucket(b);
-        if (ba != bb) return ba < bb;
-        const int *pa = pos + 3 * a, *pb = pos + 3 * b;
-        if (pa[1] != pb[1]) return pa[1] < pb[1];
-        return pa[0] < pb[0];
-    });
+    // bucket, then (j, i) within the tile, of every position that injects
+    // (with a free surface, positions on the plane k = 0 inject nothing)
+    const long long area = (long long)sh.tx * sh.ty;
+    std::vector<long long> key;
+    std::vector<int> kept;
+    key.reserve(n);
+    kept.reserve(n);
+    for (int q = 0; q < n; ++q) {
+        const int *p = pos + 3 * q;
+        if (c.free_surface && p[2] == 0) continue;
+        const int ty = p[1] / sh.ty, tx = p[0] / sh.tx;
+        const long long bucket = ((long long)ty * t->tiles_x + tx) * c.nz + p[2];
+        key.push_back(bucket * area + (long long)(p[1] - ty * sh.ty) * sh.tx + (p[0] - tx * sh.tx));
+        kept.push_back(q);
+    }
+    const std::vector<int> order = order_by_key(key);
     const int m = (int)order.size();
-    std::vector<int> pt_i, pt_j, pt_k, pt_first, src_row(m), si(m), sj(m), sk(m);
+    std::vector<int> pt_i, pt_j, pt_k, pt_first, src_row(m);
     std::vector<long long> pt_off;
     std::vector<int> tile_start((size_t)(c.nz * tiles + 1), 0);
     for (int q = 0; q < m; ++q) {
-        const int s = order[q];
+        const int s = kept[order[q]];
         const int *p = pos + 3 * s;
         src_row[q] = s;
-        si[q] = p[0];
-        sj[q] = p[1];
-        sk[q] = p[2];
-        const bool same = q > 0 && std::memcmp(pos + 3 * order[q - 1], p, 3 * sizeof(int)) == 0;
+        const bool same = q > 0 && key[order[q]] == key[order[q - 1]];
         if (!same) {
             pt_i.push_back(p[0]);
             pt_j.push_back(p[1]);
             pt_k.push_back(p[2]);
             pt_off.push_back((long long)p[2] * plane + (long long)p[1] * nxp + p[0]);
             pt_first.push_back(q);
-            tile_start[(size_t)bucket(s) + 1]++;
+            tile_start[(size_t)(key[order[q]] / area) + 1]++;
         }
     }
     pt_first.push_back(m);
     for (size_t b = 1; b < tile_start.size(); ++b) tile_start[b] += tile_start[b - 1];
     t->npts = (int)pt_i.size();
-    t->nsrc = m;
     cudaError_t e;
     if ((e = upload(&t->tile_start, tile_start)) || (e = upload(&t->pt_i, pt_i)) || (e = upload(&t->pt_j, pt_j)) ||
         (e = upload(&t->pt_k, pt_k)) || (e = upload(&t->pt_off, pt_off)) || (e = upload(&t->pt_first, pt_first)) ||
-        (e = upload(&t->src_row, src_row)) || (e = upload(&t->src_i, si)) || (e = upload(&t->src_j, sj)) ||
-        (e = upload(&t->src_k, sk)))
+        (e = upload(&t->src_row, src_row)))
         return e;
-    e = cudaMalloc(&t->src_scale, sizeof(float) * std::max(m, 1));
-    if (e != cudaSuccess) return e;
-    return cudaMemset(t->src_scale, 0, sizeof(float) * std::max(m, 1));
+    return cudaSuccess;
+}
+
+// The positions of a geometry's injections, in the caller's order, and room
+// for their scales.
+cudaError_t build_positions(const int *pos, int n, Geometry *g) {
+    std::vector<int> si(n), sj(n), sk(n);
+    for (int q = 0; q < n; ++q) {
+        si[q] = pos[3 * q];
+        sj[q] = pos[3 * q + 1];
+        sk[q] = pos[3 * q + 2];
+    }
+    g->npos = n;
+    cudaError_t e;
+    if ((e = upload(&g->si, si)) || (e = upload(&g->sj, sj)) || (e = upload(&g->sk, sk))) return e;
+    if ((e = cudaMalloc(&g->scale, sizeof(float) * std::max(n, 1)))) return e;
+    return cudaMemset(g->scale, 0, sizeof(float) * std::max(n, 1));
 }
 
 // Gather positions pos[n][3] bucketed per (64 x 16 tile, plane), tile-major
@@ -185,13 +219,12 @@ cudaError_t build_inj(const mmod_config &c, long long plane, int nxp, const int 
 cudaError_t build_gather_buckets(const mmod_config &c, long long plane, int nxp, const int *pos, int n,
                                  Geometry *g) {
     const int tiles_x = (c.nx + kInjTileX - 1) / kInjTileX, tiles_y = (c.ny + kInjTileY - 1) / kInjTileY;
-    auto bucket = [&](int r) {
+    std::vector<long long> bucket(n);
+    for (int r = 0; r < n; ++r) {
         const int *p = pos + 3 * r;
-        return ((long long)(p[1] / kInjTileY) * tiles_x + p[0] / kInjTileX) * c.nz + p[2];
-    };
-    std::vector<int> order(n);
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return bucket(a) < bucket(b); });
+        bucket[r] = ((long long)(p[1] / kInjTileY) * tiles_x + p[0] / kInjTileX) * c.nz + p[2];
+    }
+    const std::vector<int> order = order_by_key(bucket);
     std::vector<int> start((size_t)tiles_x * tiles_y * c.nz + 1, 0), idx(n);
     std::vector<long long> off(n);
     for (int q = 0; q < n; ++q) {
@@ -199,7 +232,7 @@ cudaError_t build_gather_buckets(const mmod_config &c, long long plane, int nxp,
         const int *p = pos + 3 * r;
         idx[q] = r;
         off[q] = (long long)p[2] * plane + (long long)p[1] * nxp + p[0];
-        start[(size_t)bucket(r) + 1]++;
+        start[(size_t)bucket[r] + 1]++;
     }
     for (size_t b = 1; b < start.size(); ++b) start[b] += start[b - 1];
     cudaError_t e;
@@ -351,24 +384,57 @@ static const TmaPlan &plan_with_options(const mmod_handle *h, int v, TmaPlan &q)
     return q;
 }
 
-const TmaPlan &active_plan(const mmod_handle *h) {
-    return plan_with_options(h, h->variant >= 0 ? h->variant : kTmaDefaultVariant, h->plan_tmp);
+// The variant of the next run: the caller's choice, else the handle's own; the
+// persistent and work-claiming forms exist for the default variant only.
+static int active_variant(const mmod_handle *h) {
+    if (h->variant >= 0) return h->variant;
+    return h->persistent || h->claim_planes > 0 ? kTmaDefaultVariant : h->auto_variant;
 }
 
-// Steps that also write g^n run the variant compiled with that output (the
-// same bits as every other variant).
-static const TmaPlan &g_plan(const mmod_handle *h) { return plan_with_options(h, kTmaGVariant, h->plan_tmp_g); }
+const TmaPlan &active_plan(const mmod_handle *h) { return plan_with_options(h, active_variant(h), h->plan_tmp); }
+
+int active_shape(const mmod_handle *h) { return h->tma_ok ? h->plans[active_variant(h)].shape : 0; }
+
+// Steps that also write g^n: the active variant where it has that output, else
+// the default variant (shape 0, as every variant without it; the same bits).
+static const TmaPlan &g_plan(const mmod_handle *h) {
+    const int v = active_variant(h);
+    return plan_with_options(h, h->plans[v].has_g ? v : kTmaDefaultVariant, h->plan_tmp_g);
+}
+
+mmod_status ensure_shape(mmod_handle *h, int shape) {
+    auto &m = h->shapes[shape];
+    if (m.ready) return MMOD_OK;
+    const mmod_config &c = h->cfg;
+    if (h->tma_ok) {
+        bool ok = encode_maps(c, h->nxp, h->c, shape, &m.c);
+        for (int b = 0; b < 2; ++b) ok = ok && encode_maps(c, h->nxp, h->u[b], shape, &m.u[b]);
+        if (!ok) return fail(h, MMOD_ERR_CUDA, "tensor map encoding failed");
+    }
+    const TmaShape &sh = kTmaShapes[shape];
+    try {
+        for (Geometry *g : {&h->fwd, &h->adj}) {
+            free_inj(g->inj[shape]);   // left by an attempt that failed half way
+            const auto &pos = g == &h->fwd ? h->src : h->rec;
+            MMOD_CK(h, build_inj(c, h->plane, h->nxp, pos.data(), g->npos, sh, &g->inj[shape]));
+        }
+    } catch (const std::bad_alloc &) {
+        return fail(h, MMOD_ERR_OOM, "host memory for the injection tables");
+    }
+    m.ready = true;
+    return MMOD_OK;
+}
 
 // Step arguments shared by every step of a run (n, buffers and gathers are
 // filled per step).
-StepArgs base_args(mmod_handle *h, const Geometry &geo, const float *wavelet) {
+StepArgs base_args(mmod_handle *h, const Geometry &geo, const float *wavelet, int shape) {
     StepArgs a{};
     a.nx = h->cfg.nx; a.ny = h->cfg.ny; a.nz = h->cfg.nz;
     a.nxp = h->nxp; a.plane = h->plane; a.nbl = h->cfg.nbl; a.nt = h->cfg.nt;
     a.w = h->w;
     a.c = h->c;
     a.ex = h->eta; a.ey = h->eta + h->cfg.nx; a.ez = h->eta + h->cfg.nx + h->cfg.ny;
-    a.inj = geo.inj.view();
+    a.inj = geo.view(shape);
     a.wavelet = wavelet;
     a.wrs = h->cfg.nt;
     a.wcs = 1;
@@ -395,7 +461,7 @@ cudaError_t enqueue_step(mmod_handle *h, const StepArgs &a, const VolMaps &cur, 
                          float *plain_gather_dst, cudaStream_t s, long long *count) {
     cudaError_t e;
     if (tma) {
-        e = launch_step_tma(a, cur, prev, h->c_map, a.gout ? g_plan(h) : active_plan(h), s);
+        e = launch_step_tma(a, cur, prev, h->shapes[active_shape(h)].c.own, a.gout ? g_plan(h) : active_plan(h), s);
         ++*count;
         return e;
     }
@@ -433,7 +499,9 @@ static mmod_status enqueue_loop(mmod_handle *h, const Geometry &geo, const float
         return cudaSuccess;
     };
     MMOD_CK(h, mark(0));
-    StepArgs a = base_args(h, geo, wav);
+    const int shape = active_shape(h);
+    const VolMaps *u_map = h->shapes[shape].u;
+    StepArgs a = base_args(h, geo, wav, shape);
     if (is_cpml(h)) {
         // CPML: the undamped step (sources included), the layer terms of
         // u^{n+1}, then (plain kernel) the receivers of u^{n+1}
@@ -449,7 +517,7 @@ static mmod_status enqueue_loop(mmod_handle *h, const Geometry &geo, const float
             a.uprev = h->u[n & 1];
             a.uout = h->u[n & 1];
             a.traces = (n >= 1 && tr && ng > 0) ? tr + (long long)(n - 1) * ng : nullptr;
-            MMOD_CK(h, enqueue_step(h, a, h->u_map[(n + 1) & 1], h->u_map[n & 1], tma, nullptr, s, count));
+            MMOD_CK(h, enqueue_step(h, a, u_map[(n + 1) & 1], u_map[n & 1], tma, nullptr, s, count));
             int passes = 0;
             MMOD_CK(h, launch_cpml_layers(cp, &h->cpml_tiles, (n + 1) & 1, a.ucur, a.uout, s, &passes));
             *count += passes;
@@ -476,7 +544,7 @@ static mmod_status enqueue_loop(mmod_handle *h, const Geometry &geo, const float
         a.uprev = h->u[n & 1];
         a.uout = h->u[n & 1];
         a.traces = (n >= 1 && tr && ng > 0) ? tr + (long long)(n - 1) * ng : nullptr;
-        MMOD_CK(h, enqueue_step(h, a, h->u_map[(n + 1) & 1], h->u_map[n & 1], tma,
+        MMOD_CK(h, enqueue_step(h, a, u_map[(n + 1) & 1], u_map[n & 1], tma,
                                 (tr && ng > 0) ? tr + (long long)n * ng : nullptr, s, count));
         MMOD_CK(h, mark(tma ? n : n + 1));   // the TMA kernel of step n gathers row n - 1
     }
@@ -494,7 +562,8 @@ static mmod_status enqueue_loop(mmod_handle *h, const Geometry &geo, const float
 // changed.
 mmod_status run_loop_graph(mmod_handle *h, GraphSlot &g, const Geometry &geo, const float *wav, float *tr,
                            cudaStream_t s, long long *launches) {
-    const int pgrid = persistent_grid_of(h);
+    const int pgrid = persistent_grid_of(h), shape = active_shape(h);
+    if (mmod_status st = ensure_shape(h, shape)) return st;
     if (pgrid > 0 && h->cfg.nt > 0) {
         // one cooperative launch for the whole loop: no graph needed
         const TmaPlan &plan = active_plan(h);
@@ -503,7 +572,7 @@ mmod_status run_loop_graph(mmod_handle *h, GraphSlot &g, const Geometry &geo, co
         MMOD_CK(h, cudaMemsetAsync(h->counters, 0, sizeof(int) * (size_t)units, s));
         MMOD_CK(h, cudaMemsetAsync(h->queue, 0, sizeof(unsigned long long), s));
         MMOD_CK(h, cudaEventRecord(h->ev_t0, s));
-        StepArgs a = base_args(h, geo, wav);
+        StepArgs a = base_args(h, geo, wav, shape);
         a.pdl = 0;
         PersistArgs pa{};
         // MMOD_OPT_TEST_STALL: start at step 1 with the counters at 0, so
@@ -523,10 +592,10 @@ mmod_status run_loop_graph(mmod_handle *h, GraphSlot &g, const Geometry &geo, co
         pa.u[1] = h->u[1];
         TmaMaps maps;
         for (int b = 0; b < 2; ++b) {
-            maps.cur[b] = h->u_map[b].halo;
-            maps.prev[b] = h->u_map[b].own;
+            maps.cur[b] = h->shapes[shape].u[b].halo;
+            maps.prev[b] = h->shapes[shape].u[b].own;
         }
-        maps.c = h->c_map;
+        maps.c = h->shapes[shape].c.own;
         MMOD_CK(h, launch_step_tma_persistent(a, maps, plan, pa, pgrid, s));
         MMOD_CK(h, cudaEventRecord(h->ev_t1, s));
         *launches += 1;
@@ -649,11 +718,11 @@ MMOD_API mmod_status mmod_create(const mmod_config *cfg, int device, mmod_handle
     CKC(cudaMalloc(&h->vmax_bits, sizeof(unsigned int)));
     CKC(cudaMalloc(&h->bad, sizeof(unsigned long long)));
     // forward: sources injected, receivers gathered; adjoint: the reverse
-    CKC(build_inj(h->cfg, h->plane, h->nxp, h->src.data(), cfg->nsrc, &h->fwd.inj));
+    CKC(build_positions(h->src.data(), cfg->nsrc, &h->fwd));
     CKC(build_gather(h->plane, h->nxp, h->rec.data(), cfg->nrec, &h->fwd.gather_off));
     h->fwd.ngather = cfg->nrec;
     h->fwd.cell = cfg->hx * cfg->hy * cfg->hz;
-    CKC(build_inj(h->cfg, h->plane, h->nxp, h->rec.data(), cfg->nrec, &h->adj.inj));
+    CKC(build_positions(h->rec.data(), cfg->nrec, &h->adj));
     CKC(build_gather(h->plane, h->nxp, h->src.data(), cfg->nsrc, &h->adj.gather_off));
     h->adj.ngather = cfg->nsrc;
     h->adj.cell = 1.0;
@@ -672,7 +741,13 @@ MMOD_API mmod_status mmod_create(const mmod_config *cfg, int device, mmod_handle
     *h->err_host = 0;
     CKC(cudaHostGetDevicePointer(&h->err_dev, h->err_host, 0));
     if (is_cpml(h)) make_cpml_tiles(cpml_args(h), h->u, &h->cpml_tiles);   // axes it cannot tile keep the march
-    h->tma_ok = make_tma_plan(h->cfg, h->nxp, h->u, h->c, h->u_map, &h->c_map, h->plans);
+    h->tma_ok = make_tma_plan(h->cfg, h->plans);
+    if (h->tma_ok) h->auto_variant = auto_tma_variant(h->plans);
+    if (ensure_shape(h, active_shape(h)) != MMOD_OK) {   // maps the encoder rejects: the plain kernel
+        h->tma_ok = false;
+        h->latched = cudaSuccess;
+        if (ensure_shape(h, 0) != MMOD_OK) return bail(cudaErrorMemoryAllocation, h->err.c_str());
+    }
     if (h->tma_ok) {   // counters of the persistent kernel, sized for the plan with the most units
         for (int v = 0; v < tma_variant_count(); ++v)
             h->ncounters = std::max<long long>(h->ncounters, (long long)h->plans[v].tiles_x * h->plans[v].tiles_y *
@@ -818,8 +893,7 @@ MMOD_API mmod_status mmod_set_model(mmod_handle *h, const float *vel, mmod_strea
     MMOD_CK(h, launch_model_fill(dvel, c.nx, c.ny, c.nz, h->nxp, c.dt, h->c, s));
     if (is_cpml(h)) MMOD_CK(h, launch_cpml_pack_c(cpml_args(h), s));
     for (Geometry *g : {&h->fwd, &h->adj})
-        MMOD_CK(h, launch_source_scale(dvel, c.nx, c.ny, g->inj.nsrc, g->inj.src_i, g->inj.src_j, g->inj.src_k,
-                                       c.dt, g->cell, g->inj.src_scale, s));
+        MMOD_CK(h, launch_source_scale(dvel, c.nx, c.ny, g->npos, g->si, g->sj, g->sk, c.dt, g->cell, g->scale, s));
     if (!h->vel_copy) MMOD_CK(h, cudaMalloc(&h->vel_copy, sizeof(float) * (size_t)h->npts));
     MMOD_CK(h, cudaMemcpyAsync(h->vel_copy, dvel, sizeof(float) * (size_t)h->npts, cudaMemcpyDeviceToDevice, s));
     std::vector<float> eta(c.nx + c.ny + c.nz);

@@ -116,6 +116,22 @@ mmod_status enqueue_batch_steps(mmod_batch *b, int n0, int n1, cudaStream_t s) {
     return MMOD_OK;
 }
 
+// The maps and arguments of the fused and persistent kernels (64 x 16 tiles).
+mmod_status fill_desc(mmod_batch *b) {
+    for (size_t i = 0; i < b->shots.size(); ++i) {
+        mmod_handle *h = b->shots[i];
+        if (mmod_status st = ensure_shape(h, 0)) return bfail(b, st, "shot " + std::to_string(i) + ": " + h->err);
+        ShotDesc &d = b->desc[i];
+        for (int k = 0; k < 2; ++k) {
+            d.cur[k] = h->shapes[0].u[k].halo;
+            d.prev[k] = h->shapes[0].u[k].own;
+        }
+        d.cmap = h->shapes[0].c.own;
+        d.args = base_args(h, h->fwd, nullptr, 0);
+    }
+    return MMOD_OK;
+}
+
 mmod_status zero_states(mmod_batch *b, cudaStream_t s) {
     for (mmod_handle *h : b->shots) {
         BCK(b, cudaMemsetAsync(h->u[0], 0, sizeof(float) * (size_t)h->vol, s));
@@ -168,7 +184,10 @@ namespace mmod {
 mmod_status enqueue_tune_steps(mmod_handle *h, int steps, cudaStream_t s) {
     MMOD_CK(h, cudaMemsetAsync(h->u[0], 0, sizeof(float) * (size_t)h->vol, s));
     MMOD_CK(h, cudaMemsetAsync(h->u[1], 0, sizeof(float) * (size_t)h->vol, s));
-    StepArgs a = base_args(h, h->fwd, nullptr);
+    const int shape = active_shape(h);
+    if (mmod_status st = ensure_shape(h, shape)) return st;
+    const VolMaps *u_map = h->shapes[shape].u;
+    StepArgs a = base_args(h, h->fwd, nullptr, shape);
     a.inj.npts = 0;   // no sources while tuning
     a.nrec = 0;
     long long count = 0;
@@ -177,7 +196,7 @@ mmod_status enqueue_tune_steps(mmod_handle *h, int steps, cudaStream_t s) {
         a.ucur = h->u[(n + 1) & 1];
         a.uprev = h->u[n & 1];
         a.uout = h->u[n & 1];
-        MMOD_CK(h, enqueue_step(h, a, h->u_map[(n + 1) & 1], h->u_map[n & 1], true, nullptr, s, &count));
+        MMOD_CK(h, enqueue_step(h, a, u_map[(n + 1) & 1], u_map[n & 1], true, nullptr, s, &count));
     }
     h->state_pending = false;
     h->ran = false;
@@ -223,12 +242,8 @@ MMOD_API mmod_status mmod_batch_create(mmod_handle *const *shots, int nshots, mm
         d.rec_idx = h->fwd.g_idx;
         d.rec_boff = h->fwd.g_off;
         for (int k = 0; k < 2; ++k) {
-            d.cur[k] = h->u_map[k].halo;
-            d.prev[k] = h->u_map[k].own;
             d.u[k] = h->u[k];
         }
-        d.cmap = h->c_map;
-        d.args = base_args(h, h->fwd, nullptr);
         const TmaPlan &p = h->plans[0];
         // MMOD_OPT_ZLEN of the shot, at least the stencil radius (a persistent
         // unit's halo then reaches only the adjacent z ranges)
@@ -310,7 +325,7 @@ MMOD_API const char *mmod_batch_last_error(const mmod_batch *b) { return b ? b->
 MMOD_API mmod_status mmod_batch_set_variant(mmod_batch *b, int v) {
     if (!b) return MMOD_ERR_ARG;
     int block, smem;
-    if (v < 0 || !tma_variant_shape(v, &block, &smem)) return bfail(b, MMOD_ERR_ARG, "unknown TMA variant");
+    if (!tma_variant_has_batch(v) || !tma_variant_shape(v, &block, &smem)) return bfail(b, MMOD_ERR_ARG, "unknown TMA variant");
     b->variant = v;
     b->variant_set = true;
     for (mmod_handle *h : b->shots) h->variant = v;   // streams mode runs each handle's own plan
@@ -356,6 +371,7 @@ MMOD_API mmod_status mmod_batch_forward(mmod_batch *b, const float *const *wavel
         b->ran = b->nt > 0;
         return MMOD_OK;
     }
+    if (mmod_status st = fill_desc(b)) return st;
     for (int i = 0; i < ns; ++i) {
         mmod_handle *h = b->shots[i];
         if (mmod_status st = check_latched(h)) return bfail(b, st, "shot " + std::to_string(i) + ": " + h->err);
@@ -508,11 +524,12 @@ MMOD_API mmod_status mmod_batch_autotune(mmod_batch *b, int steps, mmod_stream s
         cudaEventDestroy(e1);
         for (mmod_handle *h : b->shots) h->variant = best;
         if (st != MMOD_OK) return bfail(b, st, "autotuning the batch failed");
-        b->variant = best;
+        if (tma_variant_has_batch(best)) b->variant = best;   // the fused mode's kernels: 64 x 16 tiles only
         b->variant_set = true;
         if (variant_out) *variant_out = best;
         return MMOD_OK;
     }
+    if (mmod_status st = fill_desc(b)) return st;
     for (int i = 0; i < ns; ++i) {
         if (!b->shots[i]->model_set) return bfail(b, MMOD_ERR_STATE, "shot " + std::to_string(i) + " has no model");
         b->desc[i].args.wavelet = nullptr;   // no sources while tuning
@@ -526,6 +543,7 @@ MMOD_API mmod_status mmod_batch_autotune(mmod_batch *b, int steps, mmod_stream s
     int best = keep;
     float best_ms = 1e30f;
     for (int v = 0; v < tma_variant_count(); ++v) {
+        if (!tma_variant_has_batch(v)) continue;
         b->variant = v;
         mmod_status st;
         time_steps(b, std::min(2, steps), s, &st);   // warm-up
@@ -539,7 +557,6 @@ MMOD_API mmod_status mmod_batch_autotune(mmod_batch *b, int steps, mmod_stream s
             best = v;
         }
     }
-    for (int i = 0; i < ns; ++i) b->desc[i].args.inj.npts = b->shots[i]->fwd.inj.npts;
     b->variant = best;
     if (variant_out) *variant_out = best;
     return MMOD_OK;

@@ -10,28 +10,31 @@
 
 namespace mmod {
 
-// Device-side injection table (see InjTable) plus the per-source positions
-// the scale kernel reads.
+// Device-side injection table for one tile shape (see InjTable).
 struct DevInj {
     int *tile_start = nullptr, *pt_i = nullptr, *pt_j = nullptr, *pt_k = nullptr, *pt_first = nullptr;
-    int *src_row = nullptr, *src_i = nullptr, *src_j = nullptr, *src_k = nullptr;
+    int *src_row = nullptr;
     long long *pt_off = nullptr;
-    float *src_scale = nullptr;
-    int npts = 0, nsrc = 0, tiles_x = 0, tiles_y = 0;
-    InjTable view() const {
-        InjTable t;
-        t.tile_start = tile_start; t.pt_i = pt_i; t.pt_j = pt_j; t.pt_k = pt_k; t.pt_off = pt_off;
-        t.pt_first = pt_first; t.src_row = src_row; t.src_scale = src_scale;
-        t.tiles_x = tiles_x; t.tiles_y = tiles_y; t.npts = npts;
-        return t;
-    }
+    int npts = 0, tiles_x = 0, tiles_y = 0;
 };
 
 // Who injects and who is recorded: the forward run injects the sources
 // (scale c / (hx hy hz)) and gathers at the receivers; the adjoint run
 // injects at the receivers (scale c) and gathers at the sources.
 struct Geometry {
-    DevInj inj;
+    DevInj inj[kNumShapes];   // filled by ensure_shape
+    // positions in the caller's order and their injection scales (set_model)
+    int *si = nullptr, *sj = nullptr, *sk = nullptr;
+    float *scale = nullptr;
+    int npos = 0;
+    InjTable view(int shape) const {
+        const DevInj &d = inj[shape];
+        InjTable t;
+        t.tile_start = d.tile_start; t.pt_i = d.pt_i; t.pt_j = d.pt_j; t.pt_k = d.pt_k; t.pt_off = d.pt_off;
+        t.pt_first = d.pt_first; t.src_row = d.src_row; t.src_scale = scale;
+        t.tiles_x = d.tiles_x; t.tiles_y = d.tiles_y; t.npts = d.npts;
+        return t;
+    }
     long long *gather_off = nullptr;
     int ngather = 0;
     double cell = 1.0;   // divisor of the injection scale
@@ -114,12 +117,16 @@ struct mmod_handle {
     long long ncounters = 0;
     int ckpt_scheme = MMOD_SCHEME_SEGMENTS;   // MMOD_OPT_CKPT_SCHEME
     bool tma_ok = false;
-    mmod::VolMaps u_map[2];             // tensor maps of u[0], u[1]
-    CUtensorMap c_map;
+    // per tile shape in use (ensure_shape): tensor maps of u[0], u[1] and c, injection tables in fwd / adj
+    struct ShapeMaps {
+        bool ready = false;
+        mmod::VolMaps u[2], c;
+    } shapes[mmod::kNumShapes];
+    int auto_variant = mmod::kTmaDefaultVariant;
 
     // gradient work space (lazy, sized for the last checkpoint layout)
     struct GradWork {
-        int nslot = 0, nwork = 0, dtype = -1;
+        int nslot = 0, nwork = 0, dtype = -1, shape = -1;
         std::vector<float *> seg;           // nwork padded FP32 work volumes
         std::vector<mmod::VolMaps> seg_map;
         float *psi[2] = {nullptr, nullptr};
@@ -166,7 +173,12 @@ void drop_graphs(mmod_handle *h);   // mmod_api.cu: captured loops must be re-ca
 inline bool is_cpml(const mmod_handle *h) { return h->cfg.boundary == MMOD_BOUNDARY_CPML; }
 CpmlArgs cpml_args(const mmod_handle *h);
 const TmaPlan &active_plan(const mmod_handle *h);
-StepArgs base_args(mmod_handle *h, const Geometry &geo, const float *wavelet);
+// Tile shape of the handle's next run (0 without TMA kernels), with its
+// tensor maps and injection tables built: allocates on first use, so it runs
+// before any capture.
+mmod_status ensure_shape(mmod_handle *h, int shape);
+int active_shape(const mmod_handle *h);
+StepArgs base_args(mmod_handle *h, const Geometry &geo, const float *wavelet, int shape);
 // Enqueues one step (plain path: step, injection, optional gather of
 // u^{n+1} into plain_gather_dst; TMA path: one kernel).
 cudaError_t enqueue_step(mmod_handle *h, const StepArgs &a, const VolMaps &cur, const VolMaps &prev, bool tma,

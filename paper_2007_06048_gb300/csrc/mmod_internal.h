@@ -13,11 +13,11 @@
 namespace mmod {
 
 // Point sources grouped by grid point and bucketed per (x-y tile, plane) of
-// the TMA kernel (64 x 16 tiles): the points of plane k in tile (tx, ty) are
+// the TMA kernel's tile shape: the points of plane k in tile (tx, ty) are
 // [tile_start[b], tile_start[b+1]), b = (ty * tiles_x + tx) * nz + k, so the
 // points of one tile over a z range [k0, k1) are one contiguous run.
 // Point p carries the sources [pt_first[p], pt_first[p+1]) in a fixed order.
-constexpr int kInjTileX = 64, kInjTileY = 16;
+constexpr int kInjTileX = 64, kInjTileY = 16;   // the tiles of shape 0 (batch and persistent kernels' gathers)
 
 struct InjTable {
     const int *tile_start;      // [tiles_y * tiles_x * nz + 1]
@@ -25,7 +25,7 @@ struct InjTable {
     const long long *pt_off;    // padded offset of the point
     const int *pt_first;        // [npts + 1]
     const int *src_row;         // wavelet row of each source (point order)
-    const float *src_scale;     // injection scale of each source
+    const float *src_scale;     // injection scale by wavelet row
     int tiles_x, tiles_y, npts;
 };
 
@@ -72,7 +72,7 @@ __device__ __forceinline__ void inject_point_at(const StepArgs &a, float *uout, 
     float *dst = uout + __ldg(a.inj.pt_off + p);
     float v = *dst;
     for (int s = __ldg(a.inj.pt_first + p); s < __ldg(a.inj.pt_first + p + 1); ++s)
-        v = add_source(v, __ldg(a.inj.src_scale + s),
+        v = add_source(v, __ldg(a.inj.src_scale + __ldg(a.inj.src_row + s)),
                        __ldg(a.wavelet + (long long)__ldg(a.inj.src_row + s) * a.wrs + (long long)n * a.wcs), r);
     *dst = v;
 }
@@ -110,8 +110,9 @@ __device__ __forceinline__ void inject_points(const StepArgs &a, float *uout, in
 #pragma unroll
         for (int q = 0; q < G; ++q) {
             v[q] = uout[off[q]];
-            sc[q] = __ldg(a.inj.src_scale + s0[q]);
-            w[q] = __ldg(a.wavelet + (long long)__ldg(a.inj.src_row + s0[q]) * a.wrs + (long long)n * a.wcs);
+            const int row = __ldg(a.inj.src_row + s0[q]);
+            sc[q] = __ldg(a.inj.src_scale + row);
+            w[q] = __ldg(a.wavelet + (long long)row * a.wrs + (long long)n * a.wcs);
         }
 #pragma unroll
         for (int q = 0; q < G; ++q) {
@@ -119,7 +120,7 @@ __device__ __forceinline__ void inject_points(const StepArgs &a, float *uout, in
             const float r = damp_factor(e[q]);
             float x = add_source(v[q], sc[q], w[q], r);   // every point has at least one source
             for (int s = s0[q] + 1; s < s1[q]; ++s)
-                x = add_source(x, __ldg(a.inj.src_scale + s),
+                x = add_source(x, __ldg(a.inj.src_scale + __ldg(a.inj.src_row + s)),
                                __ldg(a.wavelet + (long long)__ldg(a.inj.src_row + s) * a.wrs + (long long)n * a.wcs),
                                r);
             uout[off[q]] = x;

@@ -231,9 +231,9 @@ extern "C" __attribute__((visibility("default"))) mmod_status mmod_forward_noall
         const int sidx = order[q];
         const int *p = c.src_ijk + 3 * sidx;
         src_row[q] = sidx;
-        src_i[q] = p[0];
-        src_j[q] = p[1];
-        src_k[q] = p[2];
+        src_i[sidx] = p[0];   // scales are kept by wavelet row
+        src_j[sidx] = p[1];
+        src_k[sidx] = p[2];
         const bool same = q > 0 && std::memcmp(c.src_ijk + 3 * order[q - 1], p, 3 * sizeof(int)) == 0;
         if (!same) {
             pt_i[npt] = p[0];
@@ -293,7 +293,7 @@ extern "C" __attribute__((visibility("default"))) mmod_status mmod_forward_noall
     CKS(launch_model_fill(vel, c.nx, c.ny, c.nz, nxp, c.dt, cvol, s));
     {
         int *tab_src_i = tab_d + 4 * kMaxSrc + 1 + kMaxSrc;
-        CKS(launch_source_scale(vel, c.nx, c.ny, nkeep, tab_src_i, tab_src_i + kMaxSrc, tab_src_i + 2 * kMaxSrc,
+        CKS(launch_source_scale(vel, c.nx, c.ny, c.nsrc, tab_src_i, tab_src_i + kMaxSrc, tab_src_i + 2 * kMaxSrc,
                                 c.dt, c.hx * c.hy * c.hz, src_scale, s));
     }
     float eta_h[3 * kMaxAxis];
@@ -306,10 +306,10 @@ extern "C" __attribute__((visibility("default"))) mmod_status mmod_forward_noall
     // ---- time loop: u^{-1} = u^0 = 0, one step kernel per step
     CKS(cudaMemsetAsync(u[0], 0, sizeof(float) * vol, s));
     CKS(cudaMemsetAsync(u[1], 0, sizeof(float) * vol, s));
-    VolMaps u_map[2];
-    CUtensorMap c_map;
+    VolMaps u_map[2], c_map;
     TmaPlan plans[kMaxTmaVariants];
-    const bool tma = make_tma_plan(c, nxp, u, cvol, u_map, &c_map, plans);
+    bool tma = make_tma_plan(c, plans) && encode_maps(c, nxp, cvol, 0, &c_map);
+    for (int b = 0; b < 2; ++b) tma = tma && encode_maps(c, nxp, u[b], 0, &u_map[b]);
     StepArgs a{};
     a.nx = c.nx; a.ny = c.ny; a.nz = c.nz; a.nxp = nxp; a.plane = plane; a.nbl = c.nbl; a.nt = c.nt;
     for (int m = 0; m < kRadius; ++m) {
@@ -339,7 +339,7 @@ extern "C" __attribute__((visibility("default"))) mmod_status mmod_forward_noall
         a.uout = u[n & 1];
         if (tma) {
             a.traces = (n >= 1 && want_tr) ? traces + (long long)(n - 1) * c.nrec : nullptr;
-            CKS(launch_step_tma(a, u_map[(n + 1) & 1], u_map[n & 1], c_map, plans[kTmaDefaultVariant], s));
+            CKS(launch_step_tma(a, u_map[(n + 1) & 1], u_map[n & 1], c_map.own, plans[kTmaDefaultVariant], s));
         } else {
             a.traces = nullptr;
             CKS(launch_step_simple(a, s));

@@ -458,7 +458,7 @@ __device__ __forceinline__ void step_tma_body(const StepArgs &a, const StepVar &
     // per injection point.
     __syncthreads();
     if (!*c.abort_flag && a.inj.npts > 0) {
-        const long long b = ((long long)(c.y0 / kInjTileY) * a.inj.tiles_x + c.x0 / kInjTileX) * a.nz + c.z0;
+        const long long b = ((long long)ty * a.inj.tiles_x + tx) * a.nz + c.z0;
         const int lo = __ldg(a.inj.tile_start + b), hi = __ldg(a.inj.tile_start + b + T);
         inject_points(a, v.uout, v.n, lo, hi, tid, S::NT);
         if constexpr (G) inject_g_points(a, v.n, lo, hi, tid, S::NT);
@@ -746,19 +746,20 @@ bool encode(CUtensorMap *map, const float *base, const mmod_config &cfg, int nxp
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Compiled variants.  All use tile height 16 (the tensor maps' box).
+// Compiled variants.  0 .. 8 use 64 x 16 tiles (shape 0).
 constexpr int kTY = 16;
-static_assert(kTY == kInjTileY && TX == kInjTileX, "injection buckets must match the kernel's tiles");
+template <int SH>
+using StagedShape = Staged<kTmaShapes[SH].tx, kTmaShapes[SH].ty, kTmaShapes[SH].pitch>;
 using V22_1 = Shape<kTY, 2, 1>;
 using V22_2 = Shape<kTY, 2, 2>;
-using V22_4 = Staged<TX, kTY, HX>;
+using V22_4 = StagedShape<0>;
+static_assert(V22_4::TX == TX && V22_4::TY == kTY && V22_4::PITCH == HX, "shape 0 is the ring form's tile");
 using V24_1 = Shape<kTY, 4, 1>;
 using V24_2 = Shape<kTY, 4, 2>;
 using V24_2s = Shape<kTY, 4, 2, 6, 2>;
 using V22_4s = Shape<kTY, 2, 4, 6, 2>;
 using V22_4s3 = Shape<kTY, 2, 4, 6, 2, 3>;
 using V22_2s3 = Shape<kTY, 2, 2, 6, 2, 3>;
-static_assert(kTmaGVariant == 2, "the g^n forms are compiled for V22_4, variant 2");
 
 struct Variant {
     const char *name;
@@ -767,17 +768,25 @@ struct Variant {
     const void *persist_fn;   // null: no persistent form compiled
     const void *claim_fn;     // null: no work-claiming form compiled
     int nt, smem, batch_smem;
+    int shape;                // tile shape
+    const void *g_fn;         // null: no form that also writes g^n
+    const void *claim_g_fn;
 };
 
 #define MMOD_VARIANT(V, desc, P, C) \
     {desc, (const void *)step_tma_kernel<V>, (const void *)step_tma_batch_kernel<V>, P, C, V::NT, V::SMEM, \
-     batch_smem<V>()}
+     batch_smem<V>(), 0, nullptr, nullptr}
+#define MMOD_STAGED_VARIANT(SH, desc)                                                                              \
+    {desc, (const void *)step_tma_kernel<StagedShape<SH>>, nullptr, nullptr, nullptr, StagedShape<SH>::NT,         \
+     StagedShape<SH>::SMEM, 0, SH, (const void *)step_tma_kernel<StagedShape<SH>, true>, nullptr}
 const Variant kVariants[] = {
     MMOD_VARIANT(V22_1, "64x16 tile, 2x2 points/thread, z unroll 1", nullptr, nullptr),
     MMOD_VARIANT(V22_2, "64x16 tile, 2x2 points/thread, z unroll 2", nullptr,
                  (const void *)step_tma_claim_kernel<V22_2>),
-    MMOD_VARIANT(V22_4, "64x16 tile, 2x2 points/thread, z unroll 4",
-                 (const void *)step_tma_persistent_kernel<V22_4>, (const void *)step_tma_claim_kernel<V22_4>),
+    {"64x16 tile, 2x2 points/thread, z unroll 4", (const void *)step_tma_kernel<V22_4>,
+     (const void *)step_tma_batch_kernel<V22_4>, (const void *)step_tma_persistent_kernel<V22_4>,
+     (const void *)step_tma_claim_kernel<V22_4>, V22_4::NT, V22_4::SMEM, batch_smem<V22_4>(), 0,
+     (const void *)step_tma_kernel<V22_4, true>, (const void *)step_tma_claim_kernel<V22_4, true>},
     MMOD_VARIANT(V24_1, "64x16 tile, 2x4 points/thread, z unroll 1", nullptr, nullptr),
     MMOD_VARIANT(V24_2, "64x16 tile, 2x4 points/thread, z unroll 2", nullptr, nullptr),
     MMOD_VARIANT(V24_2s, "64x16 tile, 2x4 points/thread, z unroll 2, shallow rings",
@@ -786,9 +795,14 @@ const Variant kVariants[] = {
                  (const void *)step_tma_claim_kernel<V22_4s>),
     MMOD_VARIANT(V22_4s3, "64x16 tile, 2x2 points/thread, z unroll 4, shallow rings, 3 CTAs/SM", nullptr, nullptr),
     MMOD_VARIANT(V22_2s3, "64x16 tile, 2x2 points/thread, z unroll 2, shallow rings, 3 CTAs/SM", nullptr, nullptr),
+    MMOD_STAGED_VARIANT(1, "48x20 tile, 2x2 points/thread, z unroll 4"),
+    MMOD_STAGED_VARIANT(2, "40x24 tile, 2x2 points/thread, z unroll 4"),
+    MMOD_STAGED_VARIANT(3, "32x32 tile, 2x2 points/thread, z unroll 4"),
 };
 #undef MMOD_VARIANT
+#undef MMOD_STAGED_VARIANT
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
+static_assert(kNumVariants <= kMaxTmaVariants, "room for the plans");
 
 }  // namespace
 
@@ -804,40 +818,33 @@ bool encode_box(CUtensorMap *map, const float *base, int nx, int ny, int nz, int
     return encode(map, base, c, nxp, bx, by);
 }
 
-bool encode_maps(const mmod_config &cfg, int nxp, const float *buf, VolMaps *m) {
-    return encode(&m->halo, buf, cfg, nxp, HX, kTY + 2 * kRadius) && encode(&m->own, buf, cfg, nxp, TX, kTY);
+bool encode_maps(const mmod_config &cfg, int nxp, const float *buf, int shape, VolMaps *m) {
+    const TmaShape &t = kTmaShapes[shape];
+    return encode(&m->halo, buf, cfg, nxp, t.pitch, t.ty + 2 * kRadius) && encode(&m->own, buf, cfg, nxp, t.tx, t.ty);
 }
 
-bool make_tma_plan(const mmod_config &cfg, int nxp, float *const u[2], const float *c, VolMaps u_map[2],
-                   CUtensorMap *c_map, TmaPlan plans[]) {
-    for (int b = 0; b < 2; ++b)
-        if (!encode_maps(cfg, nxp, u[b], &u_map[b])) return false;
-    if (!encode(c_map, c, cfg, nxp, TX, kTY)) return false;
+namespace {
+// Dynamic shared memory of a kernel (null: none compiled).
+bool set_smem(const void *fn, int bytes) {
+    return !fn || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+}
+}  // namespace
+
+bool make_tma_plan(const mmod_config &cfg, TmaPlan plans[]) {
+    if (!encoder()) return false;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int tiles_x = (cfg.nx + TX - 1) / TX, tiles_y = (cfg.ny + kTY - 1) / kTY;
-    const long long tiles = (long long)tiles_x * tiles_y;
     for (int v = 0; v < kNumVariants; ++v) {
         const Variant &var = kVariants[v];
+        const int tiles_x = (cfg.nx + kTmaShapes[var.shape].tx - 1) / kTmaShapes[var.shape].tx;
+        const int tiles_y = (cfg.ny + kTmaShapes[var.shape].ty - 1) / kTmaShapes[var.shape].ty;
+        const long long tiles = (long long)tiles_x * tiles_y;
         int occ = 0;
-        if (cudaFuncSetAttribute(var.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, var.smem) != cudaSuccess ||
-            cudaFuncSetAttribute(var.batch_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, var.batch_smem) != cudaSuccess ||
-            (var.claim_fn &&
-             cudaFuncSetAttribute(var.claim_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, var.smem) !=
-                 cudaSuccess) ||
-            (var.persist_fn &&
-             cudaFuncSetAttribute(var.persist_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, var.smem) !=
-                 cudaSuccess) ||
+        if (!set_smem(var.fn, var.smem) || !set_smem(var.batch_fn, var.batch_smem) ||
+            !set_smem(var.claim_fn, var.smem) || !set_smem(var.persist_fn, var.smem) ||
+            !set_smem(var.g_fn, var.smem) || !set_smem(var.claim_g_fn, var.smem) ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, var.fn, var.nt, var.smem) != cudaSuccess || occ < 1) {
-            cudaGetLastError();
-            return false;
-        }
-        if (v == kTmaGVariant &&
-            (cudaFuncSetAttribute((const void *)step_tma_kernel<V22_4, true>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, var.smem) != cudaSuccess ||
-             cudaFuncSetAttribute((const void *)step_tma_claim_kernel<V22_4, true>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, var.smem) != cudaSuccess)) {
             cudaGetLastError();
             return false;
         }
@@ -859,6 +866,8 @@ bool make_tma_plan(const mmod_config &cfg, int nxp, float *const u[2], const flo
         }
         TmaPlan &p = plans[v];
         p.variant = v;
+        p.shape = var.shape;
+        p.has_g = var.g_fn != nullptr;
         p.tiles_x = tiles_x;
         p.tiles_y = tiles_y;
         p.zchunks = best_c;
@@ -872,6 +881,41 @@ bool make_tma_plan(const mmod_config &cfg, int nxp, float *const u[2], const flo
     }
     return true;
 }
+
+// Why several tile shapes: on grids of up to a few waves a launch takes
+// about 0.82 us per plane of a CTA, whatever its tile's fill, so the number
+// of planes, ceil(nz / (slots / tiles)), decides, and 64 x 16 tiles waste up
+// to a third of it (200^3: 4 x 13 tiles of 40 planes against 5 x 9 tiles of 40 x
+// 24 with 34 planes).  The cost below was fitted to 4 shapes x 28 grids from
+// 64^3 to 400^3 and 77 x 210 x 64 (3 % residual): per wave 1.2 us and 0.60 us
+// per plane of 256 threads, and 0.033 us per MB moved into shared memory.
+// Measured there, best shape against 64 x 16 (us per step): 96^3 5.12 / 5.95
+// (32 x 32), 144^3 11.1 / 13.1 (48 x 20), 200^3 27.2 / 32.3 (40 x 24), 240^3 39.7 /
+// 41.5 (48 x 20), 160 x 120 x 100 7.8 / 9.6 (40 x 24), 77 x 210 x 64 6.2 / 8.2 (40 x
+// 24).  64 x 16 stays where the model sees less than 1.5 % (128^3, 192^3, 256^3,
+// 320^3, 512^3).
+int auto_tma_variant(const TmaPlan plans[]) {
+    auto cost = [&](const TmaPlan &p) {
+        const TmaShape &t = kTmaShapes[p.shape];
+        const double waves = (double)((p.grid + (long long)p.slots - 1) / p.slots);
+        const double mb = 4e-6 * p.grid * (t.pitch * (t.ty + 2.0 * kRadius) * (p.zlen + 4.0) +
+                                           t.tx * t.ty * (2.0 * p.zlen + 4.0));
+        return waves * (1.2 + 0.60 * p.zlen * p.block / 256.0) + 0.033 * mb;
+    };
+    int best = kTmaDefaultVariant;
+    double least = 0.985 * cost(plans[best]);
+    for (int v = 0; v < kNumVariants; ++v) {
+        if (plans[v].shape == 0) continue;
+        const double c = cost(plans[v]);
+        if (c < least) {
+            least = c;
+            best = v;
+        }
+    }
+    return best;
+}
+
+bool tma_variant_has_batch(int v) { return v >= 0 && v < kNumVariants && kVariants[v].batch_fn; }
 
 bool claim_geom(const TmaPlan &plan, int nz, Geom *g, int *units, int *grid) {
     if (plan.claim <= 0 || plan.variant < 0 || plan.variant >= kNumVariants || !kVariants[plan.variant].claim_fn ||
@@ -891,50 +935,12 @@ cudaError_t launch_step_tma(const StepArgs &a, const VolMaps &cur, const VolMaps
     const StepMaps maps{cur.halo, cur.own, prev.own, c_map};
     Geom cg;
     int units = 0, cgrid = 0;
-    const bool claim = a.claim && claim_geom(plan, a.nz, &cg, &units, &cgrid);
-    if (a.gout) {   // g^n as well: variant 2 only (the caller passes its plan)
-        if (plan.variant != kTmaGVariant) return cudaErrorInvalidValue;
-        cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3(claim ? cgrid : plan.grid);
-        lc.blockDim = dim3(plan.block);
-        lc.dynamicSmemBytes = plan.smem;
-        lc.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        lc.attrs = attr;
-        lc.numAttrs = a.pdl ? 1 : 0;
-        const Geom g{plan.tiles_x, plan.tiles_y, plan.zchunks, plan.zlen};
-        const cudaError_t e =
-            claim ? cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_4, true>, a, maps, cg, units)
-                  : cudaLaunchKernelEx(&lc, step_tma_kernel<V22_4, true>, a, maps, g);
-        if (e != cudaSuccess) return e;
-        return cudaGetLastError();
-    }
-    if (claim) {
-        cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3(cgrid);
-        lc.blockDim = dim3(plan.block);
-        lc.dynamicSmemBytes = plan.smem;
-        lc.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        lc.attrs = attr;
-        lc.numAttrs = a.pdl ? 1 : 0;
-        cudaError_t e;
-        switch (plan.variant) {
-            case 1: e = cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_2>, a, maps, cg, units); break;
-            case 2: e = cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_4>, a, maps, cg, units); break;
-            case 6: e = cudaLaunchKernelEx(&lc, step_tma_claim_kernel<V22_4s>, a, maps, cg, units); break;
-            default: return cudaErrorInvalidValue;
-        }
-        if (e != cudaSuccess) return e;
-        return cudaGetLastError();
-    }
-    const Geom g{plan.tiles_x, plan.tiles_y, plan.zchunks, plan.zlen};
+    const bool claim = a.claim && claim_geom(plan, a.nz, &cg, &units, &cgrid) &&
+                       (!a.gout || kVariants[plan.variant].claim_g_fn);
+    if (a.gout && !plan.has_g) return cudaErrorInvalidValue;
+    const Geom g = claim ? cg : Geom{plan.tiles_x, plan.tiles_y, plan.zchunks, plan.zlen};
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(plan.grid);
+    lc.gridDim = dim3(claim ? cgrid : plan.grid);
     lc.blockDim = dim3(plan.block);
     lc.dynamicSmemBytes = plan.smem;
     lc.stream = s;
@@ -943,21 +949,15 @@ cudaError_t launch_step_tma(const StepArgs &a, const VolMaps &cur, const VolMaps
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = a.pdl ? 1 : 0;
-#define MMOD_LAUNCH(V) cudaLaunchKernelEx(&lc, step_tma_kernel<V>, a, maps, g)
-    switch (plan.variant) {
-        case 0: MMOD_LAUNCH(V22_1); break;
-        case 1: MMOD_LAUNCH(V22_2); break;
-        case 2: MMOD_LAUNCH(V22_4); break;
-        case 3: MMOD_LAUNCH(V24_1); break;
-        case 4: MMOD_LAUNCH(V24_2); break;
-        case 5: MMOD_LAUNCH(V24_2s); break;
-        case 6: MMOD_LAUNCH(V22_4s); break;
-        case 7: MMOD_LAUNCH(V22_4s3); break;
-        case 8: MMOD_LAUNCH(V22_2s3); break;
-        default: return cudaErrorInvalidValue;
-    }
-#undef MMOD_LAUNCH
-    return cudaGetLastError();
+    if (plan.variant < 0 || plan.variant >= kNumVariants) return cudaErrorInvalidValue;
+    const Variant &var = kVariants[plan.variant];
+    StepArgs args = a;
+    StepMaps m = maps;
+    Geom geom = g;
+    void *params[4] = {&args, &m, &geom, &units};
+    const cudaError_t e = cudaLaunchKernelExC(
+        &lc, claim ? (a.gout ? var.claim_g_fn : var.claim_fn) : (a.gout ? var.g_fn : var.fn), params);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 Geom persistent_geom(const TmaPlan &plan, int nz) {
@@ -1080,7 +1080,7 @@ bool tma_variant_shape(int v, int *block, int *smem) {
 
 cudaError_t launch_step_tma_batch(int variant, const ShotDesc *shots, const int *cta_shot, const int *cta_local,
                                   int nctas, int n, bool pdl, cudaStream_t s) {
-    if (variant < 0 || variant >= kNumVariants) return cudaErrorInvalidValue;
+    if (!tma_variant_has_batch(variant)) return cudaErrorInvalidValue;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(nctas);
     lc.blockDim = dim3(kVariants[variant].nt);

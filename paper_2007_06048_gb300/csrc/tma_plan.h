@@ -7,14 +7,24 @@
 namespace mmod {
 
 constexpr int kMaxTmaVariants = 12;
-// Variant used unless a handle selects another: the fastest measured on the
-// 240^3 workload (64x16 tile, 2x2 points per thread, z unroll 4).
+// The 64 x 16 staged variant: what the batch, persistent and work-claiming
+// forms are compiled for, and what a handle runs when no other tile shape
+// serves its grid better (TmaShape).
 constexpr int kTmaDefaultVariant = 2;
-// The variant whose step kernels can also write g^n = L u^n + s^n (StepArgs::gout).
-constexpr int kTmaGVariant = 2;
+
+// Tile shapes of the compiled variants: TX x TY points, halo rows of `pitch`
+// floats.  Injection tables are bucketed per tile, so a handle keeps tensor
+// maps and tables per shape it runs (ensure_shape).
+struct TmaShape {
+    int tx, ty, pitch;
+};
+constexpr int kNumShapes = 4;
+constexpr TmaShape kTmaShapes[kNumShapes] = {{64, 16, 72}, {48, 20, 56}, {40, 24, 52}, {32, 32, 40}};
 
 struct TmaPlan {
     int variant = 0;                // index into the compiled variants
+    int shape = 0;                  // index into kTmaShapes
+    bool has_g = false;             // compiled with the g^n output (StepArgs::gout)
     int tiles_x = 0, tiles_y = 0;   // x-y tiles covering the plane
     int zchunks = 0;                // z-ranges per tile column
     int zlen = 0;                   // planes per z-range (last one may be shorter)
@@ -34,17 +44,19 @@ bool claim_geom(const TmaPlan &plan, int nz, Geom *g, int *units, int *grid);
 int tma_variant_count();
 const char *tma_variant_name(int v);
 
-// Encodes the tensor maps of both wavefield buffers and of the coefficient
-// volume and fills one plan per compiled variant.  Returns false when the TMA
-// kernel cannot serve the grid (the caller then uses the plain kernel).
-// Tensor maps of one padded volume buffer: the halo box (u^n) and the tile
-// box (u^{n-1}, and the planes of u^n that need no halo).
+// Tensor maps of one padded volume buffer for a tile shape: the halo box
+// (u^n) and the tile box (u^{n-1}, c, and the planes of u^n without halo).
 struct VolMaps {
     CUtensorMap halo, own;
 };
-bool encode_maps(const mmod_config &cfg, int nxp, const float *buf, VolMaps *m);
+bool encode_maps(const mmod_config &cfg, int nxp, const float *buf, int shape, VolMaps *m);
 
-bool make_tma_plan(const mmod_config &cfg, int nxp, float *const u[2], const float *c, VolMaps u_map[2],
-                   CUtensorMap *c_map, TmaPlan plans[]);
+// Fills one plan per compiled variant.  False when the TMA kernels cannot
+// run (the caller then uses the plain kernel).
+bool make_tma_plan(const mmod_config &cfg, TmaPlan plans[]);
+// The variant a handle runs by default: the tile shape and z split of least
+// cost for its grid (rule beside the definition).
+int auto_tma_variant(const TmaPlan plans[]);
+bool tma_variant_has_batch(int v);
 
 }  // namespace mmod
