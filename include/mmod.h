@@ -180,6 +180,13 @@ enum { MMOD_CKPT_FP32 = 0, MMOD_CKPT_BF16 = 1, MMOD_CKPT_FP16 = 2, MMOD_CKPT_BFP
 mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const float *resid, float *grad_v,
                           int ckpt_count, int ckpt_dtype, mmod_stream stream);
 
+/* mmod_gradient and mmod_adjoint of the same residual in one call: writes
+ * grad_v as mmod_gradient and adj_src [nsrc][nt] as mmod_adjoint (the same
+ * bits), recording the gradient's own adjoint sweep at the sources.  adj_src
+ * may be NULL when nsrc == 0.  Errors: STATE, ARG, OOM, CUDA, TIMEOUT. */
+mmod_status mmod_gradient_adjoint(mmod_handle *h, const float *wavelet, const float *resid, float *grad_v,
+                                  float *adj_src, int ckpt_count, int ckpt_dtype, mmod_stream stream);
+
 /* Bytes of device memory mmod_gradient allocates for this checkpoint layout
  * under the handle's current scheme (on top of the handle's own volumes);
  * -1 for invalid arguments. */

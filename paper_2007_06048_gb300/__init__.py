@@ -46,7 +46,7 @@ EXPORTED = ["mmod_create", "mmod_destroy", "mmod_set_model", "mmod_forward", "mm
             "mmod_cfl_dt", "mmod_last_error", "mmod_version", "mmod_check_recip",
             "mmod_tma_variant_count", "mmod_tma_variant_name", "mmod_set_tma_variant", "mmod_get_plan",
             "mmod_forward_noalloc", "mmod_set_option", "mmod_adjoint", "mmod_gradient",
-            "mmod_gradient_memory", "mmod_dot", "mmod_batch_create", "mmod_batch_destroy",
+            "mmod_gradient_adjoint", "mmod_gradient_memory", "mmod_dot", "mmod_batch_create", "mmod_batch_destroy",
             "mmod_batch_forward", "mmod_batch_set_variant", "mmod_batch_last_loop_ms", "mmod_batch_last_error",
             "mmod_autotune", "mmod_batch_autotune", "mmod_revolve_schedule", "mmod_persistent_grid",
             "mmod_tma_variant_info", "mmod_batch_set_mode", "mmod_optimized_coefficients",
@@ -111,6 +111,7 @@ def load():
         "mmod_set_option": ([P, I, I], I),
         "mmod_adjoint": ([P, P, P, P], I),
         "mmod_gradient": ([P, P, P, P, I, I, P], I),
+        "mmod_gradient_adjoint": ([P, P, P, P, P, I, I, P], I),
         "mmod_gradient_memory": ([P, I, I], ctypes.c_longlong),
         "mmod_dot": ([P, P, ctypes.c_longlong, ctypes.POINTER(ctypes.c_double), P], I),
         "mmod_batch_create": ([ctypes.POINTER(P), I, ctypes.POINTER(P)], I),
@@ -277,6 +278,12 @@ def mmod_adjoint(h, resid, adj_src, stream=None):
 def mmod_gradient(h, wavelet, resid, grad_v, ckpt_count, ckpt_dtype=0, stream=None):
     _check(h, load().mmod_gradient(h, _addr(wavelet), _addr(resid), _addr(grad_v), int(ckpt_count),
                                    int(ckpt_dtype), _stream(stream)))
+
+
+def mmod_gradient_adjoint(h, wavelet, resid, grad_v, adj_src, ckpt_count, ckpt_dtype=0, stream=None):
+    """mmod_gradient and mmod_adjoint of one residual in one adjoint sweep."""
+    _check(h, load().mmod_gradient_adjoint(h, _addr(wavelet), _addr(resid), _addr(grad_v), _addr(adj_src),
+                                           int(ckpt_count), int(ckpt_dtype), _stream(stream)))
 
 
 def mmod_gradient_memory(h, ckpt_count, ckpt_dtype=0) -> int:
@@ -461,6 +468,9 @@ class Propagator:
 
     def gradient(self, wavelet, resid, grad_v, ckpt_count, ckpt_dtype=0, stream=None):
         mmod_gradient(self.handle, wavelet, resid, grad_v, ckpt_count, ckpt_dtype, stream)
+
+    def gradient_adjoint(self, wavelet, resid, grad_v, adj_src, ckpt_count, ckpt_dtype=0, stream=None):
+        mmod_gradient_adjoint(self.handle, wavelet, resid, grad_v, adj_src, ckpt_count, ckpt_dtype, stream)
 
     def gradient_memory(self, ckpt_count, ckpt_dtype=0) -> int:
         return mmod_gradient_memory(self.handle, ckpt_count, ckpt_dtype)

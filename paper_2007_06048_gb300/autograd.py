@@ -3,7 +3,8 @@
 The backward pass is the library's own transpose: for an upstream gradient g
 of the traces, the velocity gradient is mmod_gradient with g as the residual
 (the zero-lag imaging condition of the adjoint wavefield, forward states
-recomputed from checkpoints), and the wavelet gradient is mmod_adjoint(g).
+recomputed from checkpoints), and the wavelet gradient is mmod_adjoint(g);
+when both are wanted, mmod_gradient_adjoint gives them from one adjoint sweep.
 Argument marshalling only: every step runs in libmmod.so.
 """
 from __future__ import annotations
@@ -35,9 +36,13 @@ class _ForwardMap(torch.autograd.Function):
         if ctx.needs_input_grad[0]:
             prop.set_model(vel)   # the handle may have seen another model since
             grad_vel = torch.empty_like(vel)
-            prop.gradient(wavelet, g, grad_vel, *ctx.ckpt)
         if ctx.needs_input_grad[1]:
             grad_wav = torch.empty_like(wavelet)
+        if grad_vel is not None and grad_wav is not None:   # one adjoint sweep for both
+            prop.gradient_adjoint(wavelet, g, grad_vel, grad_wav, *ctx.ckpt)
+        elif grad_vel is not None:
+            prop.gradient(wavelet, g, grad_vel, *ctx.ckpt)
+        elif grad_wav is not None:
             prop.adjoint(g, grad_wav)
         return grad_vel, grad_wav, None, None, None
 

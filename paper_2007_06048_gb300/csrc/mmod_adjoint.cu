@@ -352,6 +352,24 @@ mmod_status device_input(mmod_handle *h, const float *p, size_t n, float **stage
     return MMOD_OK;
 }
 
+// The adjoint sweep's gathers [nt][nsrc] (st_adjg) -> adj_src [nsrc][nt] in time order, host or device.
+mmod_status adjoint_output(mmod_handle *h, float *adj_src, cudaStream_t s) {
+    const auto &c = h->cfg;
+    const size_t nadj = (size_t)c.nt * c.nsrc;
+    const bool dev_out = is_device_ptr(adj_src);
+    float *dst = adj_src;
+    if (!dev_out) {
+        if (!h->st_adjo) MMOD_CK(h, cudaMalloc(&h->st_adjo, sizeof(float) * nadj));
+        dst = h->st_adjo;
+    }
+    MMOD_CK(h, launch_unreverse_transpose(h->st_adjg, c.nt, c.nsrc, 1.0 / (c.hx * c.hy * c.hz), dst, s));
+    if (!dev_out) {
+        MMOD_CK(h, cudaMemcpyAsync(adj_src, dst, sizeof(float) * nadj, cudaMemcpyDeviceToHost, s));
+        MMOD_CK(h, cudaStreamSynchronize(s));
+    }
+    return MMOD_OK;
+}
+
 }  // namespace
 
 namespace mmod {
@@ -405,25 +423,18 @@ MMOD_API mmod_status mmod_adjoint(mmod_handle *h, const float *resid, float *adj
             return st;
     h->ran = false;   // the wavefield buffers now hold the adjoint state
     if (nadj) {
-        const bool dev_out = is_device_ptr(adj_src);
-        float *dst = adj_src;
-        if (!dev_out) {
-            if (!h->st_adjo) MMOD_CK(h, cudaMalloc(&h->st_adjo, sizeof(float) * nadj));
-            dst = h->st_adjo;
-        }
-        MMOD_CK(h, launch_unreverse_transpose(h->st_adjg, c.nt, c.nsrc, 1.0 / (c.hx * c.hy * c.hz), dst, s));
+        if (mmod_status st = adjoint_output(h, adj_src, s)) return st;
         ++launches;
-        if (!dev_out) {
-            MMOD_CK(h, cudaMemcpyAsync(adj_src, dst, sizeof(float) * nadj, cudaMemcpyDeviceToHost, s));
-            MMOD_CK(h, cudaStreamSynchronize(s));
-        }
     }
     h->last_launches = launches;
     return check_latched(h);
 }
 
-MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const float *resid, float *grad_v,
-                                   int ckpt_count, int ckpt_dtype, mmod_stream stream) {
+// The velocity gradient and, with adj_src, the adjoint sources of the same
+// residual: the gradient's adjoint sweep is mmod_adjoint's, so recording it at
+// the sources saves the second sweep.
+static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const float *resid, float *grad_v,
+                                float *adj_src, int ckpt_count, int ckpt_dtype, mmod_stream stream) {
     if (!h) return MMOD_ERR_ARG;
     if (mmod_status st = check_latched(h)) return st;
     if (is_cpml(h)) return fail(h, MMOD_ERR_UNSUPPORTED, "the gradient is built for the damping layers only");
@@ -464,7 +475,9 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
     fa.nrec = 0;   // no receivers in the gradient's forward sweeps
     fa.inv_cell = (float)(1.0 / (c.hx * c.hy * c.hz));
     StepArgs aa = base_args(h, h->adj, h->st_adjw, shape);
-    aa.nrec = 0;
+    const int nadj = adj_src ? c.nsrc : 0;   // adjoint sources recorded per step
+    aa.nrec = nadj;
+    if (nadj && !h->st_adjg) MMOD_CK(h, cudaMalloc(&h->st_adjg, sizeof(float) * std::max<size_t>((size_t)nt * nadj, 1)));
     // forward step n in place on the handle's buffers: u^{n-1} in u[n & 1],
     // u^n in u[(n + 1) & 1], u^{n+1} over u^{n-1}
     auto fwd_step_in_place = [&](int n) {
@@ -495,7 +508,10 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
         aa.ucur = gw.psi[(m + 1) & 1];
         aa.uprev = gw.psi[m & 1];
         aa.uout = gw.psi[m & 1];
-        return enqueue_step(h, aa, gw.psi_map[(m + 1) & 1], gw.psi_map[m & 1], tma, nullptr, s, &launches);
+        // the step kernel records the field it reads (adjoint step m - 1); the plain path the one it writes
+        aa.traces = nadj && m >= 1 ? h->st_adjg + (size_t)(m - 1) * nadj : nullptr;
+        return enqueue_step(h, aa, gw.psi_map[(m + 1) & 1], gw.psi_map[m & 1], tma,
+                            nadj ? h->st_adjg + (size_t)m * nadj : nullptr, s, &launches);
     };
     // imaging terms of forward steps n (and n - 1 when ns = 2) from g[t] =
     // g^{n-t}, after their adjoint steps: psi^{n+1} in psi[(nt-1-n) & 1],
@@ -632,8 +648,28 @@ MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const f
         MMOD_CK(h, cudaMemcpyAsync(grad_v, dst, sizeof(float) * npts, cudaMemcpyDeviceToHost, s));
         MMOD_CK(h, cudaStreamSynchronize(s));
     }
+    if (nadj && nt > 0) {
+        if (tma) {   // the last adjoint step had no successor
+            MMOD_CK(h, launch_gather(gw.psi[(nt - 1) & 1], h->adj.gather_off, nadj, h->st_adjg + (size_t)(nt - 1) * nadj, s));
+            ++launches;
+        }
+        if (mmod_status st = adjoint_output(h, adj_src, s)) return st;
+        ++launches;
+    }
     h->last_launches = launches;
     return check_latched(h);
+}
+
+MMOD_API mmod_status mmod_gradient(mmod_handle *h, const float *wavelet, const float *resid, float *grad_v,
+                                   int ckpt_count, int ckpt_dtype, mmod_stream stream) {
+    return run_gradient(h, wavelet, resid, grad_v, nullptr, ckpt_count, ckpt_dtype, stream);
+}
+
+MMOD_API mmod_status mmod_gradient_adjoint(mmod_handle *h, const float *wavelet, const float *resid, float *grad_v,
+                                           float *adj_src, int ckpt_count, int ckpt_dtype, mmod_stream stream) {
+    if (!h) return MMOD_ERR_ARG;
+    if (h->cfg.nsrc > 0 && h->cfg.nt > 0 && !adj_src) return fail(h, MMOD_ERR_ARG, "null adjoint source with nsrc > 0");
+    return run_gradient(h, wavelet, resid, grad_v, adj_src, ckpt_count, ckpt_dtype, stream);
 }
 
 MMOD_API long long mmod_gradient_memory(const mmod_handle *h, int ckpt_count, int ckpt_dtype) {
