@@ -24,7 +24,11 @@
 // Bound by DRAM on large grids and by the pipeline's latencies on one-wave
 // grids.  us per step, ring form -> staged: 64^3 4.47 -> 3.83, 128^3 8.68 ->
 // 7.89, 200^3 34.98 -> 32.35, 240^3 41.96 -> 41.20, 512^3 337.0 -> 325.5 (6.60
-// TB/s); 110 registers instead of 120.
+// TB/s); 110 registers instead of 120.  Then, with the tensor maps prefetched,
+// u^n requested ahead of the block barrier, and the source and receiver
+// look-ups taken off the critical path (they were dependent loads right after
+// the wait and at the end): 64^3 3.83 -> 3.58, 151 x 117 x 98 7.8 -> 7.4, 240^3 39.4
+// -> 38.8.
 // PITCH, the halo tile's row pitch, is chosen so that a half-warp whose lanes
 // span two row pairs reads 16 different bank pairs: 2 PITCH = TX (mod 32).
 #pragma once
@@ -169,6 +173,25 @@ __device__ __forceinline__ void step_staged_body(const StepArgs &a, const StepVa
     auto load_halo = [&](int p, uint64_t *bar) {   // u^n at z0 + p
         tma_load_3d(ring + p % S::NSU * S::CUR_S, halo_map, x0 - kRadius, y0 - kRadius, z0 + p, bar);
     };
+    // The maps of u^n are first used on the critical path, right after the wait.
+    if (tid == 32) {
+        tma_prefetch_map(own_map);
+        tma_prefetch_map(halo_map);
+    }
+    // This tile's run of the injection table, for the end of the kernel.
+    int inj_lo = 0, inj_hi = 0;
+    if (a.inj.npts > 0) {
+        const long long bucket = ((long long)ty * a.inj.tiles_x + tx) * a.nz + z0;
+        inj_lo = __ldg(a.inj.tile_start + bucket);
+        inj_hi = __ldg(a.inj.tile_start + bucket + T);
+    }
+    // Receivers of the previous step (u^n, read-only during this launch), one
+    // per thread of the grid and more only where there are more: the offset is
+    // loaded here, the value once u^n is there, and it is stored after the plane
+    // loop, so the two dependent loads keep nobody waiting.
+    const int r0 = bid * S::NT + tid;
+    const bool rec0 = v.traces && r0 < a.nrec;
+    const long long rec_off0 = rec0 ? __ldg(a.rec_off + r0) : 0;
     if (tid == 0) {
         if (dep.reinit()) {   // the previous unit consumed every copy it issued
             for (int s = 0; s <= S::U; ++s) mbar_inval(&c.full[s]);
@@ -189,8 +212,10 @@ __device__ __forceinline__ void step_staged_body(const StepArgs &a, const StepVa
         }
     }
     dep.wait(tid, c.abort_flag, a.err);
-    __syncthreads();
-    const bool dep_ok = !*c.abort_flag;
+    // a wait that cannot fail and that every thread makes itself: u^n may be
+    // requested before the other warps are here
+    if constexpr (Dep::kProxyFence) __syncthreads();
+    const bool dep_ok = !Dep::kProxyFence || !*c.abort_flag;
     if (tid == 0 && dep_ok) {
         if constexpr (Dep::kProxyFence) fence_proxy_async_global();
         mbar_expect_tx(init, S::FIRST_BYTES);
@@ -209,10 +234,10 @@ __device__ __forceinline__ void step_staged_body(const StepArgs &a, const StepVa
         }
     }
     int armed = dep_ok ? min(S::U, T) : 0;   // planes whose stage has been filled
-    // receivers of the previous step (u^n, read-only during this launch)
+    if constexpr (!Dep::kProxyFence) __syncthreads();   // the barriers are set up
+    const float rec_val0 = rec0 ? v.ucur[rec_off0] : 0.0f;
     if (v.traces) {
-        for (int r = bid * S::NT + tid; r < a.nrec; r += nbid * S::NT)
-            v.traces[r] = v.ucur[__ldg(a.rec_off + r)];
+        for (int r = r0 + nbid * S::NT; r < a.nrec; r += nbid * S::NT) v.traces[r] = v.ucur[__ldg(a.rec_off + r)];
     }
 
     Wts w;
@@ -296,16 +321,15 @@ __device__ __forceinline__ void step_staged_body(const StepArgs &a, const StepVa
             for (int r = 0; r < S::RY; ++r) q[i][r] = q[i + S::U][r];
     }
 #undef MMOD_STAGED
+    if (rec0) v.traces[r0] = rec_val0;
     // Sources of this CTA's tile and planes: nothing in this launch reads the
     // u^{n+1} it writes, so they are added once the whole z range is stored
     // (the block barrier makes every thread's stores visible).  The points of
     // one tile over planes [z0, z0 + T) are one run of the table.
     __syncthreads();
-    if (!*c.abort_flag && a.inj.npts > 0) {
-        const long long bucket = ((long long)ty * a.inj.tiles_x + tx) * a.nz + z0;
-        const int lo = __ldg(a.inj.tile_start + bucket), hi = __ldg(a.inj.tile_start + bucket + T);
-        inject_points(a, v.uout, v.n, lo, hi, tid, S::NT);
-        if constexpr (G) inject_g_points(a, v.n, lo, hi, tid, S::NT);
+    if (!*c.abort_flag && inj_lo < inj_hi) {
+        inject_points(a, v.uout, v.n, inj_lo, inj_hi, tid, S::NT);
+        if constexpr (G) inject_g_points(a, v.n, inj_lo, inj_hi, tid, S::NT);
     }
     // After a give-up, wait (bounded) for the copies this CTA still has in
     // flight (the first planes and the latest phase of every stage) before its

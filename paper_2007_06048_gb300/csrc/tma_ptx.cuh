@@ -88,6 +88,12 @@ __device__ __noinline__ void mbar_drain(uint64_t *bar, uint32_t parity) {
         if (mbar_try_wait(bar, parity)) return;
 }
 
+// Fetches a tensor map into the descriptor cache (every launch has its own
+// copy in its parameters, so the first copy through a map misses).
+__device__ __forceinline__ void tma_prefetch_map(const CUtensorMap *map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
 __device__ __forceinline__ void tma_load_3d(float *dst, const CUtensorMap *map, int x, int y, int z,
                                             uint64_t *bar) {
     asm volatile(
