@@ -248,8 +248,9 @@ constexpr int VNSO = 3;    // own velocity slots
 constexpr int VNSB = 4;    // buoyancy slots (planes k and k + 1 resident)
 // slots start on 128-byte boundaries (the b box, 68 x 17 floats, is padded)
 constexpr int V_SLOT_P = PHX * PHY, V_SLOT_O = 3 * OWN, V_BOX_B = BX * BY, V_SLOT_B = (V_BOX_B + 31) / 32 * 32;
+static_assert(VNSB == VNSO + 1, "b of plane t + VNSO + 1 takes the slot of plane t");
 static_assert(V_SLOT_P % 32 == 0 && V_SLOT_O % 32 == 0, "128-byte slots");
-constexpr int V_SMEM = (VNSP * V_SLOT_P + VNSO * V_SLOT_O + VNSB * V_SLOT_B) * 4 + (VNSP + VNSO + VNSB) * 8 + 16;
+constexpr int V_SMEM = (VNSP * V_SLOT_P + VNSO * V_SLOT_O + VNSB * V_SLOT_B) * 4 + (VNSP + VNSO) * 8 + 16;
 
 constexpr int PNSC = 3;    // centre slots: vx (72 x 16), vy (64 x 24), p, dt K (64 x 16)
 constexpr int PNSZ = 8;    // vz own slots feeding the queue
@@ -403,7 +404,7 @@ __host__ __device__ constexpr int vq(int J, int i) { return kVU == 8 ? (J + i) %
 
 struct VCtx {
     float *ring_p, *ring_o, *ring_b;
-    uint64_t *bar_p, *bar_o, *bar_b;
+    uint64_t *bar_p, *bar_o;
     int *abort_flag;
     int x0, y0, z0, T, lane, warp, xl, x;
     float2 egx, ehx;       // eps at this thread's two columns (grid, half points)
@@ -428,9 +429,7 @@ __device__ __forceinline__ bool v_plane(const VdArgs &a, const VCtx &c, int t, f
         gz1 = t + 1 < c.T ? a.Gh[2][k + 1] : 0.0f;
     }
     if (!(mbar_wait(&c.bar_p[(t + 7) % VNSP], ((t + 7) / VNSP) & 1, c.abort_flag, a.err) &&
-          mbar_wait(&c.bar_o[t % VNSO], (t / VNSO) & 1, c.abort_flag, a.err) &&
-          mbar_wait(&c.bar_b[t % VNSB], (t / VNSB) & 1, c.abort_flag, a.err) &&
-          mbar_wait(&c.bar_b[(t + 1) % VNSB], ((t + 1) / VNSB) & 1, c.abort_flag, a.err)))
+          mbar_wait(&c.bar_o[t % VNSO], (t / VNSO) & 1, c.abort_flag, a.err)))
         return false;
     v_read_q(c, t + 7, q[vq(J, 7)]);
     const float *ctr = c.ring_p + ((t + 3) % VNSP) * V_SLOT_P;
@@ -515,16 +514,14 @@ __global__ void __launch_bounds__(NT, 2)
     c.ring_b = c.ring_o + VNSO * V_SLOT_O;
     c.bar_p = reinterpret_cast<uint64_t *>(c.ring_b + VNSB * V_SLOT_B);
     c.bar_o = c.bar_p + VNSP;
-    c.bar_b = c.bar_o + VNSO;
-    c.abort_flag = reinterpret_cast<int *>(c.bar_b + VNSB);
+    c.abort_flag = reinterpret_cast<int *>(c.bar_o + VNSO);
     const int tid = threadIdx.x;
     c.lane = tid & 31;
     c.warp = tid >> 5;
     tile_of(g, blockIdx.x, a.nz, c.x0, c.y0, c.z0, c.T);
     const int x0 = c.x0, y0 = c.y0, z0 = c.z0, T = c.T;
     const int nseq_p = T + 2 * kRadius - 1;   // p planes z0-3 .. z0+T+3
-    const int nseq_b = T + 1;                 // b planes z0 .. z0+T
-    int hi_p = 0, hi_o = 0, hi_b = 0;         // sequences issued per ring (elected thread only)
+    int hi_p = 0, hi_o = 0;                   // sequences issued per ring (elected thread only)
 
     auto issue_p = [&](int seq) {
         const int s = seq % VNSP;
@@ -534,40 +531,41 @@ __global__ void __launch_bounds__(NT, 2)
         tma_load_3d(c.ring_p + s * V_SLOT_P, &maps.p_halo, x0 - kRadius, y0 - kRadius, z, &c.bar_p[s]);
         hi_p = seq + 1;
     };
+    // own velocities of plane z0 + seq and, on the same barrier, b of the plane after it (the
+    // first also b of z0): what step seq needs besides p, so a plane costs two waits
     auto issue_o = [&](int seq) {
         const int s = seq % VNSO;
-        mbar_expect_tx(&c.bar_o[s], V_SLOT_O * 4);
+        mbar_expect_tx(&c.bar_o[s], (V_SLOT_O + (seq == 0 ? 2 : 1) * V_BOX_B) * 4);
 #pragma unroll
         for (int f = 0; f < 3; ++f)
             tma_load_3d(c.ring_o + s * V_SLOT_O + f * OWN, &maps.own[f], x0, y0, z0 + seq, &c.bar_o[s]);
+        for (int q = seq == 0 ? 0 : seq + 1; q <= seq + 1; ++q)
+            tma_load_3d(c.ring_b + q % VNSB * V_SLOT_B, &maps.b_box, x0, y0, z0 + q, &c.bar_o[s]);
         hi_o = seq + 1;
     };
-    auto issue_b = [&](int seq) {
-        const int s = seq % VNSB;
-        mbar_expect_tx(&c.bar_b[s], V_BOX_B * 4);
-        tma_load_3d(c.ring_b + s * V_SLOT_B, &maps.b_box, x0, y0, z0 + seq, &c.bar_b[s]);
-        hi_b = seq + 1;
-    };
 
+    if (tid == 32) tma_prefetch_map(&maps.p_halo);   // first used right after the wait
+    // Receivers of the previous step (p^n, read-only in this kernel), one per thread of the grid and
+    // more only where there are more: the offset is loaded here, the value after the wait, and it is
+    // stored after the plane loop, so the two dependent loads keep nobody waiting.
+    const int r0 = blockIdx.x * NT + tid;
+    const bool rec0 = a.traces && r0 < a.nrec;
+    const long long rec_off0 = rec0 ? a.rec_off[r0] : 0;
     if (tid == 0) {
         for (int s = 0; s < VNSP; ++s) mbar_init(&c.bar_p[s], 1);
         for (int s = 0; s < VNSO; ++s) mbar_init(&c.bar_o[s], 1);
-        for (int s = 0; s < VNSB; ++s) mbar_init(&c.bar_b[s], 1);
         *c.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         // own velocities (last written two launches back) and buoyancy first
-        if (T > 0) {
-            for (int q = 0; q < VNSO && q < T; ++q) issue_o(q);
-            for (int q = 0; q < VNSB && q < nseq_b; ++q) issue_b(q);
-        }
+        for (int q = 0; q < VNSO && q < T; ++q) issue_o(q);
     }
     pdl_wait();   // p^n of the pressure kernel and the source add
     if (tid == 0 && T > 0)
         for (int q = 0; q < VNSP && q < nseq_p; ++q) issue_p(q);
-    // receivers of the previous step: p^n, read-only in this kernel
+    const float rec_val0 = rec0 ? a.p[rec_off0] : 0.0f;
     if (a.traces)
-        for (int r = blockIdx.x * NT + tid; r < a.nrec; r += gridDim.x * NT) a.traces[r] = a.p[a.rec_off[r]];
+        for (int r = r0 + gridDim.x * NT; r < a.nrec; r += gridDim.x * NT) a.traces[r] = a.p[a.rec_off[r]];
     __syncthreads();
     if (T <= 0) return;
 
@@ -622,7 +620,6 @@ __global__ void __launch_bounds__(NT, 2)
         if (tid == 0) {                                                               \
             if (t + (J) + 3 + VNSP < nseq_p) issue_p(t + (J) + 3 + VNSP);             \
             if (t + (J) + VNSO < T) issue_o(t + (J) + VNSO);                          \
-            if (t + (J) + VNSB < nseq_b) issue_b(t + (J) + VNSB);                     \
         }                                                                             \
     }
     if (!*c.abort_flag) {
@@ -641,11 +638,11 @@ __global__ void __launch_bounds__(NT, 2)
         }
     }
 #undef VD_VSTEP
+    if (rec0) a.traces[r0] = rec_val0;
     pdl_release();
     if (*c.abort_flag && tid == 0) {
         drain(c.bar_p, hi_p, VNSP);
         drain(c.bar_o, hi_o, VNSO);
-        drain(c.bar_b, hi_b, VNSB);
     }
 }
 
@@ -785,6 +782,18 @@ __global__ void __launch_bounds__(NT, 2)
         hi_z = seq + 1;
     };
 
+    if (tid == 32) {   // first used right after the wait
+        tma_prefetch_map(&maps.vx_halo);
+        tma_prefetch_map(&maps.vy_halo);
+        tma_prefetch_map(&maps.own[2]);
+    }
+    // Does source group gi lie in this CTA's tile and planes?  The first NT
+    // groups (all of them, in practice) are looked up here, ahead of use.
+    auto source_here = [&](int gi) {
+        const int *q = a.grp_ijk + 3 * gi;
+        return q[0] >= x0 && q[0] < x0 + TX && q[1] >= y0 && q[1] < y0 + TY && q[2] >= z0 && q[2] < z0 + T;
+    };
+    const bool src0 = tid < a.ngrp && source_here(tid);
     if (tid == 0) {
         for (int s = 0; s < PNSC; ++s) mbar_init(&c.bar_c[s], 1);
         for (int s = 0; s < PNSZ; ++s) mbar_init(&c.bar_z[s], 1);
@@ -867,9 +876,7 @@ __global__ void __launch_bounds__(NT, 2)
         __syncthreads();
         if (!*c.abort_flag)
             for (int gi = tid; gi < a.ngrp; gi += NT) {
-                const int *q = a.grp_ijk + 3 * gi;
-                if (q[0] < x0 || q[0] >= x0 + TX || q[1] < y0 || q[1] >= y0 + TY || q[2] < z0 || q[2] >= z0 + T)
-                    continue;
+                if (gi < NT ? !src0 : !source_here(gi)) continue;
                 float *dst = a.p + a.grp_off[gi];
                 float v = *dst;
                 for (int m = a.grp_first[gi]; m < a.grp_first[gi + 1]; ++m) {
