@@ -485,7 +485,7 @@ mmod_status mmod_batch_autotune(mmod_batch *b, int steps, mmod_stream stream, in
  *   velocity and pressure kernels) or MMOD_KERNEL_SIMPLE (one thread per
  *   point, the same FP32 operations: the same bits).
  * mmod_vd_uses_tma: 1 when the next run uses the TMA kernels (-1: NULL).
- * mmod_vd_set_option: MMOD_OPT_PDL 0 / 1 (default 0): launch the TMA
+ * mmod_vd_set_option: MMOD_OPT_PDL 0 / 1 (default 1): launch the TMA
  *   kernels as programmatic dependents, so that each requests the data its
  *   predecessor does not write (own velocities and buoyancy; p and dt K)
  *   while the predecessor finishes; MMOD_OPT_ZLEN >= 0: planes per z range
