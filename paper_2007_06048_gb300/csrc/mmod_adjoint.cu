@@ -286,6 +286,11 @@ mmod_status encode_grad_maps(mmod_handle *h, int shape) {
     bool ok = true;
     for (int i = 0; i < gw.nwork; ++i) ok = ok && encode_maps(h->cfg, h->nxp, gw.seg[i], shape, &gw.seg_map[i]);
     for (int b = 0; b < 2; ++b) ok = ok && encode_maps(h->cfg, h->nxp, gw.psi[b], shape, &gw.psi_map[b]);
+    if (gw.dtype == MMOD_CKPT_FP32) {
+        for (int i = 0; i < 2 * gw.nslot; ++i)
+            ok = ok && encode_maps(h->cfg, h->nxp, static_cast<float *>(gw.ckpt) + (size_t)i * h->vol, shape,
+                                   &gw.ckpt_map[i]);
+    }
     if (!ok) return fail(h, MMOD_ERR_CUDA, "tensor map encoding failed for a work volume");
     gw.shape = shape;
     return MMOD_OK;
@@ -300,6 +305,7 @@ mmod_status ensure_grad_work(mmod_handle *h, int nslot, int nwork, int dtype, in
     const size_t vb = sizeof(float) * (size_t)h->vol;
     gw.seg.assign(nwork, nullptr);
     gw.seg_map.resize(nwork);
+    gw.ckpt_map.resize(2 * (size_t)nslot);
     for (int i = 0; i < nwork; ++i) {
         MMOD_CK(h, cudaMalloc(&gw.seg[i], vb));
         MMOD_CK(h, cudaMemset(gw.seg[i], 0, vb));
@@ -380,6 +386,7 @@ void free_grad_work(mmod_handle *h) {
         if (p) cudaFree(p);
     gw.seg.clear();
     gw.seg_map.clear();
+    gw.ckpt_map.clear();
     for (float *&p : gw.psi) {
         if (p) cudaFree(p);
         p = nullptr;
@@ -468,8 +475,12 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
     if (!h->st_adjw) MMOD_CK(h, cudaMalloc(&h->st_adjw, sizeof(float) * std::max<size_t>(nres, 1)));
     if (nres) MMOD_CK(h, cudaMemcpyAsync(h->st_adjw, dres, sizeof(float) * nres, cudaMemcpyDeviceToDevice, s));
 
-    MMOD_CK(h, cudaMemsetAsync(h->u[0], 0, vb, s));
-    MMOD_CK(h, cudaMemsetAsync(h->u[1], 0, vb, s));
+    // segments with FP32 checkpoints step through the checkpoint volumes themselves
+    const bool through = ckpt_dtype == MMOD_CKPT_FP32 && seglen >= 2;
+    if (!through) {
+        MMOD_CK(h, cudaMemsetAsync(h->u[0], 0, vb, s));
+        MMOD_CK(h, cudaMemsetAsync(h->u[1], 0, vb, s));
+    }
     h->state_pending = false;
     StepArgs fa = base_args(h, h->fwd, dwav, shape);
     fa.nrec = 0;   // no receivers in the gradient's forward sweeps
@@ -494,17 +505,39 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
         fa.uout = h->u[n & 1];
         return enqueue_step(h, fa, u_map[(n + 1) & 1], u_map[n & 1], tma, nullptr, s, &launches);
     };
-    // forward step n of a replay in the work volumes w0, w1 (u^{n-1} in w0,
-    // u^n in w1, u^{n+1} over u^{n-1}), also writing g^n into gout
-    auto fwd_step_g = [&](int n, int w0, int w1, float *gout) {
+    // forward step n from u^{n-1} in prev and u^n in cur into out (prev's
+    // volume or another), also writing g^n into gout (null: not)
+    struct Vol {
+        float *p;
+        const VolMaps *m;
+    };
+    auto seg = [&](int i) { return Vol{gw.seg[i], &gw.seg_map[i]}; };
+    auto slot = [&](int sg, int i) {
+        return Vol{static_cast<float *>(gw.ckpt) + (size_t)(2 * sg + i) * h->vol, &gw.ckpt_map[2 * sg + i]};
+    };
+    auto fwd_step = [&](int n, Vol prev, Vol cur, Vol out, float *gout) {
         fa.n = n;
-        fa.ucur = gw.seg[w1];
-        fa.uprev = gw.seg[w0];
-        fa.uout = gw.seg[w0];
+        fa.ucur = cur.p;
+        fa.uprev = prev.p;
+        fa.uout = out.p;
         fa.gout = gout;
-        const cudaError_t e = enqueue_step(h, fa, gw.seg_map[w1], gw.seg_map[w0], tma, nullptr, s, &launches);
+        const cudaError_t e = enqueue_step(h, fa, *cur.m, *prev.m, tma, nullptr, s, &launches);
         fa.gout = nullptr;
         return e;
+    };
+    // forward step n of a replay in the work volumes w0, w1 (u^{n-1} in w0,
+    // u^n in w1, u^{n+1} over u^{n-1}), also writing g^n into gout
+    auto fwd_step_g = [&](int n, int w0, int w1, float *gout) { return fwd_step(n, seg(w0), seg(w1), seg(w0), gout); };
+    // forward steps a0 .. b0-1 from the state in p0 (u^{a0-1}), p1 (u^{a0}),
+    // which stay as they are, through q0, q1: u^{a0+1+j} lands in q0, q1 in
+    // turn; gof(j): where g of step a0 + j goes (null: not written)
+    auto fwd_range = [&](int a0, int b0, Vol p0, Vol p1, Vol q0, Vol q1, auto gof) -> cudaError_t {
+        for (int n = a0; n < b0; ++n) {
+            const int j = n - a0;
+            const Vol out = j & 1 ? q1 : q0, prev = j == 0 ? p0 : j == 1 ? p1 : out, cur = j == 0 ? p1 : j & 1 ? q0 : q1;
+            if (cudaError_t e = fwd_step(n, prev, cur, out, gof(j))) return e;
+        }
+        return cudaSuccess;
     };
     // adjoint step of forward step n: adjoint step m = nt-1-n produces
     // psi^{n+1} in psi[m & 1] (psi^{n+2} stays in the other buffer until the
@@ -609,18 +642,29 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
         // bit, so the first sweep writes g^n of the last segment straight into
         // the segment buffer and that segment is neither saved nor replayed.
         // (A 16-bit checkpoint would start its replay from the rounded state.)
-        const bool keep_last = ckpt_dtype == MMOD_CKPT_FP32;
         // ---- sweep 1: forward with a checkpoint at the start of every segment
-        for (int sg = 0; sg < nseg; ++sg) {
-            const int a0 = sg * seglen, b0 = std::min(nt, a0 + seglen);
-            const bool last = keep_last && sg == nseg - 1;
-            if (!last)   // at step a0: u^{a0-1} in u[a0 & 1], u^{a0} in u[(a0 + 1) & 1]
+        if (through) {
+            // no copies: the volumes that hold the state at step a0 are segment
+            // sg's checkpoint (slot sg) and the segment steps on into the next
+            // slot's; the last segment stays in its own slot.  (Saving and
+            // restoring 20 checkpoints of 200^3 took 78 copies of 34 MB, 1 of
+            // 42 ms.)  After a full segment u^{b0} is in volume (seglen - 1) & 1.
+            MMOD_CK(h, cudaMemsetAsync(slot(0, 0).p, 0, 2 * vb, s));
+            for (int sg = 0; sg < nseg; ++sg) {
+                const int a0 = sg * seglen, b0 = std::min(nt, a0 + seglen), i = sg == 0 ? 0 : seglen & 1;
+                if (sg < nseg - 1)
+                    MMOD_CK(h, fwd_range(a0, b0, slot(sg, i), slot(sg, 1 - i), slot(sg + 1, 0), slot(sg + 1, 1),
+                                         [](int) -> float * { return nullptr; }));
+                else
+                    MMOD_CK(h, fwd_range(a0, b0, slot(sg, i), slot(sg, 1 - i), slot(sg, i), slot(sg, 1 - i),
+                                         [&](int j) { return gw.seg[2 + j]; }));
+            }
+        } else {
+            for (int sg = 0; sg < nseg; ++sg) {
+                const int a0 = sg * seglen, b0 = std::min(nt, a0 + seglen);
+                // at step a0: u^{a0-1} in u[a0 & 1], u^{a0} in u[(a0 + 1) & 1]
                 MMOD_CK(h, save_state(h, sg, h->u[a0 & 1], h->u[(a0 + 1) & 1], s));
-            for (int n = a0; n < b0; ++n) {
-                fa.gout = last ? gw.seg[2 + n - a0] : nullptr;
-                const cudaError_t e = fwd_step_in_place(n);
-                fa.gout = nullptr;
-                MMOD_CK(h, e);
+                for (int n = a0; n < b0; ++n) MMOD_CK(h, fwd_step_in_place(n));
             }
         }
         // ---- backward: replay each segment (g^n of its steps), then its
@@ -630,7 +674,11 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
         MMOD_CK(h, cudaMemsetAsync(gw.gradc, 0, vb, s));
         for (int sg = nseg - 1; sg >= 0; --sg) {
             const int a0 = sg * seglen, b0 = std::min(nt, a0 + seglen);
-            if (!(keep_last && sg == nseg - 1)) {
+            if (through && sg < nseg - 1) {
+                const int i = sg == 0 ? 0 : seglen & 1;
+                MMOD_CK(h, fwd_range(a0, b0, slot(sg, i), slot(sg, 1 - i), seg(0), seg(1),
+                                     [&](int j) { return gw.seg[2 + j]; }));
+            } else if (!through) {
                 MMOD_CK(h, restore_state(h, sg, gw.seg[0], gw.seg[1], s));
                 for (int n = a0; n < b0; ++n) {   // seg[2 + n - a0] receives g^n
                     const int j = n - a0;

@@ -131,6 +131,7 @@ struct mmod_handle {
         std::vector<mmod::VolMaps> seg_map;
         float *psi[2] = {nullptr, nullptr};
         mmod::VolMaps psi_map[2];
+        std::vector<mmod::VolMaps> ckpt_map;   // FP32 checkpoints: the steps read and write them in place
         float *gradc = nullptr;             // padded FP32 sum of psi^{n+1} g^n
         void *ckpt = nullptr;               // nslot * 2 volumes (FP32 or 16-bit)
         float *ckpt_scale = nullptr;        // 16-bit storage: per-plane (BF16, FP16) or per-32-value
