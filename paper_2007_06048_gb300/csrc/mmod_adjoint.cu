@@ -106,6 +106,9 @@ __global__ void __cluster_dims__(kPlaneCtas, 1, 1) __launch_bounds__(256)
     compress_kernel(const CkptPair<T> p, long long plane) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
+    // programmatic dependent launch: the step that follows only reads these volumes before its own wait
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int k = blockIdx.x / kPlaneCtas, rank = blockIdx.x % kPlaneCtas, vol = blockIdx.y;
     const float4 *u = reinterpret_cast<const float4 *>(p.u[vol] + (long long)k * plane);
     const long long groups = plane >> 3;
@@ -145,6 +148,8 @@ __global__ void __cluster_dims__(kPlaneCtas, 1, 1) __launch_bounds__(256)
 
 template <class T>
 __global__ void __launch_bounds__(256) decompress_kernel(const CkptPair<T> p, long long plane, int ctas) {
+    // no early release: the step that follows reads what this kernel writes before its own wait
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int k = blockIdx.x / ctas, vol = blockIdx.y;   // ctas CTAs per plane
     const uint4 *in = reinterpret_cast<const uint4 *>(p.q[vol] + (long long)k * plane);
     float4 *u = reinterpret_cast<float4 *>(p.u[vol] + (long long)k * plane);
@@ -176,6 +181,8 @@ __device__ __forceinline__ short bfp_value(float v, float m) {
 }
 
 __global__ void __launch_bounds__(256) compress_bfp_kernel(const CkptPair<short> p, long long nblocks) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // as compress_kernel
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const float4 *u = reinterpret_cast<const float4 *>(p.u[blockIdx.y]);
     uint4 *out = reinterpret_cast<uint4 *>(p.q[blockIdx.y]);
     const long long groups = 4 * nblocks, stride = (long long)gridDim.x * 256;
@@ -196,6 +203,7 @@ __global__ void __launch_bounds__(256) compress_bfp_kernel(const CkptPair<short>
 }
 
 __global__ void __launch_bounds__(256) decompress_bfp_kernel(const CkptPair<short> p, long long nblocks) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // no early release, as decompress_kernel
     const uint4 *in = reinterpret_cast<const uint4 *>(p.q[blockIdx.y]);
     float4 *u = reinterpret_cast<float4 *>(p.u[blockIdx.y]);
     const long long groups = 4 * nblocks, stride = (long long)gridDim.x * 256;
@@ -236,6 +244,22 @@ CkptPair<T> ckpt_pair(mmod_handle *h, int slot, float *u_prev, float *u_cur) {
     return p;
 }
 
+// Launch of a checkpoint kernel, chained to its stream predecessor by
+// programmatic dependent launch where the handle uses it.
+template <class... P, class... A>
+cudaError_t launch_ckpt(const mmod_handle *h, void (*fn)(P...), dim3 grid, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = grid;
+    lc.blockDim = dim3(256);
+    lc.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = h->pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&lc, fn, P(args)...);
+}
+
 // Save the state (u^{a-1}, u^a) into checkpoint slot (FP32: copies; 16-bit: compress).
 cudaError_t save_state(mmod_handle *h, int slot, float *u_prev, float *u_cur, cudaStream_t s) {
     const int dtype = h->gw.dtype;
@@ -249,12 +273,12 @@ cudaError_t save_state(mmod_handle *h, int slot, float *u_prev, float *u_cur, cu
     }
     if (dtype == MMOD_CKPT_BFP16) {
         const long long nb = h->vol / kBfpBlock;
-        compress_bfp_kernel<<<dim3(bfp_grid(nb), 2), 256, 0, s>>>(ckpt_pair<short>(h, slot, u_prev, u_cur), nb);
-    } else if (dtype == MMOD_CKPT_BF16)
-        compress_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(ckpt_pair<__nv_bfloat16>(h, slot, u_prev, u_cur), h->plane);
-    else
-        compress_kernel<__half><<<grid, 256, 0, s>>>(ckpt_pair<__half>(h, slot, u_prev, u_cur), h->plane);
-    return cudaGetLastError();
+        return launch_ckpt(h, compress_bfp_kernel, dim3(bfp_grid(nb), 2), s, ckpt_pair<short>(h, slot, u_prev, u_cur), nb);
+    }
+    if (dtype == MMOD_CKPT_BF16)
+        return launch_ckpt(h, compress_kernel<__nv_bfloat16>, grid, s,
+                           ckpt_pair<__nv_bfloat16>(h, slot, u_prev, u_cur), h->plane);
+    return launch_ckpt(h, compress_kernel<__half>, grid, s, ckpt_pair<__half>(h, slot, u_prev, u_cur), h->plane);
 }
 
 cudaError_t restore_state(mmod_handle *h, int slot, float *u_prev, float *u_cur, cudaStream_t s) {
@@ -270,13 +294,13 @@ cudaError_t restore_state(mmod_handle *h, int slot, float *u_prev, float *u_cur,
     }
     if (dtype == MMOD_CKPT_BFP16) {
         const long long nb = h->vol / kBfpBlock;
-        decompress_bfp_kernel<<<dim3(bfp_grid(nb), 2), 256, 0, s>>>(ckpt_pair<short>(h, slot, u_prev, u_cur), nb);
-    } else if (dtype == MMOD_CKPT_BF16)
-        decompress_kernel<__nv_bfloat16>
-            <<<grid, 256, 0, s>>>(ckpt_pair<__nv_bfloat16>(h, slot, u_prev, u_cur), h->plane, per);
-    else
-        decompress_kernel<__half><<<grid, 256, 0, s>>>(ckpt_pair<__half>(h, slot, u_prev, u_cur), h->plane, per);
-    return cudaGetLastError();
+        return launch_ckpt(h, decompress_bfp_kernel, dim3(bfp_grid(nb), 2), s, ckpt_pair<short>(h, slot, u_prev, u_cur),
+                           nb);
+    }
+    if (dtype == MMOD_CKPT_BF16)
+        return launch_ckpt(h, decompress_kernel<__nv_bfloat16>, grid, s,
+                           ckpt_pair<__nv_bfloat16>(h, slot, u_prev, u_cur), h->plane, per);
+    return launch_ckpt(h, decompress_kernel<__half>, grid, s, ckpt_pair<__half>(h, slot, u_prev, u_cur), h->plane, per);
 }
 
 // Tensor maps of the work volumes for the run's tile shape.
