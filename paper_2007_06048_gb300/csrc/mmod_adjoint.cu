@@ -310,6 +310,7 @@ mmod_status encode_grad_maps(mmod_handle *h, int shape) {
     bool ok = true;
     for (int i = 0; i < gw.nwork; ++i) ok = ok && encode_maps(h->cfg, h->nxp, gw.seg[i], shape, &gw.seg_map[i]);
     for (int b = 0; b < 2; ++b) ok = ok && encode_maps(h->cfg, h->nxp, gw.psi[b], shape, &gw.psi_map[b]);
+    ok = ok && encode_maps(h->cfg, h->nxp, gw.gradc, shape, &gw.gradc_map);
     if (gw.dtype == MMOD_CKPT_FP32) {
         for (int i = 0; i < 2 * gw.nslot; ++i)
             ok = ok && encode_maps(h->cfg, h->nxp, static_cast<float *>(gw.ckpt) + (size_t)i * h->vol, shape,
@@ -624,6 +625,9 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
         MMOD_CK(h, cudaMemsetAsync(gw.psi[1], 0, vb, s));
         MMOD_CK(h, cudaMemsetAsync(gw.gradc, 0, vb, s));
         float *unext = gw.seg[0], *gn = gw.seg[1];
+        // the imaging form of the step kernel: g^n is formed and used in one pass
+        const bool one_pass = tma && active_plan(h).has_image && h->claim_planes == 0 &&
+                              h->fwd.inj[shape].npts <= kMaxImageSources;
         for (const RevAction &act : sched) {
             switch (act.kind) {
                 case MMOD_REV_ADVANCE:
@@ -640,8 +644,21 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
                         MMOD_CK(h, restore_state(h, act.a, h->u[act.b & 1], h->u[(act.b + 1) & 1], s));
                     }
                     break;
-                case MMOD_REV_REVERSE: {   // g^n from the working state, then the adjoint step and its term
+                case MMOD_REV_REVERSE: {   // the adjoint step and its term, g^n from the working state
                     const int n = act.a;
+                    if (one_pass) {
+                        MMOD_CK(h, adj_step(n));
+                        StepArgs ia = fa;
+                        ia.n = n;
+                        ia.pdl = h->pdl;
+                        ia.image = 1;
+                        ia.ucur = h->u[(n + 1) & 1];
+                        ia.uprev = ia.uout = gw.gradc;
+                        ia.c = gw.psi[(nt - 1 - n) & 1];
+                        MMOD_CK(h, enqueue_step(h, ia, u_map[(n + 1) & 1], gw.gradc_map, tma, nullptr, s, &launches,
+                                                &gw.psi_map[(nt - 1 - n) & 1].own));
+                        break;
+                    }
                     fa.n = n;
                     fa.ucur = h->u[(n + 1) & 1];
                     fa.uprev = h->u[n & 1];

@@ -458,10 +458,11 @@ StepArgs base_args(mmod_handle *h, const Geometry &geo, const float *wavelet, in
 // injection kernel, then (if plain_gather_dst) the receivers of u^{n+1}.
 // TMA path: one kernel (injection inside; receivers of u^n go to a.traces).
 cudaError_t enqueue_step(mmod_handle *h, const StepArgs &a, const VolMaps &cur, const VolMaps &prev, bool tma,
-                         float *plain_gather_dst, cudaStream_t s, long long *count) {
+                         float *plain_gather_dst, cudaStream_t s, long long *count, const CUtensorMap *c_map) {
     cudaError_t e;
     if (tma) {
-        e = launch_step_tma(a, cur, prev, h->shapes[active_shape(h)].c.own, a.gout ? g_plan(h) : active_plan(h), s);
+        e = launch_step_tma(a, cur, prev, c_map ? *c_map : h->shapes[active_shape(h)].c.own,
+                            a.gout ? g_plan(h) : active_plan(h), s);
         ++*count;
         return e;
     }

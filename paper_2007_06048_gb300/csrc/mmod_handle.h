@@ -130,7 +130,7 @@ struct mmod_handle {
         std::vector<float *> seg;           // nwork padded FP32 work volumes
         std::vector<mmod::VolMaps> seg_map;
         float *psi[2] = {nullptr, nullptr};
-        mmod::VolMaps psi_map[2];
+        mmod::VolMaps psi_map[2], gradc_map;
         std::vector<mmod::VolMaps> ckpt_map;   // FP32 checkpoints: the steps read and write them in place
         float *gradc = nullptr;             // padded FP32 sum of psi^{n+1} g^n
         void *ckpt = nullptr;               // nslot * 2 volumes (FP32 or 16-bit)
@@ -183,7 +183,8 @@ StepArgs base_args(mmod_handle *h, const Geometry &geo, const float *wavelet, in
 // Enqueues one step (plain path: step, injection, optional gather of
 // u^{n+1} into plain_gather_dst; TMA path: one kernel).
 cudaError_t enqueue_step(mmod_handle *h, const StepArgs &a, const VolMaps &cur, const VolMaps &prev, bool tma,
-                         float *plain_gather_dst, cudaStream_t s, long long *count);
+                         float *plain_gather_dst, cudaStream_t s, long long *count,
+                         const CUtensorMap *c_map = nullptr);   // c_map: the operand in c's place (null: c)
 // The nt-step loop of a run from u[0], u[1] with geometry geo, captured into
 // the graph slot g on first use and replayed.
 mmod_status run_loop_graph(mmod_handle *h, GraphSlot &g, const Geometry &geo, const float *wav, float *tr,

@@ -60,6 +60,8 @@ struct StepArgs {
                                           // 0 between launches (null: the static plan)
     float *gout;                          // gradient replay: also write g^n = L u^n + s^n here
                                           // (padded layout; null: not written)
+    int image;                            // not a step but its imaging term: uout = uprev + c (L u^n + s^n)
+                                          // with the accumulator as uprev and uout and psi^{n+1} as c
     float inv_cell;                       // 1 / (hx hy hz): s^n = w[n] / (hx hy hz) at a source
 };
 
@@ -140,6 +142,33 @@ __device__ __forceinline__ void inject_g_points(const StepArgs &a, int n, int lo
                           a.inv_cell, v);
         *dst = v;
     }
+}
+
+// u = 0 outside the grid, except above a free surface: the odd image
+// u(i, j, -m) = -u(i, j, m).
+__device__ __forceinline__ float ld0(const float *__restrict__ u, const StepArgs &a, int i, int j,
+                                     int k) {
+    const bool image = a.fs && k < 0;
+    if (image) k = -k;
+    const bool in = (unsigned)i < (unsigned)a.nx && (unsigned)j < (unsigned)a.ny &&
+                    (unsigned)k < (unsigned)a.nz;
+    const float v = in ? __ldg(u + (long long)k * a.plane + (long long)j * a.nxp + i) : 0.0f;
+    return image ? -v : v;
+}
+
+// L u at one point, p = u(i, j, k): the plain kernel's operations (stencil.cuh's order).
+__device__ __forceinline__ float lap_point(const StepArgs &a, const float *u, float p, int i, int j, int k) {
+    const float two_p = __fadd_rn(p, p);
+    float lx = pair_first(a.w.x[0], ld0(u, a, i + 1, j, k), ld0(u, a, i - 1, j, k), two_p);
+    float ly = pair_first(a.w.y[0], ld0(u, a, i, j + 1, k), ld0(u, a, i, j - 1, k), two_p);
+    float lz = pair_first(a.w.z[0], ld0(u, a, i, j, k + 1), ld0(u, a, i, j, k - 1), two_p);
+#pragma unroll
+    for (int m = 2; m <= kRadius; ++m) {
+        lx = pair_acc(lx, a.w.x[m - 1], ld0(u, a, i + m, j, k), ld0(u, a, i - m, j, k), two_p);
+        ly = pair_acc(ly, a.w.y[m - 1], ld0(u, a, i, j + m, k), ld0(u, a, i, j - m, k), two_p);
+        lz = pair_acc(lz, a.w.z[m - 1], ld0(u, a, i, j, k + m), ld0(u, a, i, j, k - m), two_p);
+    }
+    return lap_sum(lx, ly, lz);
 }
 
 // Host helpers shared by the entry points (mmod_api.cu).

@@ -9,18 +9,6 @@
 namespace mmod {
 namespace {
 
-// u = 0 outside the grid, except above a free surface: the odd image
-// u(i, j, -m) = -u(i, j, m).
-__device__ __forceinline__ float ld0(const float *__restrict__ u, const StepArgs &a, int i, int j,
-                                     int k) {
-    const bool image = a.fs && k < 0;
-    if (image) k = -k;
-    const bool in = (unsigned)i < (unsigned)a.nx && (unsigned)j < (unsigned)a.ny &&
-                    (unsigned)k < (unsigned)a.nz;
-    const float v = in ? __ldg(u + (long long)k * a.plane + (long long)j * a.nxp + i) : 0.0f;
-    return image ? -v : v;
-}
-
 __global__ void __launch_bounds__(128) step_simple_kernel(const StepArgs a) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -29,16 +17,7 @@ __global__ void __launch_bounds__(128) step_simple_kernel(const StepArgs a) {
     const long long o = (long long)k * a.plane + (long long)j * a.nxp + i;
     const float p = __ldg(a.ucur + o);
     const float two_p = __fadd_rn(p, p);
-    float lx = pair_first(a.w.x[0], ld0(a.ucur, a, i + 1, j, k), ld0(a.ucur, a, i - 1, j, k), two_p);
-    float ly = pair_first(a.w.y[0], ld0(a.ucur, a, i, j + 1, k), ld0(a.ucur, a, i, j - 1, k), two_p);
-    float lz = pair_first(a.w.z[0], ld0(a.ucur, a, i, j, k + 1), ld0(a.ucur, a, i, j, k - 1), two_p);
-#pragma unroll
-    for (int m = 2; m <= kRadius; ++m) {
-        lx = pair_acc(lx, a.w.x[m - 1], ld0(a.ucur, a, i + m, j, k), ld0(a.ucur, a, i - m, j, k), two_p);
-        ly = pair_acc(ly, a.w.y[m - 1], ld0(a.ucur, a, i, j + m, k), ld0(a.ucur, a, i, j - m, k), two_p);
-        lz = pair_acc(lz, a.w.z[m - 1], ld0(a.ucur, a, i, j, k + m), ld0(a.ucur, a, i, j, k - m), two_p);
-    }
-    const float lap = lap_sum(lx, ly, lz);
+    const float lap = lap_point(a, a.ucur, p, i, j, k);
     const float e = __fadd_rn(__fadd_rn(__ldg(a.ex + i), __ldg(a.ey + j)), __ldg(a.ez + k));
     const float out = __fmul_rn(num_damped(two_p, a.uprev[o], __ldg(a.c + o), lap, e), damp_factor(e));
     a.uout[o] = (a.fs && k == 0) ? 0.0f : out;   // p = 0 on a free surface

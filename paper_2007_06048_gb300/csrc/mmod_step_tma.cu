@@ -132,11 +132,10 @@ __device__ __forceinline__ PlaneInfo plane_info(const StepArgs &a, int k) {
 
 // One z step computing plane z0 + t.  The queue window of this step is
 // q[J .. J+8] (planes k-4 .. k+4); the leading plane k+4 lands in q[J+8].
-template <class S, int J, bool G>
+template <class S, int J>
 __device__ __forceinline__ void step(const StepArgs &a, const Ctx &c, int t, float2 (&q)[S::QD][S::RY],
                                      const Wts &w, float2 exr, const float (&eyr)[S::RY], bool xy_damped,
-                                     const PlaneInfo &pi, float *const (&out_row)[S::RY],
-                                     float *const (&g_row)[S::RY]) {
+                                     const PlaneInfo &pi, float *const (&out_row)[S::RY]) {
     constexpr int RY = S::RY;
     const int k = c.z0 + t;
     // 1. the leading plane k+4 (sequence t+8) enters the queue
@@ -197,16 +196,6 @@ __device__ __forceinline__ void step(const StepArgs &a, const Ctx &c, int t, flo
                 *reinterpret_cast<float2 *>(dst) = num;
             else
                 dst[0] = num.x;
-        }
-        if constexpr (G) {   // g^n = L u^n (sources added after the z range), 0 on a free surface
-            if (g_row[r]) {
-                const float2 gv = (a.fs && k == 0) ? make_float2(0.0f, 0.0f) : lap;
-                float *dst = g_row[r] + koff;
-                if (c.x0 + 2 * c.lane + 1 < a.nx)
-                    *reinterpret_cast<float2 *>(dst) = gv;
-                else
-                    dst[0] = gv.x;
-            }
         }
     }
 }
@@ -285,7 +274,7 @@ __device__ __noinline__ void NeighborDep::wait(int tid, int *abort_flag, int *er
 // shot).  The single-shot kernel passes its parameters; the batch kernel a
 // shot's arguments staged in shared memory and that shot's tensor maps in
 // global memory.
-template <class S, class Dep, bool G = false>
+template <class S, class Dep>
 __device__ __forceinline__ void step_tma_body(const StepArgs &a, const StepVar &v, const CUtensorMap *cur_map,
                                               const CUtensorMap *prev_map, const CUtensorMap *c_map, const Geom &g,
                                               int bid, int nbid, const Dep &dep) {
@@ -366,13 +355,11 @@ __device__ __forceinline__ void step_tma_body(const StepArgs &a, const StepVar &
     exr.y = x + 1 < a.nx ? __ldg(a.ex + x + 1) : 0.0f;
     float eyr[RY];
     float *out_row[RY];   // u^{n+1} row pointers at plane 0; null outside the grid
-    float *g_row[RY];     // the same rows of g^n (G only)
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
         const int y = c.y0 + RY * c.warp + r;
         eyr[r] = y < a.ny ? __ldg(a.ey + y) : 0.0f;
         out_row[r] = (y < a.ny && x < a.nx) ? v.uout + (long long)y * a.nxp + x : nullptr;
-        g_row[r] = (G && y < a.ny && x < a.nx) ? a.gout + (long long)y * a.nxp + x : nullptr;
     }
     const bool xy_damped = c.x0 < a.nbl || c.x0 + TX - 1 > a.nx - 1 - a.nbl || c.y0 < a.nbl ||
                            c.y0 + S::TY - 1 > a.ny - 1 - a.nbl;
@@ -427,7 +414,7 @@ __device__ __forceinline__ void step_tma_body(const StepArgs &a, const StepVar &
 #define MMOD_STEP(J)                                                                        \
     if (t + (J) < T) {                                                                      \
         const PlaneInfo pi_next = plane_info(a, c.z0 + t + (J) + 1);                        \
-        step<S, (J), G>(a, c, t + (J), q, w, exr, eyr, xy_damped, pi, out_row, g_row);     \
+        step<S, (J)>(a, c, t + (J), q, w, exr, eyr, xy_damped, pi, out_row);                \
         pi = pi_next;                                                                       \
         __syncthreads();                                                                    \
         if (*c.abort_flag) break;                                                           \
@@ -461,7 +448,6 @@ __device__ __forceinline__ void step_tma_body(const StepArgs &a, const StepVar &
         const long long b = ((long long)ty * a.inj.tiles_x + tx) * a.nz + c.z0;
         const int lo = __ldg(a.inj.tile_start + b), hi = __ldg(a.inj.tile_start + b + T);
         inject_points(a, v.uout, v.n, lo, hi, tid, S::NT);
-        if constexpr (G) inject_g_points(a, v.n, lo, hi, tid, S::NT);
     }
     // After a give-up, wait (bounded) for the copies this CTA still has in
     // flight (the latest sequence of every slot) before its shared memory is
@@ -480,21 +466,20 @@ __device__ __forceinline__ void step_tma_body(const StepArgs &a, const StepVar &
 namespace mmod {
 namespace {
 
-template <class S, class Dep, bool G = false>
+template <class S, class Dep, int MODE = kStepOnly>
 __device__ __forceinline__ void step_body(const StepArgs &a, const StepVar &v, const CUtensorMap *halo_map,
                                           const CUtensorMap *own_map, const CUtensorMap *prev_map,
                                           const CUtensorMap *c_map, const Geom &g, int bid, int nbid, const Dep &dep) {
     if constexpr (S::kStaged)
-        step_staged_body<S, Dep, G>(a, v, halo_map, own_map, prev_map, c_map, g, bid, nbid, dep);
+        step_staged_body<S, Dep, MODE>(a, v, halo_map, own_map, prev_map, c_map, g, bid, nbid, dep);
     else
-        step_tma_body<S, Dep, G>(a, v, halo_map, prev_map, c_map, g, bid, nbid, dep);
+        step_tma_body<S, Dep>(a, v, halo_map, prev_map, c_map, g, bid, nbid, dep);
 }
 
-// G: also write g^n = L u^n + s^n into a.gout (the gradient's imaging factor).
-template <class S, bool G = false>
+template <class S, int MODE = kStepOnly>
 __global__ void __launch_bounds__(S::NT, S::MINB)
     step_tma_kernel(const StepArgs a, const __grid_constant__ StepMaps maps, const Geom g) {
-    step_body<S, PdlDep, G>(a, StepVar{a.n, a.uout, a.ucur, a.traces}, &maps.halo, &maps.own, &maps.prev, &maps.c, g,
+    step_body<S, PdlDep, MODE>(a, StepVar{a.n, a.uout, a.ucur, a.traces}, &maps.halo, &maps.own, &maps.prev, &maps.c, g,
                             blockIdx.x, gridDim.x, PdlDep{a.pdl});
 }
 
@@ -523,7 +508,7 @@ struct ClaimDep {
     }
 };
 
-template <class S, bool G = false>
+template <class S, int MODE = kStepOnly>
 __global__ void __launch_bounds__(S::NT, S::MINB2)
     step_tma_claim_kernel(const StepArgs a, const __grid_constant__ StepMaps maps, const Geom g, int units) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -532,7 +517,7 @@ __global__ void __launch_bounds__(S::NT, S::MINB2)
     int *next = abort_flag + 1;
     bool first = true;
     for (int unit = blockIdx.x; unit < units;) {
-        step_body<S, ClaimDep, G>(a, StepVar{a.n, a.uout, a.ucur, a.traces}, &maps.halo, &maps.own, &maps.prev,
+        step_body<S, ClaimDep, MODE>(a, StepVar{a.n, a.uout, a.ucur, a.traces}, &maps.halo, &maps.own, &maps.prev,
                                   &maps.c, g, unit, units, ClaimDep{a.pdl, first});
         first = false;
         __syncthreads();
@@ -771,14 +756,16 @@ struct Variant {
     int shape;                // tile shape
     const void *g_fn;         // null: no form that also writes g^n
     const void *claim_g_fn;
+    const void *image_fn;     // null: no imaging form (StepArgs::image)
 };
 
 #define MMOD_VARIANT(V, desc, P, C) \
     {desc, (const void *)step_tma_kernel<V>, (const void *)step_tma_batch_kernel<V>, P, C, V::NT, V::SMEM, \
-     batch_smem<V>(), 0, nullptr, nullptr}
+     batch_smem<V>(), 0, nullptr, nullptr, nullptr}
 #define MMOD_STAGED_VARIANT(SH, desc)                                                                              \
     {desc, (const void *)step_tma_kernel<StagedShape<SH>>, nullptr, nullptr, nullptr, StagedShape<SH>::NT,         \
-     StagedShape<SH>::SMEM, 0, SH, (const void *)step_tma_kernel<StagedShape<SH>, true>, nullptr}
+     StagedShape<SH>::SMEM, 0, SH, (const void *)step_tma_kernel<StagedShape<SH>, kStepG>, nullptr, \
+     (const void *)step_tma_kernel<StagedShape<SH>, kImage>}
 const Variant kVariants[] = {
     MMOD_VARIANT(V22_1, "64x16 tile, 2x2 points/thread, z unroll 1", nullptr, nullptr),
     MMOD_VARIANT(V22_2, "64x16 tile, 2x2 points/thread, z unroll 2", nullptr,
@@ -786,7 +773,8 @@ const Variant kVariants[] = {
     {"64x16 tile, 2x2 points/thread, z unroll 4", (const void *)step_tma_kernel<V22_4>,
      (const void *)step_tma_batch_kernel<V22_4>, (const void *)step_tma_persistent_kernel<V22_4>,
      (const void *)step_tma_claim_kernel<V22_4>, V22_4::NT, V22_4::SMEM, batch_smem<V22_4>(), 0,
-     (const void *)step_tma_kernel<V22_4, true>, (const void *)step_tma_claim_kernel<V22_4, true>},
+     (const void *)step_tma_kernel<V22_4, kStepG>, (const void *)step_tma_claim_kernel<V22_4, kStepG>,
+     (const void *)step_tma_kernel<V22_4, kImage>},
     MMOD_VARIANT(V24_1, "64x16 tile, 2x4 points/thread, z unroll 1", nullptr, nullptr),
     MMOD_VARIANT(V24_2, "64x16 tile, 2x4 points/thread, z unroll 2", nullptr, nullptr),
     MMOD_VARIANT(V24_2s, "64x16 tile, 2x4 points/thread, z unroll 2, shallow rings",
@@ -843,7 +831,7 @@ bool make_tma_plan(const mmod_config &cfg, TmaPlan plans[]) {
         int occ = 0;
         if (!set_smem(var.fn, var.smem) || !set_smem(var.batch_fn, var.batch_smem) ||
             !set_smem(var.claim_fn, var.smem) || !set_smem(var.persist_fn, var.smem) ||
-            !set_smem(var.g_fn, var.smem) || !set_smem(var.claim_g_fn, var.smem) ||
+            !set_smem(var.g_fn, var.smem) || !set_smem(var.claim_g_fn, var.smem) || !set_smem(var.image_fn, var.smem) ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, var.fn, var.nt, var.smem) != cudaSuccess || occ < 1) {
             cudaGetLastError();
             return false;
@@ -868,6 +856,7 @@ bool make_tma_plan(const mmod_config &cfg, TmaPlan plans[]) {
         p.variant = v;
         p.shape = var.shape;
         p.has_g = var.g_fn != nullptr;
+        p.has_image = var.image_fn != nullptr;
         p.tiles_x = tiles_x;
         p.tiles_y = tiles_y;
         p.zchunks = best_c;
@@ -936,8 +925,10 @@ cudaError_t launch_step_tma(const StepArgs &a, const VolMaps &cur, const VolMaps
     Geom cg;
     int units = 0, cgrid = 0;
     const bool claim = a.claim && claim_geom(plan, a.nz, &cg, &units, &cgrid) &&
-                       (!a.gout || kVariants[plan.variant].claim_g_fn);
-    if (a.gout && !plan.has_g) return cudaErrorInvalidValue;
+                       !a.image && (!a.gout || kVariants[plan.variant].claim_g_fn);
+    if ((a.gout && !plan.has_g) || (a.image && (!plan.has_image || a.gout || a.pdl == 2)) ||
+        (a.image && a.inj.npts > kMaxImageSources))
+        return cudaErrorInvalidValue;
     const Geom g = claim ? cg : Geom{plan.tiles_x, plan.tiles_y, plan.zchunks, plan.zlen};
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(claim ? cgrid : plan.grid);
@@ -955,8 +946,8 @@ cudaError_t launch_step_tma(const StepArgs &a, const VolMaps &cur, const VolMaps
     StepMaps m = maps;
     Geom geom = g;
     void *params[4] = {&args, &m, &geom, &units};
-    const cudaError_t e = cudaLaunchKernelExC(
-        &lc, claim ? (a.gout ? var.claim_g_fn : var.claim_fn) : (a.gout ? var.g_fn : var.fn), params);
+    const void *fn = a.image ? var.image_fn : claim ? (a.gout ? var.claim_g_fn : var.claim_fn) : a.gout ? var.g_fn : var.fn;
+    const cudaError_t e = cudaLaunchKernelExC(&lc, fn, params);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

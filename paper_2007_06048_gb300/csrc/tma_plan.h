@@ -21,10 +21,14 @@ struct TmaShape {
 constexpr int kNumShapes = 4;
 constexpr TmaShape kTmaShapes[kNumShapes] = {{64, 16, 72}, {48, 20, 56}, {40, 24, 52}, {32, 32, 40}};
 
+// Source points the imaging form takes: one per thread of its smallest block.
+constexpr int kMaxImageSources = 240;
+
 struct TmaPlan {
     int variant = 0;                // index into the compiled variants
     int shape = 0;                  // index into kTmaShapes
     bool has_g = false;             // compiled with the g^n output (StepArgs::gout)
+    bool has_image = false;         // compiled with the imaging form (StepArgs::image)
     int tiles_x = 0, tiles_y = 0;   // x-y tiles covering the plane
     int zchunks = 0;                // z-ranges per tile column
     int zlen = 0;                   // planes per z-range (last one may be shorter)
