@@ -21,7 +21,8 @@
 // on the plane k = 0; above it p is the odd image p(-m) = -p(m) and v_z (at
 // the half points) the even image v_z(-m) = v_z(m - 1); no top layer.
 //
-// Kernels.  Both step kernels give a CTA a 64 x 16 x-y tile and a range of
+// Kernels.  Both step kernels give a CTA an x-y tile (64 x 16 or another of
+// kTmaShapes; the numbers below are its) and a range of
 // planes; one elected thread streams planes into shared-memory rings with
 // cp.async.bulk.tensor (mbarrier per slot, transaction bytes, bounded waits),
 // the tensor maps' zero fill being the "zero outside the grid" reading:
@@ -91,10 +92,33 @@ struct VdArgs {
 
 namespace {
 
-constexpr int TX = 64, TY = 16, RY = 2, NWARP = TY / RY, NT = NWARP * 32;
-constexpr int PHX = TX + 2 * kRadius, PHY = TY + 2 * kRadius;   // 72 x 24: p with its halo
-constexpr int BX = TX + 4, BY = TY + 1;                         // 68 x 17: b with +1 halo (16-byte rows)
-constexpr int OWN = TX * TY;
+constexpr int RY = 2;   // rows per thread (2 x 2 points)
+constexpr int VNSP = 8;    // p halo slots (8-plane window from the queue's leading plane to the centre + prefetch)
+constexpr int VNSO = 3;    // own velocity slots
+constexpr int VNSB = 4;    // buoyancy slots (planes k and k + 1 resident)
+constexpr int PNSC = 3;    // centre slots: vx (x halo), vy (y halo), p, dt K
+constexpr int PNSZ = 8;    // vz own slots feeding the queue
+
+// One tile shape (kTmaShapes) of both kernels.
+template <int SH>
+struct VdShape {
+    static constexpr int TX = kTmaShapes[SH].tx, TY = kTmaShapes[SH].ty;
+    static constexpr int LX = TX / 2, NT = LX * (TY / RY);
+    static constexpr int PHX = kTmaShapes[SH].pitch, PHY = TY + 2 * kRadius;   // p with its halo; vx rows too
+    static constexpr int BX = TX + 4, BY = TY + 1;                             // b with +1 halo (16-byte rows)
+    static constexpr int OWN = TX * TY;
+    // slots start on 128-byte boundaries
+    static constexpr int pad(int n) { return (n + 31) / 32 * 32; }
+    static constexpr int SLOT_P = pad(PHX * PHY), OWN_S = pad(OWN), SLOT_O = 3 * OWN_S, BOX_B = BX * BY,
+                         SLOT_B = pad(BOX_B);
+    static constexpr int V_SMEM = (VNSP * SLOT_P + VNSO * SLOT_O + VNSB * SLOT_B) * 4 + (VNSP + VNSO) * 8 + 16;
+    static constexpr int P_VX = pad(PHX * TY), P_VY = pad(TX * PHY);
+    static constexpr int SLOT_C = P_VX + P_VY + 2 * OWN_S;
+    static constexpr int P_SMEM = (PNSC * SLOT_C + PNSZ * OWN_S) * 4 + (PNSC + PNSZ) * 8 + 16;
+    static_assert(V_SMEM <= 113 * 1024 && P_SMEM <= 113 * 1024, "two CTAs per SM");
+    static_assert(NT <= 256, "128 registers per thread");
+};
+static_assert(VNSB == VNSO + 1, "b of plane t + VNSO + 1 takes the slot of plane t");
 
 // ---------------------------------------------------------------------------
 // Per-point arithmetic shared by the TMA and plain kernels.
@@ -243,42 +267,26 @@ __global__ void vd_pressure_simple(VdArgs a) {
 // TMA kernels.
 // ---------------------------------------------------------------------------
 
-constexpr int VNSP = 8;    // p halo slots (8-plane window from the queue's leading plane to the centre + prefetch)
-constexpr int VNSO = 3;    // own velocity slots
-constexpr int VNSB = 4;    // buoyancy slots (planes k and k + 1 resident)
-// slots start on 128-byte boundaries (the b box, 68 x 17 floats, is padded)
-constexpr int V_SLOT_P = PHX * PHY, V_SLOT_O = 3 * OWN, V_BOX_B = BX * BY, V_SLOT_B = (V_BOX_B + 31) / 32 * 32;
-static_assert(VNSB == VNSO + 1, "b of plane t + VNSO + 1 takes the slot of plane t");
-static_assert(V_SLOT_P % 32 == 0 && V_SLOT_O % 32 == 0, "128-byte slots");
-constexpr int V_SMEM = (VNSP * V_SLOT_P + VNSO * V_SLOT_O + VNSB * V_SLOT_B) * 4 + (VNSP + VNSO) * 8 + 16;
-
-constexpr int PNSC = 3;    // centre slots: vx (72 x 16), vy (64 x 24), p, dt K (64 x 16)
-constexpr int PNSZ = 8;    // vz own slots feeding the queue
-constexpr int P_VX = PHX * TY, P_VY = TX * PHY;
-constexpr int P_SLOT_C = P_VX + P_VY + 2 * OWN;
-constexpr int P_SMEM = (PNSC * P_SLOT_C + PNSZ * OWN) * 4 + (PNSC + PNSZ) * 8 + 16;
-
-static_assert(V_SMEM <= 113 * 1024 && P_SMEM <= 113 * 1024, "two CTAs per SM");
-
 struct VdMaps {
-    CUtensorMap p_halo;          // p, 72 x 24 box
-    CUtensorMap own[3];          // vx, vy, vz, 64 x 16 box
-    CUtensorMap b_box;           // dt / rho, 68 x 17 box
-    CUtensorMap vx_halo;         // vx, 72 x 16 box
-    CUtensorMap vy_halo;         // vy, 64 x 24 box
-    CUtensorMap p_own, k_own;    // p, dt K, 64 x 16 box
+    CUtensorMap p_halo;          // p, PHX x PHY box
+    CUtensorMap own[3];          // vx, vy, vz, TX x TY box
+    CUtensorMap b_box;           // dt / rho, BX x BY box
+    CUtensorMap vx_halo;         // vx, PHX x TY box
+    CUtensorMap vy_halo;         // vy, TX x PHY box
+    CUtensorMap p_own, k_own;    // p, dt K, TX x TY box
 };
 
 struct VdGeom {
     int tiles_x, tiles_y, zchunks, zlen;
 };
 
+template <class S>
 __device__ __forceinline__ void tile_of(const VdGeom &g, int bid, int nz, int &x0, int &y0, int &z0, int &T) {
     const int tx = bid % g.tiles_x;
     const int ty = (bid / g.tiles_x) % g.tiles_y;
     const int ch = bid / (g.tiles_x * g.tiles_y);
-    x0 = tx * TX;
-    y0 = ty * TY;
+    x0 = tx * S::TX;
+    y0 = ty * S::TY;
     z0 = ch * g.zlen;
     T = min(nz - z0, g.zlen);
 }
@@ -406,20 +414,21 @@ struct VCtx {
     float *ring_p, *ring_o, *ring_b;
     uint64_t *bar_p, *bar_o;
     int *abort_flag;
-    int x0, y0, z0, T, lane, warp, xl, x;
+    int x0, y0, z0, T, py, xl, x;
     float2 egx, ehx;       // eps at this thread's two columns (grid, half points)
     float egy[RY], ehy[RY];
     bool lay_xy[RY];       // tile columns or this row pair touch an x or y layer (half points included)
     bool in0, in1;         // columns x, x+1 inside the grid
 };
 
+template <class S>
 __device__ __forceinline__ void v_read_q(const VCtx &c, int seq, float2 (&dst)[RY]) {
-    const float *base = c.ring_p + (seq % VNSP) * V_SLOT_P + (kRadius + RY * c.warp) * PHX + kRadius + c.xl;
+    const float *base = c.ring_p + (seq % VNSP) * S::SLOT_P + (kRadius + RY * c.py) * S::PHX + kRadius + c.xl;
 #pragma unroll
-    for (int r = 0; r < RY; ++r) dst[r] = *reinterpret_cast<const float2 *>(base + r * PHX);
+    for (int r = 0; r < RY; ++r) dst[r] = *reinterpret_cast<const float2 *>(base + r * S::PHX);
 }
 
-template <int J, bool C>
+template <class S, int J, bool C>
 __device__ __forceinline__ bool v_plane(const VdArgs &a, const VCtx &c, int t, float2 (&q)[kVQ][RY], Memory &m) {
     const int k = c.z0 + t;
     float gz = 0.0f, bz_ = 0.0f, gz1 = 0.0f;   // CPML of the z axis on this plane and the next of the range
@@ -431,11 +440,11 @@ __device__ __forceinline__ bool v_plane(const VdArgs &a, const VCtx &c, int t, f
     if (!(mbar_wait(&c.bar_p[(t + 7) % VNSP], ((t + 7) / VNSP) & 1, c.abort_flag, a.err) &&
           mbar_wait(&c.bar_o[t % VNSO], (t / VNSO) & 1, c.abort_flag, a.err)))
         return false;
-    v_read_q(c, t + 7, q[vq(J, 7)]);
-    const float *ctr = c.ring_p + ((t + 3) % VNSP) * V_SLOT_P;
-    const float *own = c.ring_o + (t % VNSO) * V_SLOT_O;
-    const float *bk = c.ring_b + (t % VNSB) * V_SLOT_B;
-    const float *bk1 = c.ring_b + ((t + 1) % VNSB) * V_SLOT_B;
+    v_read_q<S>(c, t + 7, q[vq(J, 7)]);
+    const float *ctr = c.ring_p + ((t + 3) % VNSP) * S::SLOT_P;
+    const float *own = c.ring_o + (t % VNSO) * S::SLOT_O;
+    const float *bk = c.ring_b + (t % VNSB) * S::SLOT_B;
+    const float *bk1 = c.ring_b + ((t + 1) % VNSB) * S::SLOT_B;
     const bool zl = !C && (k < a.nbl || k >= a.nz - 1 - a.nbl);
     const float egz = C ? 0.0f : a.eg[2][k], ehz = C ? 0.0f : a.eh[2][k];
     const bool zin = k + 1 < a.nz;
@@ -443,13 +452,13 @@ __device__ __forceinline__ bool v_plane(const VdArgs &a, const VCtx &c, int t, f
     float2 yc[RY + 2 * kRadius - 1];
 #pragma unroll
     for (int i = 0; i < RY + 2 * kRadius - 1; ++i)
-        yc[i] = *reinterpret_cast<const float2 *>(ctr + (RY * c.warp + 1 + i) * PHX + kRadius + c.xl);
+        yc[i] = *reinterpret_cast<const float2 *>(ctr + (RY * c.py + 1 + i) * S::PHX + kRadius + c.xl);
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
-        const int yl = RY * c.warp + r, y = c.y0 + yl;
+        const int yl = RY * c.py + r, y = c.y0 + yl;
         // x neighbours: columns xl .. xl+9 of row yl+4 as pairs xa[j] = (col 2j, col 2j+1)
         float2 xa[5];
-        const float *row = ctr + (yl + kRadius) * PHX + c.xl;
+        const float *row = ctr + (yl + kRadius) * S::PHX + c.xl;
 #pragma unroll
         for (int j = 0; j < 5; ++j) xa[j] = *reinterpret_cast<const float2 *>(row + 2 * j);
         // D+_x: point c uses cols (5+c, 4+c), (6+c, 3+c), (7+c, 2+c), (8+c, 1+c)
@@ -462,19 +471,19 @@ __device__ __forceinline__ bool v_plane(const VdArgs &a, const VCtx &c, int t, f
         const float2 dz = stag_diff2(a.w[2], q[vq(J, 4)][r], q[vq(J, 3)][r], q[vq(J, 5)][r], q[vq(J, 2)][r],
                                      q[vq(J, 6)][r], q[vq(J, 1)][r], q[vq(J, 7)][r], q[vq(J, 0)][r]);
         // dt b at the half points
-        const float *brow = bk + yl * BX + c.xl;
+        const float *brow = bk + yl * S::BX + c.xl;
         const float2 b01 = *reinterpret_cast<const float2 *>(brow);
         const float b2 = brow[2];
-        const float2 bn = *reinterpret_cast<const float2 *>(brow + BX);
-        const float2 bz = *reinterpret_cast<const float2 *>(bk1 + yl * BX + c.xl);
+        const float2 bn = *reinterpret_cast<const float2 *>(brow + S::BX);
+        const float2 bz = *reinterpret_cast<const float2 *>(bk1 + yl * S::BX + c.xl);
         const bool yin = y + 1 < a.ny;
         const float2 bhx = half_b2(b01, make_float2(b01.y, b2), c.x + 1 < a.nx, c.x + 2 < a.nx);
         const float2 bhy = half_b2(b01, bn, yin, yin);
         const float2 bhz = half_b2(b01, bz, zin, zin);
-        const float *orow = own + yl * TX + c.xl;
+        const float *orow = own + yl * S::TX + c.xl;
         const float2 vx = *reinterpret_cast<const float2 *>(orow);
-        const float2 vy = *reinterpret_cast<const float2 *>(orow + OWN);
-        const float2 vz = *reinterpret_cast<const float2 *>(orow + 2 * OWN);
+        const float2 vy = *reinterpret_cast<const float2 *>(orow + S::OWN_S);
+        const float2 vz = *reinterpret_cast<const float2 *>(orow + 2 * S::OWN_S);
         const bool in0 = c.in0 && y < a.ny, in1 = c.in1 && y < a.ny;
         const long long o = (long long)k * a.plane + (long long)y * a.nxp + c.x;
         float2 nx_, ny_, nz_;
@@ -504,21 +513,20 @@ __device__ __forceinline__ bool v_plane(const VdArgs &a, const VCtx &c, int t, f
     return true;
 }
 
-template <bool C>
-__global__ void __launch_bounds__(NT, 2)
+template <class S, bool C>
+__global__ void __launch_bounds__(S::NT, 2)
     vd_velocity_tma(const __grid_constant__ VdArgs a, const __grid_constant__ VdMaps maps, VdGeom g) {
     extern __shared__ __align__(128) unsigned char smem[];
     VCtx c;
     c.ring_p = reinterpret_cast<float *>(smem);
-    c.ring_o = c.ring_p + VNSP * V_SLOT_P;
-    c.ring_b = c.ring_o + VNSO * V_SLOT_O;
-    c.bar_p = reinterpret_cast<uint64_t *>(c.ring_b + VNSB * V_SLOT_B);
+    c.ring_o = c.ring_p + VNSP * S::SLOT_P;
+    c.ring_b = c.ring_o + VNSO * S::SLOT_O;
+    c.bar_p = reinterpret_cast<uint64_t *>(c.ring_b + VNSB * S::SLOT_B);
     c.bar_o = c.bar_p + VNSP;
     c.abort_flag = reinterpret_cast<int *>(c.bar_o + VNSO);
     const int tid = threadIdx.x;
-    c.lane = tid & 31;
-    c.warp = tid >> 5;
-    tile_of(g, blockIdx.x, a.nz, c.x0, c.y0, c.z0, c.T);
+    c.py = tid / S::LX;
+    tile_of<S>(g, blockIdx.x, a.nz, c.x0, c.y0, c.z0, c.T);
     const int x0 = c.x0, y0 = c.y0, z0 = c.z0, T = c.T;
     const int nseq_p = T + 2 * kRadius - 1;   // p planes z0-3 .. z0+T+3
     int hi_p = 0, hi_o = 0;                   // sequences issued per ring (elected thread only)
@@ -527,20 +535,20 @@ __global__ void __launch_bounds__(NT, 2)
         const int s = seq % VNSP;
         int z = z0 - (kRadius - 1) + seq;
         if (a.fs && z < 0) z = -z;   // plane -m holds the odd image of plane m (negated in the queue)
-        mbar_expect_tx(&c.bar_p[s], V_SLOT_P * 4);
-        tma_load_3d(c.ring_p + s * V_SLOT_P, &maps.p_halo, x0 - kRadius, y0 - kRadius, z, &c.bar_p[s]);
+        mbar_expect_tx(&c.bar_p[s], S::PHX * S::PHY * 4);
+        tma_load_3d(c.ring_p + s * S::SLOT_P, &maps.p_halo, x0 - kRadius, y0 - kRadius, z, &c.bar_p[s]);
         hi_p = seq + 1;
     };
     // own velocities of plane z0 + seq and, on the same barrier, b of the plane after it (the
     // first also b of z0): what step seq needs besides p, so a plane costs two waits
     auto issue_o = [&](int seq) {
         const int s = seq % VNSO;
-        mbar_expect_tx(&c.bar_o[s], (V_SLOT_O + (seq == 0 ? 2 : 1) * V_BOX_B) * 4);
+        mbar_expect_tx(&c.bar_o[s], (3 * S::OWN + (seq == 0 ? 2 : 1) * S::BOX_B) * 4);
 #pragma unroll
         for (int f = 0; f < 3; ++f)
-            tma_load_3d(c.ring_o + s * V_SLOT_O + f * OWN, &maps.own[f], x0, y0, z0 + seq, &c.bar_o[s]);
+            tma_load_3d(c.ring_o + s * S::SLOT_O + f * S::OWN_S, &maps.own[f], x0, y0, z0 + seq, &c.bar_o[s]);
         for (int q = seq == 0 ? 0 : seq + 1; q <= seq + 1; ++q)
-            tma_load_3d(c.ring_b + q % VNSB * V_SLOT_B, &maps.b_box, x0, y0, z0 + q, &c.bar_o[s]);
+            tma_load_3d(c.ring_b + q % VNSB * S::SLOT_B, &maps.b_box, x0, y0, z0 + q, &c.bar_o[s]);
         hi_o = seq + 1;
     };
 
@@ -548,7 +556,7 @@ __global__ void __launch_bounds__(NT, 2)
     // Receivers of the previous step (p^n, read-only in this kernel), one per thread of the grid and
     // more only where there are more: the offset is loaded here, the value after the wait, and it is
     // stored after the plane loop, so the two dependent loads keep nobody waiting.
-    const int r0 = blockIdx.x * NT + tid;
+    const int r0 = blockIdx.x * S::NT + tid;
     const bool rec0 = a.traces && r0 < a.nrec;
     const long long rec_off0 = rec0 ? a.rec_off[r0] : 0;
     if (tid == 0) {
@@ -565,28 +573,28 @@ __global__ void __launch_bounds__(NT, 2)
         for (int q = 0; q < VNSP && q < nseq_p; ++q) issue_p(q);
     const float rec_val0 = rec0 ? a.p[rec_off0] : 0.0f;
     if (a.traces)
-        for (int r = r0 + gridDim.x * NT; r < a.nrec; r += gridDim.x * NT) a.traces[r] = a.p[a.rec_off[r]];
+        for (int r = r0 + gridDim.x * S::NT; r < a.nrec; r += gridDim.x * S::NT) a.traces[r] = a.p[a.rec_off[r]];
     __syncthreads();
     if (T <= 0) return;
 
-    c.xl = 2 * c.lane;
+    c.xl = 2 * (tid % S::LX);
     c.x = x0 + c.xl;
     c.in0 = c.x < a.nx;
     c.in1 = c.x + 1 < a.nx;
     c.egx = C ? bc2(0.0f) : make_float2(a.eg[0][zero_clip(c.x, a.nx)], a.eg[0][zero_clip(c.x + 1, a.nx)]);
     c.ehx = C ? bc2(0.0f) : make_float2(a.eh[0][zero_clip(c.x, a.nx)], a.eh[0][zero_clip(c.x + 1, a.nx)]);
     // the half point after the last inner index (n - 1 - nbl) already lies in the layer
-    const bool lay_x = x0 < a.nbl || x0 + TX - 1 >= a.nx - 1 - a.nbl;
+    const bool lay_x = x0 < a.nbl || x0 + S::TX - 1 >= a.nx - 1 - a.nbl;
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
-        const int y = y0 + RY * c.warp + r, yi = zero_clip(y, a.ny);
+        const int y = y0 + RY * c.py + r, yi = zero_clip(y, a.ny);
         c.egy[r] = C ? 0.0f : a.eg[1][yi];
         c.ehy[r] = C ? 0.0f : a.eh[1][yi];
         c.lay_xy[r] = lay_x || y < a.nbl || y >= a.ny - 1 - a.nbl;
     }
 
     Memory m;
-    if (C) memory_init(m, a, a.Gh, a.Bh, a.psi, c.x, y0 + RY * c.warp, z0);
+    if (C) memory_init(m, a, a.Gh, a.Bh, a.psi, c.x, y0 + RY * c.py, z0);
     float2 q[kVQ][RY];
     bool ok = true;
     for (int s = 0; s < 2 * kRadius - 1 && ok; ++s) {
@@ -594,7 +602,7 @@ __global__ void __launch_bounds__(NT, 2)
         if (ok) {
 #pragma unroll
             for (int i = 0; i < 2 * kRadius - 1; ++i)
-                if (i == s) v_read_q(c, s, q[i]);
+                if (i == s) v_read_q<S>(c, s, q[i]);
         }
     }
     if (a.fs && ok) {   // queue planes above k = 0 (z0-3+i < 0) hold the images: negate
@@ -614,7 +622,7 @@ __global__ void __launch_bounds__(NT, 2)
     // end of step t: the centre tile (seq t+3), the own tile and b plane k are free
 #define VD_VSTEP(J)                                                                   \
     if (t + (J) < T) {                                                                \
-        v_plane<(J), C>(a, c, t + (J), q, m);                                             \
+        v_plane<S, (J), C>(a, c, t + (J), q, m);                                             \
         __syncthreads();                                                              \
         if (*c.abort_flag) break;                                                     \
         if (tid == 0) {                                                               \
@@ -664,20 +672,21 @@ struct PCtx {
     float *ring_c, *ring_z;
     uint64_t *bar_c, *bar_z;
     int *abort_flag;
-    int x0, y0, z0, T, lane, warp, xl, x;
+    int x0, y0, z0, T, py, xl, x;
     float2 egx;
     float egy[RY];
     bool lay_xy[RY];
     bool in0, in1;
 };
 
+template <class S>
 __device__ __forceinline__ void p_read_q(const PCtx &c, int seq, float2 (&dst)[RY]) {
-    const float *base = c.ring_z + (seq % PNSZ) * OWN + RY * c.warp * TX + c.xl;
+    const float *base = c.ring_z + (seq % PNSZ) * S::OWN_S + RY * c.py * S::TX + c.xl;
 #pragma unroll
-    for (int r = 0; r < RY; ++r) dst[r] = *reinterpret_cast<const float2 *>(base + r * TX);
+    for (int r = 0; r < RY; ++r) dst[r] = *reinterpret_cast<const float2 *>(base + r * S::TX);
 }
 
-template <int J, bool C>
+template <class S, int J, bool C>
 __device__ __forceinline__ bool p_plane(const VdArgs &a, const PCtx &c, int t, float2 (&q)[kPQ<C>][RY], Memory &m) {
     const int k = c.z0 + t;
     float gz = 0.0f, bz = 0.0f, gz1 = 0.0f;   // CPML of the z axis on this plane and the next of the range
@@ -689,21 +698,21 @@ __device__ __forceinline__ bool p_plane(const VdArgs &a, const PCtx &c, int t, f
     if (!(mbar_wait(&c.bar_z[(t + 7) % PNSZ], ((t + 7) / PNSZ) & 1, c.abort_flag, a.err) &&
           mbar_wait(&c.bar_c[t % PNSC], (t / PNSC) & 1, c.abort_flag, a.err)))
         return false;
-    p_read_q(c, t + 7, q[pq<C>(J, 7)]);
-    const float *base = c.ring_c + (t % PNSC) * P_SLOT_C;
-    const float *tvx = base, *tvy = base + P_VX, *tp = base + P_VX + P_VY, *tk = tp + OWN;
+    p_read_q<S>(c, t + 7, q[pq<C>(J, 7)]);
+    const float *base = c.ring_c + (t % PNSC) * S::SLOT_C;
+    const float *tvx = base, *tvy = base + S::P_VX, *tp = base + S::P_VX + S::P_VY, *tk = tp + S::OWN_S;
     const bool zl = !C && (k < a.nbl || k > a.nz - 1 - a.nbl);
     const float egz = C ? 0.0f : a.eg[2][k];
     // vy rows 2w .. 2w+8 at columns xl, xl+1
     float2 yc[RY + 2 * kRadius - 1];
 #pragma unroll
     for (int i = 0; i < RY + 2 * kRadius - 1; ++i)
-        yc[i] = *reinterpret_cast<const float2 *>(tvy + (RY * c.warp + i) * TX + c.xl);
+        yc[i] = *reinterpret_cast<const float2 *>(tvy + (RY * c.py + i) * S::TX + c.xl);
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
-        const int yl = RY * c.warp + r, y = c.y0 + yl;
+        const int yl = RY * c.py + r, y = c.y0 + yl;
         float2 xa[5];
-        const float *row = tvx + yl * PHX + c.xl;
+        const float *row = tvx + yl * S::PHX + c.xl;
 #pragma unroll
         for (int j = 0; j < 5; ++j) xa[j] = *reinterpret_cast<const float2 *>(row + 2 * j);
         // D-_x: point c uses cols (4+c, 3+c), (5+c, 2+c), (6+c, 1+c), (7+c, 0+c)
@@ -721,8 +730,8 @@ __device__ __forceinline__ bool p_plane(const VdArgs &a, const PCtx &c, int t, f
             memory_update(m, r, a.phi, o, t + 1 < c.T ? a.plane : 0, gz, bz, gz1, in0, in1, dx, dy, dz);
         }
         const float2 div = __fadd2_rn(__fadd2_rn(dx, dy), dz);
-        const float2 po = *reinterpret_cast<const float2 *>(tp + yl * TX + c.xl);
-        const float2 ko = *reinterpret_cast<const float2 *>(tk + yl * TX + c.xl);
+        const float2 po = *reinterpret_cast<const float2 *>(tp + yl * S::TX + c.xl);
+        const float2 ko = *reinterpret_cast<const float2 *>(tk + yl * S::TX + c.xl);
         float2 pn;
         if (a.fs && k == 0)
             pn = make_float2(0.0f, 0.0f);   // p = 0 on the free surface
@@ -735,20 +744,19 @@ __device__ __forceinline__ bool p_plane(const VdArgs &a, const PCtx &c, int t, f
     return true;
 }
 
-template <bool C>
-__global__ void __launch_bounds__(NT, 2)
+template <class S, bool C>
+__global__ void __launch_bounds__(S::NT, 2)
     vd_pressure_tma(const __grid_constant__ VdArgs a, const __grid_constant__ VdMaps maps, VdGeom g) {
     extern __shared__ __align__(128) unsigned char smem[];
     PCtx c;
     c.ring_c = reinterpret_cast<float *>(smem);
-    c.ring_z = c.ring_c + PNSC * P_SLOT_C;
-    c.bar_c = reinterpret_cast<uint64_t *>(c.ring_z + PNSZ * OWN);
+    c.ring_z = c.ring_c + PNSC * S::SLOT_C;
+    c.bar_c = reinterpret_cast<uint64_t *>(c.ring_z + PNSZ * S::OWN_S);
     c.bar_z = c.bar_c + PNSC;
     c.abort_flag = reinterpret_cast<int *>(c.bar_z + PNSZ);
     const int tid = threadIdx.x;
-    c.lane = tid & 31;
-    c.warp = tid >> 5;
-    tile_of(g, blockIdx.x, a.nz, c.x0, c.y0, c.z0, c.T);
+    c.py = tid / S::LX;
+    tile_of<S>(g, blockIdx.x, a.nz, c.x0, c.y0, c.z0, c.T);
     const int x0 = c.x0, y0 = c.y0, z0 = c.z0, T = c.T;
     const int nseq_z = T + 2 * kRadius - 1;   // vz planes z0-4 .. z0+T+2
     int hi_c = 0, hi_z = 0;                   // sequences issued per ring (elected thread only)
@@ -757,17 +765,17 @@ __global__ void __launch_bounds__(NT, 2)
     // barrier counts the bytes of all four boxes
     auto issue_c_own = [&](int seq) {
         const int s = seq % PNSC;
-        float *base = c.ring_c + s * P_SLOT_C;
-        mbar_expect_tx(&c.bar_c[s], P_SLOT_C * 4);
-        tma_load_3d(base + P_VX + P_VY, &maps.p_own, x0, y0, z0 + seq, &c.bar_c[s]);
-        tma_load_3d(base + P_VX + P_VY + OWN, &maps.k_own, x0, y0, z0 + seq, &c.bar_c[s]);
+        float *base = c.ring_c + s * S::SLOT_C;
+        mbar_expect_tx(&c.bar_c[s], (S::PHX * S::TY + S::TX * S::PHY + 2 * S::OWN) * 4);
+        tma_load_3d(base + S::P_VX + S::P_VY, &maps.p_own, x0, y0, z0 + seq, &c.bar_c[s]);
+        tma_load_3d(base + S::P_VX + S::P_VY + S::OWN_S, &maps.k_own, x0, y0, z0 + seq, &c.bar_c[s]);
         hi_c = seq + 1;
     };
     auto issue_c_vel = [&](int seq) {
         const int s = seq % PNSC;
-        float *base = c.ring_c + s * P_SLOT_C;
+        float *base = c.ring_c + s * S::SLOT_C;
         tma_load_3d(base, &maps.vx_halo, x0 - kRadius, y0, z0 + seq, &c.bar_c[s]);
-        tma_load_3d(base + P_VX, &maps.vy_halo, x0, y0 - kRadius, z0 + seq, &c.bar_c[s]);
+        tma_load_3d(base + S::P_VX, &maps.vy_halo, x0, y0 - kRadius, z0 + seq, &c.bar_c[s]);
     };
     auto issue_c = [&](int seq) {
         issue_c_own(seq);
@@ -777,8 +785,8 @@ __global__ void __launch_bounds__(NT, 2)
         const int s = seq % PNSZ;
         int z = z0 - kRadius + seq;
         if (a.fs && z < 0) z = -z - 1;   // v_z(-m) = v_z(m - 1): the even image across the surface
-        mbar_expect_tx(&c.bar_z[s], OWN * 4);
-        tma_load_3d(c.ring_z + s * OWN, &maps.own[2], x0, y0, z, &c.bar_z[s]);
+        mbar_expect_tx(&c.bar_z[s], S::OWN * 4);
+        tma_load_3d(c.ring_z + s * S::OWN_S, &maps.own[2], x0, y0, z, &c.bar_z[s]);
         hi_z = seq + 1;
     };
 
@@ -787,11 +795,11 @@ __global__ void __launch_bounds__(NT, 2)
         tma_prefetch_map(&maps.vy_halo);
         tma_prefetch_map(&maps.own[2]);
     }
-    // Does source group gi lie in this CTA's tile and planes?  The first NT
+    // Does source group gi lie in this CTA's tile and planes?  The first S::NT
     // groups (all of them, in practice) are looked up here, ahead of use.
     auto source_here = [&](int gi) {
         const int *q = a.grp_ijk + 3 * gi;
-        return q[0] >= x0 && q[0] < x0 + TX && q[1] >= y0 && q[1] < y0 + TY && q[2] >= z0 && q[2] < z0 + T;
+        return q[0] >= x0 && q[0] < x0 + S::TX && q[1] >= y0 && q[1] < y0 + S::TY && q[2] >= z0 && q[2] < z0 + T;
     };
     const bool src0 = tid < a.ngrp && source_here(tid);
     if (tid == 0) {
@@ -812,21 +820,21 @@ __global__ void __launch_bounds__(NT, 2)
     __syncthreads();
     if (T <= 0) return;
 
-    c.xl = 2 * c.lane;
+    c.xl = 2 * (tid % S::LX);
     c.x = x0 + c.xl;
     c.in0 = c.x < a.nx;
     c.in1 = c.x + 1 < a.nx;
     c.egx = C ? bc2(0.0f) : make_float2(a.eg[0][zero_clip(c.x, a.nx)], a.eg[0][zero_clip(c.x + 1, a.nx)]);
-    const bool lay_x = x0 < a.nbl || x0 + TX - 1 > a.nx - 1 - a.nbl;
+    const bool lay_x = x0 < a.nbl || x0 + S::TX - 1 > a.nx - 1 - a.nbl;
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
-        const int y = y0 + RY * c.warp + r;
+        const int y = y0 + RY * c.py + r;
         c.egy[r] = C ? 0.0f : a.eg[1][zero_clip(y, a.ny)];
         c.lay_xy[r] = lay_x || y < a.nbl || y > a.ny - 1 - a.nbl;
     }
 
     Memory m;
-    if (C) memory_init(m, a, a.Gg, a.Bg, a.phi, c.x, y0 + RY * c.warp, z0);
+    if (C) memory_init(m, a, a.Gg, a.Bg, a.phi, c.x, y0 + RY * c.py, z0);
     float2 q[kPQ<C>][RY];
     bool ok = true;
     for (int s = 0; s < 2 * kRadius - 1 && ok; ++s) {
@@ -834,7 +842,7 @@ __global__ void __launch_bounds__(NT, 2)
         if (ok) {
 #pragma unroll
             for (int i = 0; i < 2 * kRadius - 1; ++i)
-                if (i == s) p_read_q(c, s, q[i]);
+                if (i == s) p_read_q<S>(c, s, q[i]);
         }
     }
     __syncthreads();
@@ -845,7 +853,7 @@ __global__ void __launch_bounds__(NT, 2)
     // end of step t: the vz tile read into the queue (seq t+7) and the centre slot are free
 #define VD_PSTEP(J)                                                                   \
     if (t + (J) < T) {                                                                \
-        p_plane<(J), C>(a, c, t + (J), q, m);                                             \
+        p_plane<S, (J), C>(a, c, t + (J), q, m);                                             \
         __syncthreads();                                                              \
         if (*c.abort_flag) break;                                                     \
         if (tid == 0) {                                                               \
@@ -875,8 +883,8 @@ __global__ void __launch_bounds__(NT, 2)
     if (a.ngrp > 0) {
         __syncthreads();
         if (!*c.abort_flag)
-            for (int gi = tid; gi < a.ngrp; gi += NT) {
-                if (gi < NT ? !src0 : !source_here(gi)) continue;
+            for (int gi = tid; gi < a.ngrp; gi += S::NT) {
+                if (gi < S::NT ? !src0 : !source_here(gi)) continue;
                 float *dst = a.p + a.grp_off[gi];
                 float v = *dst;
                 for (int m = a.grp_first[gi]; m < a.grp_first[gi + 1]; ++m) {
@@ -960,6 +968,22 @@ __global__ void vd_source_scale(const float *vel, const float *rho, int nx, int 
 
 int grid_for(long long n, int block) { return (int)std::min<long long>((n + block - 1) / block, 152LL * 32); }
 
+using VdKernel = void (*)(const VdArgs, const VdMaps, VdGeom);
+struct VdKernels {
+    VdKernel velocity[2], pressure[2];   // damping, CPML
+    int nt, v_smem, p_smem;
+};
+template <int SH>
+constexpr VdKernels vd_kernels_of() {
+    using S = VdShape<SH>;
+    return {{vd_velocity_tma<S, false>, vd_velocity_tma<S, true>}, {vd_pressure_tma<S, false>, vd_pressure_tma<S, true>},
+            S::NT, S::V_SMEM, S::P_SMEM};
+}
+const VdKernels &vd_kernels(int shape) {
+    static const VdKernels k[kNumShapes] = {vd_kernels_of<0>(), vd_kernels_of<1>(), vd_kernels_of<2>(), vd_kernels_of<3>()};
+    return k[shape];
+}
+
 // Source groups the pressure kernel adds itself (each CTA scans the list).
 constexpr int kFoldSources = 1024;
 
@@ -1000,6 +1024,7 @@ struct mmod_vd {
     bool tma_ok = false;
     VdMaps maps{};
     VdGeom geom{};
+    int shape = 0;                    // tile shape (kTmaShapes)
     int kernel = MMOD_KERNEL_AUTO;
     int pdl = 1;                      // programmatic dependent launch of the TMA step kernels (us per step
                                       // without / with: 48^3 9.1 / 8.3, 128^3 21.7 / 21.0, 240^3 137.5 / 137.0)
@@ -1129,16 +1154,13 @@ cudaError_t enqueue_vd_step(mmod_vd *h, int n, const float *wav, float *traces_p
     a.pdl = h->pdl;
     if (vd_use_tma(h)) {
         lc.gridDim = dim3(h->geom.tiles_x * h->geom.tiles_y * h->geom.zchunks);
-        lc.blockDim = dim3(NT);
-        lc.dynamicSmemBytes = V_SMEM;
-        if ((e = cudaLaunchKernelEx(&lc, a.cpml ? vd_velocity_tma<true> : vd_velocity_tma<false>, a, h->maps,
-                                    h->geom)) != cudaSuccess)
-            return e;
+        const VdKernels &k = vd_kernels(h->shape);
+        lc.blockDim = dim3(k.nt);
+        lc.dynamicSmemBytes = k.v_smem;
+        if ((e = cudaLaunchKernelEx(&lc, k.velocity[a.cpml], a, h->maps, h->geom)) != cudaSuccess) return e;
         a.traces = nullptr;
-        lc.dynamicSmemBytes = P_SMEM;
-        if ((e = cudaLaunchKernelEx(&lc, a.cpml ? vd_pressure_tma<true> : vd_pressure_tma<false>, a, h->maps,
-                                    h->geom)) != cudaSuccess)
-            return e;
+        lc.dynamicSmemBytes = k.p_smem;
+        if ((e = cudaLaunchKernelEx(&lc, k.pressure[a.cpml], a, h->maps, h->geom)) != cudaSuccess) return e;
     } else {
         const dim3 blk(32, 8, 1), grd((h->cfg.nx + 31) / 32, (h->cfg.ny + 7) / 8, h->cfg.nz);
         vd_velocity_simple<<<grd, blk, 0, s>>>(a);
@@ -1200,26 +1222,48 @@ mmod_status vd_loop(mmod_vd *h, const float *wav, float *tr, cudaStream_t s, lon
     return MMOD_OK;
 }
 
-// Tile decomposition: x-y tiles of 64 x 16, z ranges chosen to minimise
-// waves x (planes per range + 7) over two resident CTAs per SM.
-VdGeom plan_geom(int nx, int ny, int nz, int sms) {
-    VdGeom g{};
-    g.tiles_x = (nx + TX - 1) / TX;
-    g.tiles_y = (ny + TY - 1) / TY;
-    const long long tiles = (long long)g.tiles_x * g.tiles_y, slots = 2LL * std::max(sms, 1);
-    long long best = -1;
-    for (int zc = 1; zc <= nz; ++zc) {
-        const int zlen = (nz + zc - 1) / zc;
-        const int zcount = (nz + zlen - 1) / zlen;
-        const long long waves = (tiles * zcount + slots - 1) / slots;
-        const long long cost = waves * (zlen + 2 * kRadius - 1);
-        if (best < 0 || cost < best) {
-            best = cost;
-            g.zchunks = zcount;
-            g.zlen = zlen;
+// Tile decomposition: for each tile shape the z ranges that minimise waves x
+// (planes per range + 7) over two resident CTAs per SM.  A launch takes about
+// a fixed time per plane of a CTA, so the shape with the fewest waves x planes
+// wins, and of those the one with the fewest CTAs; 64 x 16 gives way on equal
+// planes only to smaller tiles of the same number.  Measured, 64 x 16 against the
+// choice (us per step, damping): 96^3 15.5 / 13.1 (32 x 32), 144^3 36.9 / 31.9 (48 x
+// 20), 160^3 41.0 / 35.7 (32 x 32), 200^3 96.9 / 88.4 (40 x 24), 240^3 136.3 / 134.3 (48
+// x 20), 77 x 210 x 64 23.0 / 17.2 (40 x 24); on equal planes and other counts it is
+// the better one (112^3 19.8 against 20.7, 100 x 220 x 180 47.7 against 48.2).
+VdGeom plan_geom(int nx, int ny, int nz, int sms, int *shape) {
+    VdGeom best_g{};
+    long long best_load = 0, best_ctas = 0;
+    const long long slots = 2LL * std::max(sms, 1);
+    for (int sh = 0; sh < kNumShapes; ++sh) {
+        const TmaShape &t = kTmaShapes[sh];
+        VdGeom g{};
+        g.tiles_x = (nx + t.tx - 1) / t.tx;
+        g.tiles_y = (ny + t.ty - 1) / t.ty;
+        const long long tiles = (long long)g.tiles_x * g.tiles_y;
+        long long best = -1;
+        for (int zc = 1; zc <= nz; ++zc) {
+            const int zlen = (nz + zc - 1) / zc;
+            const int zcount = (nz + zlen - 1) / zlen;
+            const long long waves = (tiles * zcount + slots - 1) / slots;
+            const long long cost = waves * (zlen + 2 * kRadius - 1);
+            if (best < 0 || cost < best) {
+                best = cost;
+                g.zchunks = zcount;
+                g.zlen = zlen;
+            }
+        }
+        const long long ctas = tiles * g.zchunks, load = (ctas + slots - 1) / slots * g.zlen;
+        const bool tie = load == best_load && (*shape == 0 ? ctas == best_ctas && t.tx * t.ty < kTmaShapes[0].tx * kTmaShapes[0].ty
+                                                           : ctas < best_ctas);
+        if (sh == 0 || load < best_load || tie) {
+            best_load = load;
+            best_ctas = ctas;
+            best_g = g;
+            *shape = sh;
         }
     }
-    return g;
+    return best_g;
 }
 
 void vd_free(mmod_vd *h) {
@@ -1393,20 +1437,23 @@ MMOD_API mmod_status mmod_vd_create(const mmod_config *cfg, int device, mmod_vd 
     // TMA plan: tensor maps of every operand, two CTAs per SM
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    h->geom = plan_geom(c.nx, c.ny, c.nz, sms);
+    h->geom = plan_geom(c.nx, c.ny, c.nz, sms, &h->shape);
     h->geom_plan = h->geom;
     bool ok = true;
-    for (const void *f : {(const void *)vd_velocity_tma<false>, (const void *)vd_velocity_tma<true>})
-        ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, V_SMEM) == cudaSuccess;
-    for (const void *f : {(const void *)vd_pressure_tma<false>, (const void *)vd_pressure_tma<true>})
-        ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM) == cudaSuccess;
-    ok = ok && encode_box(&h->maps.p_halo, h->p, c.nx, c.ny, c.nz, h->nxp, PHX, PHY);
-    for (int ax = 0; ax < 3; ++ax) ok = ok && encode_box(&h->maps.own[ax], h->v[ax], c.nx, c.ny, c.nz, h->nxp, TX, TY);
-    ok = ok && encode_box(&h->maps.b_box, h->bd, c.nx, c.ny, c.nz, h->nxp, BX, BY);
-    ok = ok && encode_box(&h->maps.vx_halo, h->v[0], c.nx, c.ny, c.nz, h->nxp, PHX, TY);
-    ok = ok && encode_box(&h->maps.vy_halo, h->v[1], c.nx, c.ny, c.nz, h->nxp, TX, PHY);
-    ok = ok && encode_box(&h->maps.p_own, h->p, c.nx, c.ny, c.nz, h->nxp, TX, TY);
-    ok = ok && encode_box(&h->maps.k_own, h->kd, c.nx, c.ny, c.nz, h->nxp, TX, TY);
+    const VdKernels &kk = vd_kernels(h->shape);
+    ok = ok && cudaFuncSetAttribute((const void *)kk.velocity[cpml], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    kk.v_smem) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute((const void *)kk.pressure[cpml], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    kk.p_smem) == cudaSuccess;
+    const TmaShape &t = kTmaShapes[h->shape];
+    const int hy = t.ty + 2 * kRadius;
+    ok = ok && encode_box(&h->maps.p_halo, h->p, c.nx, c.ny, c.nz, h->nxp, t.pitch, hy);
+    for (int ax = 0; ax < 3; ++ax) ok = ok && encode_box(&h->maps.own[ax], h->v[ax], c.nx, c.ny, c.nz, h->nxp, t.tx, t.ty);
+    ok = ok && encode_box(&h->maps.b_box, h->bd, c.nx, c.ny, c.nz, h->nxp, t.tx + 4, t.ty + 1);
+    ok = ok && encode_box(&h->maps.vx_halo, h->v[0], c.nx, c.ny, c.nz, h->nxp, t.pitch, t.ty);
+    ok = ok && encode_box(&h->maps.vy_halo, h->v[1], c.nx, c.ny, c.nz, h->nxp, t.tx, hy);
+    ok = ok && encode_box(&h->maps.p_own, h->p, c.nx, c.ny, c.nz, h->nxp, t.tx, t.ty);
+    ok = ok && encode_box(&h->maps.k_own, h->kd, c.nx, c.ny, c.nz, h->nxp, t.tx, t.ty);
     cudaGetLastError();
     h->tma_ok = ok;
 #undef VD_CREATE
@@ -1601,6 +1648,6 @@ MMOD_API mmod_status mmod_vd_get_plan(const mmod_vd *h, int *out6) {
     out6[2] = h->geom.zchunks;
     out6[3] = h->geom.zlen;
     out6[4] = h->geom.tiles_x * h->geom.tiles_y * h->geom.zchunks;
-    out6[5] = NT;
+    out6[5] = vd_kernels(h->shape).nt;
     return h->tma_ok ? MMOD_OK : MMOD_ERR_UNSUPPORTED;
 }
