@@ -81,6 +81,58 @@ __device__ __forceinline__ void inject_point_at(const StepArgs &a, float *uout, 
 
 __device__ __forceinline__ void inject_point(const StepArgs &a, int p) { inject_point_at(a, a.uout, a.n, p); }
 
+// Injection point p ahead of time: everything but the wavefield value.
+// sw = scale * w[n] of its first source, r its damping factor; count sources
+// (0: p is past hi).
+struct SourcePoint {
+    long long off = 0;
+    float sw = 0.0f, r = 0.0f;
+    int count = 0;
+};
+
+__device__ __forceinline__ SourcePoint source_point(const StepArgs &a, int n, int p, int hi) {
+    SourcePoint q;
+    if (p < hi) {
+        const int s0 = __ldg(a.inj.pt_first + p), row = __ldg(a.inj.src_row + s0);
+        q.count = __ldg(a.inj.pt_first + p + 1) - s0;
+        q.off = __ldg(a.inj.pt_off + p);
+        q.r = damp_factor(__fadd_rn(__fadd_rn(__ldg(a.ex + __ldg(a.inj.pt_i + p)), __ldg(a.ey + __ldg(a.inj.pt_j + p))),
+                                    __ldg(a.ez + __ldg(a.inj.pt_k + p))));
+        q.sw = __fmul_rn(__ldg(a.inj.src_scale + row),
+                         __ldg(a.wavelet + (long long)row * a.wrs + (long long)n * a.wcs));
+    }
+    return q;
+}
+
+// Point p's table entries and wavelet sample into L2 (a CTA of the adjoint can
+// hold a thousand points: the ones past a thread's first are looked up at the
+// end, and every step's residual row is new).
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void prefetch_source_point(const StepArgs &a, int n, int p) {
+    const int row = __ldg(a.inj.src_row + __ldg(a.inj.pt_first + p));
+    prefetch_l2(a.inj.pt_i + p);
+    prefetch_l2(a.inj.pt_j + p);
+    prefetch_l2(a.inj.pt_k + p);
+    prefetch_l2(a.inj.pt_off + p);
+    prefetch_l2(a.inj.src_scale + row);
+    prefetch_l2(a.wavelet + (long long)row * a.wrs + (long long)n * a.wcs);
+}
+
+// inject_point_at of point p from its SourcePoint (the same operations: add_source is fma(scale * w, r, u)).
+__device__ __forceinline__ void inject_source_point(const StepArgs &a, float *uout, int n, int p, const SourcePoint &q) {
+    if (q.count <= 0) return;
+    float x = __fmaf_rn(q.sw, q.r, uout[q.off]);
+    if (q.count > 1) {
+        const int s0 = __ldg(a.inj.pt_first + p);
+        for (int s = s0 + 1; s < s0 + q.count; ++s) {
+            const int row = __ldg(a.inj.src_row + s);
+            x = add_source(x, __ldg(a.inj.src_scale + row),
+                           __ldg(a.wavelet + (long long)row * a.wrs + (long long)n * a.wcs), q.r);
+        }
+    }
+    uout[q.off] = x;
+}
+
 // The same for injection points [lo, hi), thread t of nthreads: each thread
 // takes up to four points at a time and issues the table, profile, wavefield
 // and wavelet loads of all four before it applies any, so the dependent loads

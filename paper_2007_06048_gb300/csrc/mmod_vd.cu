@@ -795,13 +795,29 @@ __global__ void __launch_bounds__(S::NT, 2)
         tma_prefetch_map(&maps.vy_halo);
         tma_prefetch_map(&maps.own[2]);
     }
-    // Does source group gi lie in this CTA's tile and planes?  The first S::NT
-    // groups (all of them, in practice) are looked up here, ahead of use.
+    // Does source group gi lie in this CTA's tile and planes?
     auto source_here = [&](int gi) {
         const int *q = a.grp_ijk + 3 * gi;
         return q[0] >= x0 && q[0] < x0 + S::TX && q[1] >= y0 && q[1] < y0 + S::TY && q[2] >= z0 && q[2] < z0 + T;
     };
-    const bool src0 = tid < a.ngrp && source_here(tid);
+    // The first groups (all of them, in practice) are looked up here, down to
+    // the scale and sample of their first source: a chain of dependent loads
+    // that the whole grid would wait for at the end.  One group per thread past
+    // warp 0, whose first thread issues the copies.
+    constexpr int kAhead = S::NT - 32;
+    const int g0 = tid - 32;
+    const bool src0 = g0 >= 0 && g0 < a.ngrp && source_here(g0);
+    long long src_off = 0;
+    int src_first = 0, src_last = 0;
+    float src_s = 0.0f, src_w = 0.0f;
+    if (src0) {
+        src_off = a.grp_off[g0];
+        src_first = a.grp_first[g0];
+        src_last = a.grp_first[g0 + 1];
+        const int sid = a.src_id[src_first];
+        src_s = a.src_scale[sid];
+        src_w = a.wavelet[(long long)sid * a.nt + a.n];
+    }
     if (tid == 0) {
         for (int s = 0; s < PNSC; ++s) mbar_init(&c.bar_c[s], 1);
         for (int s = 0; s < PNSZ; ++s) mbar_init(&c.bar_z[s], 1);
@@ -882,17 +898,21 @@ __global__ void __launch_bounds__(S::NT, 2)
     // sources in their order: the separate injection kernel's operations.
     if (a.ngrp > 0) {
         __syncthreads();
-        if (!*c.abort_flag)
-            for (int gi = tid; gi < a.ngrp; gi += S::NT) {
-                if (gi < S::NT ? !src0 : !source_here(gi)) continue;
-                float *dst = a.p + a.grp_off[gi];
-                float v = *dst;
-                for (int m = a.grp_first[gi]; m < a.grp_first[gi + 1]; ++m) {
-                    const int sid = a.src_id[m];
-                    v = __fmaf_rn(a.src_scale[sid], a.wavelet[(long long)sid * a.nt + a.n], v);
-                }
-                *dst = v;
+        auto add = [&](float v, int m, int last) {
+            for (; m < last; ++m) {
+                const int sid = a.src_id[m];
+                v = __fmaf_rn(a.src_scale[sid], a.wavelet[(long long)sid * a.nt + a.n], v);
             }
+            return v;
+        };
+        if (!*c.abort_flag) {
+            if (src0) a.p[src_off] = add(__fmaf_rn(src_s, src_w, a.p[src_off]), src_first + 1, src_last);
+            for (int gi = kAhead + tid; gi < a.ngrp; gi += S::NT)
+                if (source_here(gi)) {
+                    float *dst = a.p + a.grp_off[gi];
+                    *dst = add(*dst, a.grp_first[gi], a.grp_first[gi + 1]);
+                }
+        }
     }
     pdl_release();
     if (*c.abort_flag && tid == 0) {

@@ -197,6 +197,21 @@ __device__ __forceinline__ void step_staged_body(const StepArgs &a, const StepVa
         inj_lo = __ldg(a.inj.tile_start + bucket);
         inj_hi = __ldg(a.inj.tile_start + bucket + T);
     }
+    // The first injection point of each thread past warp 0 (whose first thread
+    // issues the copies), down to scale * w[n] and the damping factor: a chain
+    // of four dependent loads, which at the end of the kernel made the whole grid
+    // wait for the few CTAs that hold sources, and here runs while the previous
+    // step drains or the first planes arrive.  What is left for the end is one
+    // read-modify-write.  64^3 x 100 steps: 372 -> 325 us; gradient 200^3 41.0 ->
+    // 40.0 ms.
+    constexpr int kAhead = S::NT - 32;   // points looked up ahead
+    SourcePoint src;
+    if constexpr (MODE != kImage) {
+        if (tid >= 32) {
+            src = source_point(a, v.n, inj_lo + tid - 32, inj_hi);
+            for (int p = inj_lo + kAhead + tid - 32; p < inj_hi; p += kAhead) prefetch_source_point(a, v.n, p);
+        }
+    }
     // Receivers of the previous step (u^n, read-only during this launch), one
     // per thread of the grid and more only where there are more: the offset is
     // loaded here, the value once u^n is there, and it is stored after the plane
@@ -363,7 +378,8 @@ __device__ __forceinline__ void step_staged_body(const StepArgs &a, const StepVa
             v.uout[img_off] = __fmaf_rn(a.c[img_off], gv, img_acc);
         }
     } else if (!*c.abort_flag && inj_lo < inj_hi) {
-        inject_points(a, v.uout, v.n, inj_lo, inj_hi, tid, S::NT);
+        inject_source_point(a, v.uout, v.n, inj_lo + tid - 32, src);
+        inject_points(a, v.uout, v.n, inj_lo + kAhead, inj_hi, tid, S::NT);
         if constexpr (MODE == kStepG) inject_g_points(a, v.n, inj_lo, inj_hi, tid, S::NT);
     }
     // After a give-up, wait (bounded) for the copies this CTA still has in
