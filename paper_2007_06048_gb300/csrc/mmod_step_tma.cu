@@ -837,7 +837,11 @@ bool make_tma_plan(const mmod_config &cfg, TmaPlan plans[]) {
             return false;
         }
         const long long slots = (long long)sms * occ;
-        // the z split that minimises (waves) x (planes per CTA + halo cost)
+        // the z split that minimises (waves) x (planes per CTA + halo cost).  A
+        // CTA with an SM to itself takes 0.6 of the time per plane that two
+        // sharing one take (us per step: 64^3, 128 CTAs of 2 planes 2.79, 256 of 1
+        // 2.95; 56^3 2.86 / 3.45; 72^3 in 40 x 24 tiles, 144 of 3 planes 3.32, 216 of
+        // 2 3.75; but 96^3 in 32 x 32, 144 of 6 4.96, 288 of 3 4.42).
         int best_c = 1;
         double best = 1e300;
         for (int zc = 1; zc <= cfg.nz; ++zc) {
@@ -846,7 +850,7 @@ bool make_tma_plan(const mmod_config &cfg, TmaPlan plans[]) {
             const long long ctas = tiles * zc;
             if (ctas > (1LL << 31) - 1) break;
             const double waves = (double)((ctas + slots - 1) / slots);
-            const double cost = waves * (zlen + 2.0);
+            const double cost = ctas <= sms ? 0.6 * zlen + 1.75 : waves * (zlen + 2.0);
             if (cost < best - 1e-9) {
                 best = cost;
                 best_c = zc;
@@ -877,7 +881,8 @@ bool make_tma_plan(const mmod_config &cfg, TmaPlan plans[]) {
 // to a third of it (200^3: 4 x 13 tiles of 40 planes against 5 x 9 tiles of 40 x
 // 24 with 34 planes).  The cost below was fitted to 4 shapes x 28 grids from
 // 64^3 to 400^3 and 77 x 210 x 64 (3 % residual): per wave 1.2 us and 0.60 us
-// per plane of 256 threads, and 0.033 us per MB moved into shared memory.
+// per plane of 256 threads (0.36 us with one CTA per SM), and 0.033 us per MB
+// moved into shared memory.
 // Measured there, best shape against 64 x 16 (us per step): 96^3 5.12 / 5.95
 // (32 x 32), 144^3 11.1 / 13.1 (48 x 20), 200^3 27.2 / 32.3 (40 x 24), 240^3 39.7 /
 // 41.5 (48 x 20), 160 x 120 x 100 7.8 / 9.6 (40 x 24), 77 x 210 x 64 6.2 / 8.2 (40 x
@@ -889,7 +894,8 @@ int auto_tma_variant(const TmaPlan plans[]) {
         const double waves = (double)((p.grid + (long long)p.slots - 1) / p.slots);
         const double mb = 4e-6 * p.grid * (t.pitch * (t.ty + 2.0 * kRadius) * (p.zlen + 4.0) +
                                            t.tx * t.ty * (2.0 * p.zlen + 4.0));
-        return waves * (1.2 + 0.60 * p.zlen * p.block / 256.0) + 0.033 * mb;
+        const double plane = p.grid <= p.slots / p.occupancy ? 0.36 : 0.60;   // one CTA per SM, or two
+        return waves * (1.2 + plane * p.zlen * p.block / 256.0) + 0.033 * mb;
     };
     int best = kTmaDefaultVariant;
     double least = 0.985 * cost(plans[best]);
