@@ -678,9 +678,10 @@ struct PCtx {
     uint64_t *bar_c, *bar_z;
     int *abort_flag;
     int x0, y0, z0, T, py, xl, x;
-    float2 egx;
-    float egy[RY];
-    bool lay_xy[RY];
+    // damping off the z layers: eps_x + eps_y, 1 - that and 1 / (1 + that) at the thread's points (inside 0, 1 and
+    // 1, where relax is exactly undamped): only z-layer planes form reciprocals (240^3 128.8 -> 127.6 us per step, 180 x
+    // 220 x 100 47.4 -> 46.5)
+    float2 exy[RY], one_e[RY], rxy[RY];
     bool in0, in1;
 };
 
@@ -740,8 +741,10 @@ __device__ __forceinline__ bool p_plane(const VdArgs &a, const PCtx &c, int t, f
         float2 pn;
         if (a.fs && k == 0)
             pn = make_float2(0.0f, 0.0f);   // p = 0 on the free surface
-        else if (!C && (c.lay_xy[r] || zl))
-            pn = relax2(po, ko, div, __fadd2_rn(__fadd2_rn(c.egx, bc2(c.egy[r])), bc2(egz)));
+        else if (!C && zl)
+            pn = relax2(po, ko, div, __fadd2_rn(c.exy[r], bc2(egz)));
+        else if (!C)   // relax2 with what does not change along the march
+            pn = __fmul2_rn(__ffma2_rn(ko, div, __fmul2_rn(c.one_e[r], po)), c.rxy[r]);
         else
             pn = undamped2(po, ko, div);
         store_pair(a.p + o, pn, in0, in1);
@@ -846,13 +849,17 @@ __global__ void __launch_bounds__(S::NT, 2)
     c.x = x0 + c.xl;
     c.in0 = c.x < a.nx;
     c.in1 = c.x + 1 < a.nx;
-    c.egx = C ? bc2(0.0f) : make_float2(a.eg[0][zero_clip(c.x, a.nx)], a.eg[0][zero_clip(c.x + 1, a.nx)]);
-    const bool lay_x = x0 < a.nbl || x0 + S::TX - 1 > a.nx - 1 - a.nbl;
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
-        const int y = y0 + RY * c.py + r;
-        c.egy[r] = C ? 0.0f : a.eg[1][zero_clip(y, a.ny)];
-        c.lay_xy[r] = lay_x || y < a.nbl || y > a.ny - 1 - a.nbl;
+        const float ey = C ? 0.0f : a.eg[1][zero_clip(y0 + RY * c.py + r, a.ny)];
+        c.exy[r] = C ? bc2(0.0f)
+                     : __fadd2_rn(make_float2(a.eg[0][zero_clip(c.x, a.nx)], a.eg[0][zero_clip(c.x + 1, a.nx)]), bc2(ey));
+        c.one_e[r] = sub2(bc2(1.0f), c.exy[r]);
+        c.rxy[r] = bc2(1.0f);
+        if (!C && z0 + T > a.nbl && z0 < a.nz - a.nbl) {   // not all planes in a z layer
+            const float2 one = __fadd2_rn(bc2(1.0f), c.exy[r]);
+            c.rxy[r] = make_float2(recip_nr(one.x), recip_nr(one.y));
+        }
     }
 
     Memory m;
