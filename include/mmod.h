@@ -391,9 +391,9 @@ mmod_status mmod_forward_noalloc(const mmod_config *cfg, int device, const float
  * A batch advances several shots (one handle each: any grid sizes, the same
  * nt, the same device) together, in one of two modes (mmod_batch_set_mode):
  *   MMOD_BATCH_STREAMS (default): each shot's own time loop (the handle's
- *     graph of one-step kernels) on one of four internal streams forked
- *     from and joined back to the caller's stream, so the shots' kernels
- *     overlap;
+ *     graph of one-step kernels) on one of two internal streams (four for
+ *     small grids) forked from and joined back to the caller's stream, so the
+ *     shots' kernels overlap;
  *   MMOD_BATCH_FUSED: one kernel launch per time step covers all shots, the
  *     nt launches captured once into a CUDA graph;
  *   MMOD_BATCH_PERSISTENT: one cooperative launch runs every shot's whole

@@ -3,7 +3,7 @@
 // A batch groups handles (one per shot; grids of any size, the same number of
 // steps) and runs them in one of two ways:
 //   streams (default): each shot's own time loop (its cached graph of
-//     one-step kernels) on one of kSubStreams internal streams, forked from
+//     one-step kernels) on one of two or four internal streams, forked from
 //     and joined back to the caller's stream, so the shots' waves overlap and
 //     hide one another's tails;
 //   fused: one kernel launch per step advances every shot: CTA b serves shot
@@ -34,6 +34,17 @@ using namespace mmod;
 
 constexpr int kSubStreams = 4;
 
+// Streams a batch uses.  Two shots whose grids each fill the GPU hide one
+// another's tails, and more of them only push each other's planes out of L2;
+// smaller shots need four to fill it.  ms for 100 steps of equal cubes, two /
+// four streams: 16 of 64^3 3.03 / 2.23, 16 of 88^3 5.93 / 5.87, 16 of 96^3 5.71 /
+// 5.63, 12 of 104^3 6.00 / 5.96, 12 of 112^3 6.32 / 6.35, 8 of 120^3 4.45 / 4.58,
+// 8 of 128^3 4.93 / 5.21, 6 of 160^3 6.31 / 6.52, 4 of 224^3 10.71 / 10.69; five
+// sets of 3 to 8 uneven shots of 96 .. 256 cells per axis x 90 steps: 10.87 / 11.49,
+// 9.07 / 9.09, 12.67 / 12.88, 4.74 / 4.88, 9.71 / 9.86 (three streams between, one
+// slower than either).
+constexpr double kWideShotPoints = 1.3e6;   // mean points of a shot from which two streams serve better
+
 struct mmod_batch {
     std::vector<mmod_handle *> shots;
     int device = 0, nt = 0;
@@ -41,6 +52,7 @@ struct mmod_batch {
     int variant = kTmaDefaultVariant;
     bool variant_set = false;
     int pdl = 1;
+    int nsub = kSubStreams;           // streams in use
     cudaStream_t sub[kSubStreams] = {};
     cudaEvent_t fork = nullptr, join[kSubStreams] = {};
     std::vector<ShotDesc> desc;       // host copy, uploaded per call
@@ -162,13 +174,13 @@ float time_steps(mmod_batch *b, int steps, cudaStream_t s, mmod_status *st) {
 // Fork the internal streams from s (after everything already on s).
 mmod_status fork_streams(mmod_batch *b, cudaStream_t s) {
     BCK(b, cudaEventRecord(b->fork, s));
-    for (int k = 0; k < kSubStreams; ++k) BCK(b, cudaStreamWaitEvent(b->sub[k], b->fork, 0));
+    for (int k = 0; k < b->nsub; ++k) BCK(b, cudaStreamWaitEvent(b->sub[k], b->fork, 0));
     return MMOD_OK;
 }
 
 // Join the internal streams back into s.
 mmod_status join_streams(mmod_batch *b, cudaStream_t s) {
-    for (int k = 0; k < kSubStreams; ++k) {
+    for (int k = 0; k < b->nsub; ++k) {
         BCK(b, cudaEventRecord(b->join[k], b->sub[k]));
         BCK(b, cudaStreamWaitEvent(s, b->join[k], 0));
     }
@@ -300,7 +312,10 @@ MMOD_API mmod_status mmod_batch_create(mmod_handle *const *shots, int nshots, mm
     CKB(cudaEventCreate(&b->ev_t0));
     CKB(cudaEventCreate(&b->ev_t1));
     CKB(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
-    for (int k = 0; k < kSubStreams; ++k) {
+    double points = 0.0;
+    for (const mmod_handle *h : b->shots) points += (double)h->npts;
+    b->nsub = points >= kWideShotPoints * (double)b->shots.size() ? 2 : kSubStreams;
+    for (int k = 0; k < b->nsub; ++k) {
         CKB(cudaStreamCreateWithFlags(&b->sub[k], cudaStreamNonBlocking));
         CKB(cudaEventCreateWithFlags(&b->join[k], cudaEventDisableTiming));
     }
@@ -361,7 +376,7 @@ MMOD_API mmod_status mmod_batch_forward(mmod_batch *b, const float *const *wavel
         for (int i = 0; i < ns; ++i) {
             mmod_handle *h = b->shots[i];
             if (mmod_status st = mmod_forward(h, wavelets ? wavelets[i] : nullptr, traces ? traces[i] : nullptr,
-                                              nullptr, (mmod_stream)b->sub[i % kSubStreams])) {
+                                              nullptr, (mmod_stream)b->sub[i % b->nsub])) {
                 join_streams(b, s);
                 return bfail(b, st, "shot " + std::to_string(i) + ": " + h->err);
             }
@@ -509,7 +524,7 @@ MMOD_API mmod_status mmod_batch_autotune(mmod_batch *b, int steps, mmod_stream s
                 if (cudaEventRecord(e0, s) != cudaSuccess) st = MMOD_ERR_CUDA;
                 if (st == MMOD_OK) st = fork_streams(b, s);
                 for (int i = 0; i < ns && st == MMOD_OK; ++i)
-                    st = enqueue_tune_steps(b->shots[i], steps, b->sub[i % kSubStreams]);
+                    st = enqueue_tune_steps(b->shots[i], steps, b->sub[i % b->nsub]);
                 if (st == MMOD_OK) st = join_streams(b, s);
                 if (st == MMOD_OK && (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
                                       cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
