@@ -516,6 +516,7 @@ static mmod_status enqueue_loop(mmod_handle *h, const Geometry &geo, const float
         CpmlArgs cp = cpml_args(h);
         cp.pdl = h->pdl;
         a.pdl = h->pdl ? 2 : 0;
+        a.nbl = 0;   // the step's own damping profiles are zero
         for (int n = 0; n < nt; ++n) {
             a.n = n;
             a.ucur = h->u[(n + 1) & 1];
