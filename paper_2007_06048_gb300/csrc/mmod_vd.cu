@@ -1259,7 +1259,9 @@ mmod_status vd_loop(mmod_vd *h, const float *wav, float *tr, cudaStream_t s, lon
 // (planes per range + 7) over two resident CTAs per SM.  A launch takes about
 // a fixed time per plane of a CTA, so the shape with the fewest waves x planes
 // wins, and of those the one with the fewest CTAs; 64 x 16 gives way on equal
-// planes only to smaller tiles of the same number.  Measured, 64 x 16 against the
+// planes only to 48 x 20 tiles of the same number (40 x 24 ones lost 5 % there:
+// 105 x 45 x 118 15.8 / 16.6 us per step, 110 x 84 x 221 28.5 / 28.6 with everything
+// else 5 % faster).  Measured, 64 x 16 against the
 // choice (us per step, damping): 96^3 15.5 / 13.1 (32 x 32), 144^3 36.9 / 31.9 (48 x
 // 20), 160^3 41.0 / 35.7 (32 x 32), 200^3 96.9 / 88.4 (40 x 24), 240^3 136.3 / 134.3 (48
 // x 20), 77 x 210 x 64 23.0 / 17.2 (40 x 24); on equal planes and other counts it is
@@ -1287,7 +1289,7 @@ VdGeom plan_geom(int nx, int ny, int nz, int sms, int *shape) {
             }
         }
         const long long ctas = tiles * g.zchunks, load = (ctas + slots - 1) / slots * g.zlen;
-        const bool tie = load == best_load && (*shape == 0 ? ctas == best_ctas && t.tx * t.ty < kTmaShapes[0].tx * kTmaShapes[0].ty
+        const bool tie = load == best_load && (*shape == 0 ? ctas == best_ctas && t.tx == 48
                                                            : ctas < best_ctas);
         if (sh == 0 || load < best_load || tie) {
             best_load = load;

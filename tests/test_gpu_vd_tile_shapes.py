@@ -11,7 +11,8 @@ from test_gpu_vd import run_vd
 pytestmark = pytest.mark.gpu
 
 # (nz, ny, nx) and the (width, height) of the tiles the plan takes there
-GRIDS = [((14, 16, 64), (64, 16)), ((46, 57, 72), (48, 20)), ((37, 70, 72), (40, 24)), ((43, 88, 90), (32, 32))]
+GRIDS = [((14, 16, 64), (64, 16)), ((46, 57, 72), (48, 20)), ((37, 70, 72), (40, 24)), ((43, 62, 90), (32, 32)),
+         ((43, 88, 90), (64, 16))]   # equal planes and counts in 40 x 24: stays 64 x 16
 
 
 @pytest.mark.parametrize("surface", [False, True])
