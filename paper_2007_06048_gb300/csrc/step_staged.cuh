@@ -24,8 +24,8 @@
 //     registers (inside, e = 0 and the factor 1, where both operations are exact
 //     identities), so that only z-layer planes form reciprocals (eight per
 //     thread and plane, before on every plane of a tile that touches an x or y
-//     layer: the CTAs that ended last).  240^3 38.6 -> 37.1 us per step, 128^3
-//     batches 4 % faster, 1024 x 1024 x 512 1.3 %.
+//     layer: the CTAs that ended last).  240^3 38.6 -> 37.1 us per step,
+//     batches of uneven shots 2-4 % faster, 1024 x 1024 x 512 1.3 %.
 //   * Groups of four planes that touch a z layer run code of their own, so that
 //     a plane has no branch between its two rows: with one there, the compiler
 //     could not interleave the rows' loads and arithmetic.  240^3 37.1 -> 36.6 us
@@ -253,7 +253,7 @@ __device__ __forceinline__ void step_staged_body(const StepArgs &a, const StepVa
     const int x = x0 + 2 * px, y = y0 + S::RY * py;
     // The layer profiles at the thread's points, loaded while the previous step
     // drains: after the wait their latency would delay the first plane (151 x
-    // 117 x 98 2240 -> 2197 us, 128^3 forward and gradient 9.74 -> 9.43 ms).
+    // 117 x 98 2240 -> 2197 us, 160 x 120 x 100 forward and gradient 9.74 -> 9.43 ms).
     float ex[2], ey[S::RY];
     ex[0] = x < a.nx ? __ldg(a.ex + x) : 0.0f;
     ex[1] = x + 1 < a.nx ? __ldg(a.ex + x + 1) : 0.0f;
