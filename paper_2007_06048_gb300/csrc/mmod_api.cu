@@ -481,6 +481,14 @@ cudaError_t enqueue_step(mmod_handle *h, const StepArgs &a, const VolMaps &cur, 
     return cudaSuccess;
 }
 
+// Does the loop record the trace-row events that the download of host traces
+// waits for?  Only for traces in the handle's staging buffer, which go to the
+// host: an event between two steps keeps the second from starting before the
+// first has ended (64^3 x 100 steps 325 us with the eight of them, 301 without).
+static bool records_rows(const mmod_handle *h, const Geometry &geo, const float *tr) {
+    return tr && tr == h->st_tr && geo.ngather > 0 && &geo == &h->fwd;
+}
+
 // The time loop of a run from the state in u[0] (u^{-1}) and u[1] (u^0): nt
 // steps with the geometry geo, traces [nt][ngather] (nullable), bracketed by
 // the loop events.  Returns the number of kernels launched in *count.
@@ -490,12 +498,8 @@ static mmod_status enqueue_loop(mmod_handle *h, const Geometry &geo, const float
     const bool tma = use_tma(h);
     *count = 0;
     MMOD_CK(h, cudaEventRecordWithFlags(h->ev_t0, s, cudaEventRecordExternal));
-    // trace rows [0, done) are final: record the chunk events that wait for them.
-    // Only for traces that go to the host (through the handle's staging
-    // buffer): an event between two steps keeps the second from starting
-    // before the first has ended (64^3 x 100 steps 325 us with the eight of
-    // them, 301 without).
-    const bool marks = tr && tr == h->st_tr && ng > 0 && &geo == &h->fwd;
+    // trace rows [0, done) are final: record the chunk events that wait for them
+    const bool marks = records_rows(h, geo, tr);
     int next_mark = 0;
     auto mark = [&](long long done) -> cudaError_t {
         for (; marks && next_mark < mmod_handle::kTraceChunks && h->rows_at[next_mark] <= done; ++next_mark)
@@ -610,7 +614,9 @@ mmod_status run_loop_graph(mmod_handle *h, GraphSlot &g, const Geometry &geo, co
     const int kern = use_tma(h) ? 100 + active_plan(h).variant : MMOD_KERNEL_SIMPLE;
     const long long opts = h->pdl + 2LL * h->zlen_override + (1LL << 20) * h->claim_planes +
                            (1LL << 40) * h->cpml_planes;
-    const void *key[4] = {wav, tr, &geo, nullptr};
+    // whether the rows are recorded is part of the key: the staging buffer may
+    // get the address of device traces that an earlier loop was captured for
+    const void *key[4] = {wav, tr, &geo, records_rows(h, geo, tr) ? h->ev_rows : nullptr};
     if (!g.exec || std::memcmp(g.key, key, sizeof(key)) != 0 || g.kernel != kern || g.opts != opts) {
         free_graph(g);
         cudaGraph_t graph = nullptr;
