@@ -148,7 +148,7 @@ __global__ void __cluster_dims__(kPlaneCtas, 1, 1) __launch_bounds__(256)
 
 template <class T>
 __global__ void __launch_bounds__(256) decompress_kernel(const CkptPair<T> p, long long plane, int ctas) {
-    // no early release: the step that follows reads what this kernel writes before its own wait
+    // no early release: the step that follows needs these volumes at once
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int k = blockIdx.x / ctas, vol = blockIdx.y;   // ctas CTAs per plane
     const uint4 *in = reinterpret_cast<const uint4 *>(p.q[vol] + (long long)k * plane);
@@ -502,10 +502,8 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
 
     // segments with FP32 checkpoints step through the checkpoint volumes themselves
     const bool through = ckpt_dtype == MMOD_CKPT_FP32 && seglen >= 2;
-    if (!through) {
-        MMOD_CK(h, cudaMemsetAsync(h->u[0], 0, vb, s));
-        MMOD_CK(h, cudaMemsetAsync(h->u[1], 0, vb, s));
-    }
+    if (!through)
+        for (float *u : h->u) MMOD_CK(h, cudaMemsetAsync(u, 0, vb, s));
     h->state_pending = false;
     StepArgs fa = base_args(h, h->fwd, dwav, shape);
     fa.nrec = 0;   // no receivers in the gradient's forward sweeps
@@ -514,13 +512,29 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
     const int nadj = adj_src ? c.nsrc : 0;   // adjoint sources recorded per step
     aa.nrec = nadj;
     if (nadj && !h->st_adjg) MMOD_CK(h, cudaMalloc(&h->st_adjg, sizeof(float) * std::max<size_t>((size_t)nt * nadj, 1)));
-    // Every step may request c and its u^{n-1} before its wait (pdl 2): the
-    // only kernels here that let their successor start early are the steps, and
-    // a step's predecessor never writes the volume the step reads as u^{n-1}
-    // (the sweeps alternate two volumes; forward and adjoint steps have
-    // volumes of their own).  Not in the binomial schedule, where it measured
-    // 1 % slower (133 x 144 x 120), against 1-3 % faster in segments.
-    if (h->pdl && h->ckpt_scheme != MMOD_SCHEME_REVOLVE) fa.pdl = aa.pdl = 2;
+    // A step may request c and its u^{n-1} before its wait (pdl 2) where the
+    // operation in front of it writes neither.  Steps, imaging and saves never do
+    // (the sweeps alternate two volumes; forward and adjoint steps have volumes of
+    // their own); a restored checkpoint and a cleared volume may be the u^{n-1} of
+    // the next step, whose early copies nothing would order behind those writes:
+    // that one step waits first (unsettled).  Not in the binomial schedule, where
+    // early requests measured 1 % slower (133 x 144 x 120), against 1-3 % faster
+    // in segments.
+    const int steady_pdl = h->pdl && h->ckpt_scheme != MMOD_SCHEME_REVOLVE ? 2 : h->pdl;
+    bool unsettled = true;   // the last operation on the stream cleared or restored volumes
+    auto enqueue = [&](StepArgs &a, const VolMaps &cur, const VolMaps &prev, float *plain_gather_dst) {
+        a.pdl = unsettled ? h->pdl : steady_pdl;
+        unsettled = false;
+        return enqueue_step(h, a, cur, prev, tma, plain_gather_dst, s, &launches);
+    };
+    auto clear = [&](float *p, size_t bytes) {
+        unsettled = true;
+        return cudaMemsetAsync(p, 0, bytes, s);
+    };
+    auto restore = [&](int slot, float *u_prev, float *u_cur) {
+        unsettled = true;
+        return restore_state(h, slot, u_prev, u_cur, s);
+    };
     // forward step n in place on the handle's buffers: u^{n-1} in u[n & 1],
     // u^n in u[(n + 1) & 1], u^{n+1} over u^{n-1}
     auto fwd_step_in_place = [&](int n) {
@@ -528,7 +542,7 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
         fa.ucur = h->u[(n + 1) & 1];
         fa.uprev = h->u[n & 1];
         fa.uout = h->u[n & 1];
-        return enqueue_step(h, fa, u_map[(n + 1) & 1], u_map[n & 1], tma, nullptr, s, &launches);
+        return enqueue(fa, u_map[(n + 1) & 1], u_map[n & 1], nullptr);
     };
     // forward step n from u^{n-1} in prev and u^n in cur into out (prev's
     // volume or another), also writing g^n into gout (null: not)
@@ -546,7 +560,7 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
         fa.uprev = prev.p;
         fa.uout = out.p;
         fa.gout = gout;
-        const cudaError_t e = enqueue_step(h, fa, *cur.m, *prev.m, tma, nullptr, s, &launches);
+        const cudaError_t e = enqueue(fa, *cur.m, *prev.m, nullptr);
         fa.gout = nullptr;
         return e;
     };
@@ -575,8 +589,8 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
         aa.uout = gw.psi[m & 1];
         // the step kernel records the field it reads (adjoint step m - 1); the plain path the one it writes
         aa.traces = nadj && m >= 1 ? h->st_adjg + (size_t)(m - 1) * nadj : nullptr;
-        return enqueue_step(h, aa, gw.psi_map[(m + 1) & 1], gw.psi_map[m & 1], tma,
-                            nadj ? h->st_adjg + (size_t)m * nadj : nullptr, s, &launches);
+        return enqueue(aa, gw.psi_map[(m + 1) & 1], gw.psi_map[m & 1],
+                       nadj ? h->st_adjg + (size_t)m * nadj : nullptr);
     };
     // imaging terms of forward steps n (and n - 1 when ns = 2) from g[t] =
     // g^{n-t}, after their adjoint steps: psi^{n+1} in psi[(nt-1-n) & 1],
@@ -611,19 +625,19 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
     if (seglen == 0 && nslot == 0) {
         // every step's g^n kept: seg[0], seg[1] hold the stepped state,
         // seg[2 + n] = g^n
-        MMOD_CK(h, cudaMemsetAsync(gw.seg[0], 0, vb, s));
-        MMOD_CK(h, cudaMemsetAsync(gw.seg[1], 0, vb, s));
+        MMOD_CK(h, clear(gw.seg[0], vb));
+        MMOD_CK(h, clear(gw.seg[1], vb));
         for (int n = 0; n < nt; ++n) MMOD_CK(h, fwd_step_g(n, n & 1, (n + 1) & 1, gw.seg[2 + n]));
-        MMOD_CK(h, cudaMemsetAsync(gw.psi[0], 0, vb, s));
-        MMOD_CK(h, cudaMemsetAsync(gw.psi[1], 0, vb, s));
-        MMOD_CK(h, cudaMemsetAsync(gw.gradc, 0, vb, s));
+        MMOD_CK(h, clear(gw.psi[0], vb));
+        MMOD_CK(h, clear(gw.psi[1], vb));
+        MMOD_CK(h, clear(gw.gradc, vb));
         MMOD_CK(h, backward_range(nt - 1, 0, [&](int j) { return gw.seg[2 + j]; }));
     } else if (h->ckpt_scheme == MMOD_SCHEME_REVOLVE) {
         std::vector<RevAction> sched;
         revolve_schedule(nt, nslot, &sched);
-        MMOD_CK(h, cudaMemsetAsync(gw.psi[0], 0, vb, s));
-        MMOD_CK(h, cudaMemsetAsync(gw.psi[1], 0, vb, s));
-        MMOD_CK(h, cudaMemsetAsync(gw.gradc, 0, vb, s));
+        MMOD_CK(h, clear(gw.psi[0], vb));
+        MMOD_CK(h, clear(gw.psi[1], vb));
+        MMOD_CK(h, clear(gw.gradc, vb));
         float *unext = gw.seg[0], *gn = gw.seg[1];
         // the imaging form of the step kernel: g^n is formed and used in one pass
         const bool one_pass = tma && active_plan(h).has_image && h->claim_planes == 0 &&
@@ -638,10 +652,10 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
                     break;
                 case MMOD_REV_RESTORE:
                     if (act.a < 0) {
-                        MMOD_CK(h, cudaMemsetAsync(h->u[0], 0, vb, s));
-                        MMOD_CK(h, cudaMemsetAsync(h->u[1], 0, vb, s));
+                        MMOD_CK(h, clear(h->u[0], vb));
+                        MMOD_CK(h, clear(h->u[1], vb));
                     } else {
-                        MMOD_CK(h, restore_state(h, act.a, h->u[act.b & 1], h->u[(act.b + 1) & 1], s));
+                        MMOD_CK(h, restore(act.a, h->u[act.b & 1], h->u[(act.b + 1) & 1]));
                     }
                     break;
                 case MMOD_REV_REVERSE: {   // the adjoint step and its term, g^n from the working state
@@ -664,8 +678,7 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
                     fa.uprev = h->u[n & 1];
                     fa.uout = unext;
                     fa.gout = gn;
-                    const cudaError_t e = enqueue_step(h, fa, u_map[(n + 1) & 1], u_map[n & 1], tma,
-                                                       nullptr, s, &launches);
+                    const cudaError_t e = enqueue(fa, u_map[(n + 1) & 1], u_map[n & 1], nullptr);
                     fa.gout = nullptr;
                     MMOD_CK(h, e);
                     MMOD_CK(h, adj_step(n));
@@ -690,7 +703,7 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
             // slot's; the last segment stays in its own slot.  (Saving and
             // restoring 20 checkpoints of 200^3 took 78 copies of 34 MB, 1 of
             // 42 ms.)  After a full segment u^{b0} is in volume (seglen - 1) & 1.
-            MMOD_CK(h, cudaMemsetAsync(slot(0, 0).p, 0, 2 * vb, s));
+            MMOD_CK(h, clear(slot(0, 0).p, 2 * vb));
             for (int sg = 0; sg < nseg; ++sg) {
                 const int a0 = sg * seglen, b0 = std::min(nt, a0 + seglen), i = sg == 0 ? 0 : seglen & 1;
                 if (sg < nseg - 1)
@@ -710,9 +723,9 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
         }
         // ---- backward: replay each segment (g^n of its steps), then its
         // adjoint steps + imaging
-        MMOD_CK(h, cudaMemsetAsync(gw.psi[0], 0, vb, s));
-        MMOD_CK(h, cudaMemsetAsync(gw.psi[1], 0, vb, s));
-        MMOD_CK(h, cudaMemsetAsync(gw.gradc, 0, vb, s));
+        MMOD_CK(h, clear(gw.psi[0], vb));
+        MMOD_CK(h, clear(gw.psi[1], vb));
+        MMOD_CK(h, clear(gw.gradc, vb));
         for (int sg = nseg - 1; sg >= 0; --sg) {
             const int a0 = sg * seglen, b0 = std::min(nt, a0 + seglen);
             if (through && sg < nseg - 1) {
@@ -720,7 +733,7 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
                 MMOD_CK(h, fwd_range(a0, b0, slot(sg, i), slot(sg, 1 - i), seg(0), seg(1),
                                      [&](int j) { return gw.seg[2 + j]; }));
             } else if (!through) {
-                MMOD_CK(h, restore_state(h, sg, gw.seg[0], gw.seg[1], s));
+                MMOD_CK(h, restore(sg, gw.seg[0], gw.seg[1]));
                 for (int n = a0; n < b0; ++n) {   // seg[2 + n - a0] receives g^n
                     const int j = n - a0;
                     MMOD_CK(h, fwd_step_g(n, j & 1, (j + 1) & 1, gw.seg[2 + j]));
