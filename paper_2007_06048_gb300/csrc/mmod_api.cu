@@ -113,13 +113,18 @@ void free_all(mmod_handle *h) {
     if (h->err_host) cudaFreeHost(h->err_host);
 }
 
+// Tables go up on a stream of the handle's own, which the functions below wait
+// for while the host vectors live: whatever stream the next run is on, they are
+// in place.  (On the legacy stream a copy from pageable memory may return before
+// its last transfer has landed, and nothing orders that stream before a
+// non-blocking one.)
 template <class T>
-cudaError_t upload(T **dst, const std::vector<T> &v) {
+cudaError_t upload(T **dst, const std::vector<T> &v, cudaStream_t s) {
     const size_t n = std::max<size_t>(v.size(), 1);
     cudaError_t e = cudaMalloc(dst, sizeof(T) * n);
     if (e != cudaSuccess) return e;
-    if (v.empty()) return cudaMemset(*dst, 0, sizeof(T));
-    return cudaMemcpy(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice);
+    if (v.empty()) return cudaMemsetAsync(*dst, 0, sizeof(T), s);
+    return cudaMemcpyAsync(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, s);
 }
 
 // Indices 0 .. n-1 in stable ascending order of key (>= 0): radix sort, 16
@@ -148,7 +153,7 @@ std::vector<int> order_by_key(const std::vector<long long> &key) {
 // (stable order), points sorted by (tile, plane, j, i) and bucketed per
 // (tile of the shape, plane).  src_row = index of the position in pos.
 cudaError_t build_inj(const mmod_config &c, long long plane, int nxp, const int *pos, int n, const TmaShape &sh,
-                      DevInj *t) {
+                      cudaStream_t up, DevInj *t) {
     t->tiles_x = (c.nx + sh.tx - 1) / sh.tx;
     t->tiles_y = (c.ny + sh.ty - 1) / sh.ty;
     const long long tiles = (long long)t->tiles_x * t->tiles_y;
@@ -190,16 +195,16 @@ cudaError_t build_inj(const mmod_config &c, long long plane, int nxp, const int 
     for (size_t b = 1; b < tile_start.size(); ++b) tile_start[b] += tile_start[b - 1];
     t->npts = (int)pt_i.size();
     cudaError_t e;
-    if ((e = upload(&t->tile_start, tile_start)) || (e = upload(&t->pt_i, pt_i)) || (e = upload(&t->pt_j, pt_j)) ||
-        (e = upload(&t->pt_k, pt_k)) || (e = upload(&t->pt_off, pt_off)) || (e = upload(&t->pt_first, pt_first)) ||
-        (e = upload(&t->src_row, src_row)))
+    if ((e = upload(&t->tile_start, tile_start, up)) || (e = upload(&t->pt_i, pt_i, up)) ||
+        (e = upload(&t->pt_j, pt_j, up)) || (e = upload(&t->pt_k, pt_k, up)) || (e = upload(&t->pt_off, pt_off, up)) ||
+        (e = upload(&t->pt_first, pt_first, up)) || (e = upload(&t->src_row, src_row, up)))
         return e;
-    return cudaSuccess;
+    return cudaStreamSynchronize(up);
 }
 
 // The positions of a geometry's injections, in the caller's order, and room
 // for their scales.
-cudaError_t build_positions(const int *pos, int n, Geometry *g) {
+cudaError_t build_positions(const int *pos, int n, cudaStream_t up, Geometry *g) {
     std::vector<int> si(n), sj(n), sk(n);
     for (int q = 0; q < n; ++q) {
         si[q] = pos[3 * q];
@@ -208,16 +213,17 @@ cudaError_t build_positions(const int *pos, int n, Geometry *g) {
     }
     g->npos = n;
     cudaError_t e;
-    if ((e = upload(&g->si, si)) || (e = upload(&g->sj, sj)) || (e = upload(&g->sk, sk))) return e;
+    if ((e = upload(&g->si, si, up)) || (e = upload(&g->sj, sj, up)) || (e = upload(&g->sk, sk, up))) return e;
     if ((e = cudaMalloc(&g->scale, sizeof(float) * std::max(n, 1)))) return e;
-    return cudaMemset(g->scale, 0, sizeof(float) * std::max(n, 1));
+    if ((e = cudaMemsetAsync(g->scale, 0, sizeof(float) * std::max(n, 1), up))) return e;
+    return cudaStreamSynchronize(up);
 }
 
 // Gather positions pos[n][3] bucketed per (64 x 16 tile, plane), tile-major
 // as the injection table: entries [start[b], start[b+1]) of bucket
 // b = tile * nz + k hold the original index and the padded offset.
 cudaError_t build_gather_buckets(const mmod_config &c, long long plane, int nxp, const int *pos, int n,
-                                 Geometry *g) {
+                                 cudaStream_t up, Geometry *g) {
     const int tiles_x = (c.nx + kInjTileX - 1) / kInjTileX, tiles_y = (c.ny + kInjTileY - 1) / kInjTileY;
     std::vector<long long> bucket(n);
     for (int r = 0; r < n; ++r) {
@@ -236,14 +242,16 @@ cudaError_t build_gather_buckets(const mmod_config &c, long long plane, int nxp,
     }
     for (size_t b = 1; b < start.size(); ++b) start[b] += start[b - 1];
     cudaError_t e;
-    if ((e = upload(&g->g_start, start)) || (e = upload(&g->g_idx, idx)) || (e = upload(&g->g_off, off))) return e;
-    return cudaSuccess;
+    if ((e = upload(&g->g_start, start, up)) || (e = upload(&g->g_idx, idx, up)) || (e = upload(&g->g_off, off, up)))
+        return e;
+    return cudaStreamSynchronize(up);
 }
 
-cudaError_t build_gather(long long plane, int nxp, const int *pos, int n, long long **off) {
+cudaError_t build_gather(long long plane, int nxp, const int *pos, int n, cudaStream_t up, long long **off) {
     std::vector<long long> o(n);
     for (int r = 0; r < n; ++r) o[r] = (long long)pos[3 * r + 2] * plane + (long long)pos[3 * r + 1] * nxp + pos[3 * r];
-    return upload(off, o);
+    if (cudaError_t e = upload(off, o, up)) return e;
+    return cudaStreamSynchronize(up);
 }
 
 }  // namespace
@@ -416,7 +424,7 @@ mmod_status ensure_shape(mmod_handle *h, int shape) {
         for (Geometry *g : {&h->fwd, &h->adj}) {
             free_inj(g->inj[shape]);   // left by an attempt that failed half way
             const auto &pos = g == &h->fwd ? h->src : h->rec;
-            MMOD_CK(h, build_inj(c, h->plane, h->nxp, pos.data(), g->npos, sh, &g->inj[shape]));
+            MMOD_CK(h, build_inj(c, h->plane, h->nxp, pos.data(), g->npos, sh, h->st_copy, &g->inj[shape]));
         }
     } catch (const std::bad_alloc &) {
         return fail(h, MMOD_ERR_OOM, "host memory for the injection tables");
@@ -708,42 +716,43 @@ MMOD_API mmod_status mmod_create(const mmod_config *cfg, int device, mmod_handle
     } while (0)
 
     const size_t vbytes = sizeof(float) * (size_t)h->vol;
+    CKC(cudaStreamCreateWithFlags(&h->st_copy, cudaStreamNonBlocking));
+    cudaStream_t up = h->st_copy;
     CKC(cudaMalloc(&h->u[0], vbytes));
     CKC(cudaMalloc(&h->u[1], vbytes));
     CKC(cudaMalloc(&h->c, vbytes));
     CKC(cudaMalloc(&h->eta, sizeof(float) * (size_t)(nx + ny + nz)));
-    CKC(cudaMemset(h->u[0], 0, vbytes));
-    CKC(cudaMemset(h->u[1], 0, vbytes));
-    CKC(cudaMemset(h->c, 0, vbytes));
-    CKC(cudaMemset(h->eta, 0, sizeof(float) * (size_t)(nx + ny + nz)));
+    CKC(cudaMemsetAsync(h->u[0], 0, vbytes, up));
+    CKC(cudaMemsetAsync(h->u[1], 0, vbytes, up));
+    CKC(cudaMemsetAsync(h->c, 0, vbytes, up));
+    CKC(cudaMemsetAsync(h->eta, 0, sizeof(float) * (size_t)(nx + ny + nz), up));
     if (is_cpml(h)) {
         CKC(cudaMalloc(&h->cpml_mem, 6 * vbytes));
-        CKC(cudaMemset(h->cpml_mem, 0, 6 * vbytes));
+        CKC(cudaMemsetAsync(h->cpml_mem, 0, 6 * vbytes, up));
         CKC(cudaMalloc(&h->cpml_bg, sizeof(float) * 2 * (size_t)(nx + ny + nz)));
-        CKC(cudaMemset(h->cpml_bg, 0, sizeof(float) * 2 * (size_t)(nx + ny + nz)));
+        CKC(cudaMemsetAsync(h->cpml_bg, 0, sizeof(float) * 2 * (size_t)(nx + ny + nz), up));
         h->cpml_xc_floats = cpml_x_compact_floats(cpml_args(h));
         if (h->cpml_xc_floats > 0) {
             CKC(cudaMalloc(&h->cpml_xc, sizeof(float) * (size_t)h->cpml_xc_floats));
-            CKC(cudaMemset(h->cpml_xc, 0, sizeof(float) * (size_t)h->cpml_xc_floats));
+            CKC(cudaMemsetAsync(h->cpml_xc, 0, sizeof(float) * (size_t)h->cpml_xc_floats, up));
         }
     }
     CKC(cudaMalloc(&h->vmax_bits, sizeof(unsigned int)));
     CKC(cudaMalloc(&h->bad, sizeof(unsigned long long)));
     // forward: sources injected, receivers gathered; adjoint: the reverse
-    CKC(build_positions(h->src.data(), cfg->nsrc, &h->fwd));
-    CKC(build_gather(h->plane, h->nxp, h->rec.data(), cfg->nrec, &h->fwd.gather_off));
+    CKC(build_positions(h->src.data(), cfg->nsrc, up, &h->fwd));
+    CKC(build_gather(h->plane, h->nxp, h->rec.data(), cfg->nrec, up, &h->fwd.gather_off));
     h->fwd.ngather = cfg->nrec;
     h->fwd.cell = cfg->hx * cfg->hy * cfg->hz;
-    CKC(build_positions(h->rec.data(), cfg->nrec, &h->adj));
-    CKC(build_gather(h->plane, h->nxp, h->src.data(), cfg->nsrc, &h->adj.gather_off));
+    CKC(build_positions(h->rec.data(), cfg->nrec, up, &h->adj));
+    CKC(build_gather(h->plane, h->nxp, h->src.data(), cfg->nsrc, up, &h->adj.gather_off));
     h->adj.ngather = cfg->nsrc;
     h->adj.cell = 1.0;
-    CKC(build_gather_buckets(h->cfg, h->plane, h->nxp, h->rec.data(), cfg->nrec, &h->fwd));
-    CKC(build_gather_buckets(h->cfg, h->plane, h->nxp, h->src.data(), cfg->nsrc, &h->adj));
+    CKC(build_gather_buckets(h->cfg, h->plane, h->nxp, h->rec.data(), cfg->nrec, up, &h->fwd));
+    CKC(build_gather_buckets(h->cfg, h->plane, h->nxp, h->src.data(), cfg->nsrc, up, &h->adj));
     CKC(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
     CKC(cudaEventCreate(&h->ev_t0));
     CKC(cudaEventCreate(&h->ev_t1));
-    CKC(cudaStreamCreateWithFlags(&h->st_copy, cudaStreamNonBlocking));
     CKC(cudaEventCreateWithFlags(&h->ev_copied, cudaEventDisableTiming));
     for (int i = 0; i < mmod_handle::kTraceChunks; ++i) {
         CKC(cudaEventCreateWithFlags(&h->ev_rows[i], cudaEventDisableTiming));
@@ -767,8 +776,9 @@ MMOD_API mmod_status mmod_create(const mmod_config *cfg, int device, mmod_handle
         CKC(cudaMalloc(&h->counters, sizeof(int) * (size_t)h->ncounters));
         CKC(cudaMalloc(&h->queue, sizeof(unsigned long long)));
         CKC(cudaMalloc(&h->claim_ctr, 2 * sizeof(int)));
-        CKC(cudaMemset(h->claim_ctr, 0, 2 * sizeof(int)));
+        CKC(cudaMemsetAsync(h->claim_ctr, 0, 2 * sizeof(int), up));
     }
+    CKC(cudaStreamSynchronize(up));
 #undef CKC
     *out = h;
     return MMOD_OK;
@@ -795,6 +805,17 @@ MMOD_API mmod_status mmod_set_kernel(mmod_handle *h, int kernel) {
     return MMOD_OK;
 }
 
+// Sets what the tile shape of the next run depends on, and sets that shape up, so
+// that no run has to; keeps the old value where that fails.
+static mmod_status select(mmod_handle *h, int *what, int value) {
+    const int old = *what;
+    *what = value;
+    DeviceGuard guard(h->device);
+    const mmod_status st = ensure_shape(h, active_shape(h));
+    if (st != MMOD_OK) *what = old;
+    return st;
+}
+
 MMOD_API int mmod_tma_variant_count(void) { return tma_variant_count(); }
 
 MMOD_API const char *mmod_tma_variant_name(int v) { return tma_variant_name(v); }
@@ -803,8 +824,7 @@ MMOD_API mmod_status mmod_set_tma_variant(mmod_handle *h, int v) {
     if (!h) return MMOD_ERR_ARG;
     if (v < -1 || v >= tma_variant_count()) return fail(h, MMOD_ERR_ARG, "unknown TMA variant");
     if (v >= 0 && !h->tma_ok) return fail(h, MMOD_ERR_UNSUPPORTED, "TMA kernel unavailable for this grid");
-    h->variant = v;
-    return MMOD_OK;
+    return select(h, &h->variant, v);
 }
 
 MMOD_API mmod_status mmod_set_option(mmod_handle *h, int option, int value) {
@@ -826,8 +846,7 @@ MMOD_API mmod_status mmod_set_option(mmod_handle *h, int option, int value) {
     }
     if (option == MMOD_OPT_CLAIM) {
         if (value < 0 || value > 1 << 20) return fail(h, MMOD_ERR_ARG, "MMOD_OPT_CLAIM must be in [0, 2^20]");
-        h->claim_planes = value;
-        return MMOD_OK;
+        return select(h, &h->claim_planes, value);
     }
     if (option == MMOD_OPT_PERSISTENT_CTAS) {
         if (value < 0) return fail(h, MMOD_ERR_ARG, "MMOD_OPT_PERSISTENT_CTAS must be >= 0");
@@ -838,7 +857,7 @@ MMOD_API mmod_status mmod_set_option(mmod_handle *h, int option, int value) {
     switch (option) {
         case MMOD_OPT_PDL: h->pdl = value; return MMOD_OK;
         case MMOD_OPT_CKPT_SCHEME: h->ckpt_scheme = value; return MMOD_OK;
-        case MMOD_OPT_PERSISTENT: h->persistent = value; return MMOD_OK;
+        case MMOD_OPT_PERSISTENT: return select(h, &h->persistent, value);
         case MMOD_OPT_TEST_STALL: h->test_stall = value; return MMOD_OK;
         default: return fail(h, MMOD_ERR_ARG, "unknown option");
     }

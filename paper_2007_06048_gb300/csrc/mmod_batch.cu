@@ -341,6 +341,9 @@ MMOD_API mmod_status mmod_batch_set_variant(mmod_batch *b, int v) {
     if (!b) return MMOD_ERR_ARG;
     int block, smem;
     if (!tma_variant_has_batch(v) || !tma_variant_shape(v, &block, &smem)) return bfail(b, MMOD_ERR_ARG, "unknown TMA variant");
+    DeviceGuard guard(b->device);
+    for (mmod_handle *h : b->shots)   // 64 x 16 tiles: set up here, so that no run has to
+        if (mmod_status st = ensure_shape(h, 0)) return bfail(b, st, h->err);
     b->variant = v;
     b->variant_set = true;
     for (mmod_handle *h : b->shots) h->variant = v;   // streams mode runs each handle's own plan
@@ -351,6 +354,11 @@ MMOD_API mmod_status mmod_batch_set_mode(mmod_batch *b, int mode) {
     if (!b) return MMOD_ERR_ARG;
     if (mode != MMOD_BATCH_STREAMS && mode != MMOD_BATCH_FUSED && mode != MMOD_BATCH_PERSISTENT)
         return bfail(b, MMOD_ERR_ARG, "unknown batch mode");
+    if (mode != MMOD_BATCH_STREAMS) {   // their kernels run 64 x 16 tiles: set up here, so that no run has to
+        DeviceGuard guard(b->device);
+        for (mmod_handle *h : b->shots)
+            if (mmod_status st = ensure_shape(h, 0)) return bfail(b, st, h->err);
+    }
     b->mode = mode;
     return MMOD_OK;
 }

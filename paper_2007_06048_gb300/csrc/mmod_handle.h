@@ -90,7 +90,7 @@ struct mmod_handle {
     static constexpr int kTraceChunks = 8;
     cudaEvent_t ev_rows[kTraceChunks] = {};
     long long rows_at[kTraceChunks] = {};
-    cudaStream_t st_copy = nullptr;
+    cudaStream_t st_copy = nullptr;     // also uploads the tables at set-up
     cudaEvent_t ev_copied = nullptr;
     mmod::GraphSlot g_fwd, g_adj;
 
@@ -174,9 +174,9 @@ void drop_graphs(mmod_handle *h);   // mmod_api.cu: captured loops must be re-ca
 inline bool is_cpml(const mmod_handle *h) { return h->cfg.boundary == MMOD_BOUNDARY_CPML; }
 CpmlArgs cpml_args(const mmod_handle *h);
 const TmaPlan &active_plan(const mmod_handle *h);
-// Tile shape of the handle's next run (0 without TMA kernels), with its
-// tensor maps and injection tables built: allocates on first use, so it runs
-// before any capture.
+// Tile shape of the handle's next run (0 without TMA kernels), and its tensor
+// maps and injection tables, complete when this returns: built once per shape,
+// by the call that selects it (create, variant, option, batch mode).
 mmod_status ensure_shape(mmod_handle *h, int shape);
 int active_shape(const mmod_handle *h);
 StepArgs base_args(mmod_handle *h, const Geometry &geo, const float *wavelet, int shape);

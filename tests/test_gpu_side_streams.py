@@ -1,0 +1,48 @@
+"""Handles used on a non-blocking stream while the default stream is busy: a run
+may rely on nothing that the default stream still has to do.  Tile shapes
+selected by variant and option right before the run; the same bits as
+on the default stream."""
+import numpy as np
+import pytest
+
+import paper_2007_06048_gb300 as M
+import workloads as W
+from _gpu_util import torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+CHANGES = [None, ("variant", 2), ("variant", 10), ("option", M.OPT_PERSISTENT, 1), ("option", M.OPT_CLAIM, 8)]
+
+
+def _problem(seed=9):
+    return W.tiny_problem(shape=(40, 100, 130), nt=40, nbl=8, nsrc=4, nrec=5000, seed=seed)
+
+
+def _run(p, stream, change):
+    torch = torch_cuda()
+    vel, wav = torch.from_numpy(p.vel).cuda(), torch.from_numpy(p.wavelet).cuda()
+    resid = torch.from_numpy(np.random.default_rng(1).standard_normal((p.nt, 5000)).astype(np.float32)).cuda()
+    tr, adj = (torch.empty(s, device="cuda") for s in ((p.nt, 5000), (4, p.nt)))
+    torch.cuda.synchronize()
+    if stream is not None:
+        torch.cuda._sleep(40_000_000)   # some 20 ms of work on the default stream
+    s = None if stream is None else stream.cuda_stream
+    prop = M.Propagator.from_problem(p)
+    prop.set_model(vel, s)
+    if change:
+        prop.set_variant(change[1]) if change[0] == "variant" else prop.set_option(*change[1:])
+    prop.forward(wav, tr, None, s)
+    prop.adjoint(resid, adj, s)
+    torch.cuda.synchronize()
+    prop.close()
+    return [t.cpu().numpy() for t in (tr, adj)]
+
+
+@pytest.mark.parametrize("change", CHANGES)
+def test_side_stream_bitwise(change):
+    torch = torch_cuda()
+    p = _problem()
+    ref = _run(p, None, None)
+    got = _run(p, torch.cuda.Stream(), change)
+    for a, b in zip(got, ref):
+        assert np.abs(b).max() > 0 and np.array_equal(a, b)

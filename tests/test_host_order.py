@@ -90,3 +90,77 @@ def test_steps_read_early_only_what_is_settled(rt, ckpt, dtype, scheme):
     # three sweeps, or two where every state or term is kept; early reads are the rule in segments
     assert steps >= 2 * p.nt
     assert early >= (steps // 2 if scheme == M.SCHEME_SEGMENTS and ckpt < p.nt else 0)
+
+
+H2D = 1   # cudaMemcpyHostToDevice
+
+
+def _uploads_done(log):
+    """Every upload or fill of a set-up call ran on a stream of the library's own
+    and was waited for before the call returned."""
+    last = {}
+    for i, e in enumerate(log):
+        if e["op"] == "memset" or e["op"] == "memcpy" and e["kind"] == H2D:
+            assert e["stream"] != 0, e   # the legacy stream orders nothing for non-blocking streams
+            last[e["stream"]] = i
+    for stream, i in last.items():
+        assert any(e["op"] == "sync" and e["stream"] == stream for e in log[i:]), stream
+    return len(last)
+
+
+def _stays_on(log, stream):
+    """Nothing of a run is allocated, uploaded or put on another caller's stream."""
+    for e in log:
+        assert e["op"] != "malloc" and not (e["op"] == "memcpy" and e["kind"] == H2D), e
+        assert e.get("stream", stream) != 0, e
+
+
+def test_create_returns_with_its_tables_in_place(rt):
+    rt.log()
+    p = _problem(shape=(40, 100, 130))
+    rt.propagator(p, model=False)
+    assert _uploads_done(rt.log()) == 1
+
+
+@pytest.mark.parametrize("change", [("variant", v) for v in (9, 10, 11, 0, -1)]
+                         + [("option", (M.OPT_PERSISTENT, 1)), ("option", (M.OPT_CLAIM, 4))])
+def test_another_tile_shape_is_set_up_by_the_call_that_selects_it(rt, change):
+    """Tables of another tile shape are complete when the selecting call returns;
+    the runs that follow, on any stream, allocate and upload nothing."""
+    p = _problem(shape=(40, 100, 130))
+    prop = rt.propagator(p)
+    assert prop.plan()["variant"] == 9   # 48 x 20 tiles: the options below need 64 x 16
+    wav, traces, resid, adj, grad = (rt.malloc(n) for n in (p.wavelet.size, p.nt * 9, p.nt * 9, p.nt * 2, p.vel.size))
+    s = rt.stream()
+
+    def runs():
+        prop.forward(wav, traces, stream=s)
+        prop.adjoint(resid, adj, stream=s)
+        prop.gradient(wav, resid, grad, 4, M.CKPT_BF16, stream=s)
+
+    runs()
+    rt.log()
+    kind, value = change
+    prop.set_variant(value) if kind == "variant" else prop.set_option(*value)
+    shape_built = _uploads_done(rt.log())
+    assert shape_built == (0 if change in (("variant", 9), ("variant", -1)) else 1)
+    runs()
+    _stays_on(rt.log(), s)
+
+
+@pytest.mark.parametrize("mode,variant", [(M.BATCH_FUSED, None), (M.BATCH_PERSISTENT, None), (M.BATCH_STREAMS, 5)])
+def test_batch_sets_up_its_tiles(rt, mode, variant):
+    p = _problem(shape=(40, 100, 130))
+    props = [rt.propagator(p) for _ in range(2)]
+    b = rt.batch(props)
+    bufs = [[rt.malloc(n) for _ in props] for n in (p.wavelet.size, p.nt * 9)]
+    rt.log()
+    b.set_mode(mode)
+    if variant is not None:
+        b.set_variant(variant)
+    assert _uploads_done(rt.log()) >= 1
+    s = rt.stream()
+    b.forward(*bufs, stream=s)
+    log = rt.log()
+    assert not [e for e in log if e["op"] == "malloc"]
+    assert all(e["stream"] != 0 for e in log if "stream" in e)   # the shots' arguments go up on the caller's
