@@ -322,8 +322,9 @@ mmod_status encode_grad_maps(mmod_handle *h, int shape) {
 }
 
 // Allocate (or keep) the gradient work space: nslot checkpoints of two
-// volumes, nwork FP32 work volumes (with tensor maps), psi, grad_c.
-mmod_status ensure_grad_work(mmod_handle *h, int nslot, int nwork, int dtype, int shape) {
+// volumes, nwork FP32 work volumes (with tensor maps; cleared on the run's
+// stream, in front of the steps that write them), psi, grad_c.
+mmod_status ensure_grad_work(mmod_handle *h, int nslot, int nwork, int dtype, int shape, cudaStream_t s) {
     auto &gw = h->gw;
     if (gw.nslot == nslot && gw.nwork == nwork && gw.dtype == dtype) return encode_grad_maps(h, shape);
     free_grad_work(h);
@@ -333,7 +334,7 @@ mmod_status ensure_grad_work(mmod_handle *h, int nslot, int nwork, int dtype, in
     gw.ckpt_map.resize(2 * (size_t)nslot);
     for (int i = 0; i < nwork; ++i) {
         MMOD_CK(h, cudaMalloc(&gw.seg[i], vb));
-        MMOD_CK(h, cudaMemset(gw.seg[i], 0, vb));
+        MMOD_CK(h, cudaMemsetAsync(gw.seg[i], 0, vb, s));
     }
     for (int b = 0; b < 2; ++b) MMOD_CK(h, cudaMalloc(&gw.psi[b], vb));
     MMOD_CK(h, cudaMalloc(&gw.gradc, vb));
@@ -486,7 +487,7 @@ static mmod_status run_gradient(mmod_handle *h, const float *wavelet, const floa
     grad_layout(h, ckpt_count, ckpt_dtype, &nslot, &nwork, &seglen);
     const int shape = active_shape(h);
     if (mmod_status st = ensure_shape(h, shape)) return st;
-    if (mmod_status st = ensure_grad_work(h, nslot, nwork, ckpt_dtype, shape)) return st;
+    if (mmod_status st = ensure_grad_work(h, nslot, nwork, ckpt_dtype, shape, s)) return st;
     const VolMaps *u_map = h->shapes[shape].u;
     auto &gw = h->gw;
     const bool tma = use_tma(h);

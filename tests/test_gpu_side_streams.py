@@ -22,7 +22,7 @@ def _run(p, stream, change):
     torch = torch_cuda()
     vel, wav = torch.from_numpy(p.vel).cuda(), torch.from_numpy(p.wavelet).cuda()
     resid = torch.from_numpy(np.random.default_rng(1).standard_normal((p.nt, 5000)).astype(np.float32)).cuda()
-    tr, adj = (torch.empty(s, device="cuda") for s in ((p.nt, 5000), (4, p.nt)))
+    tr, adj, g = (torch.empty(s, device="cuda") for s in ((p.nt, 5000), (4, p.nt), p.vel.shape))
     torch.cuda.synchronize()
     if stream is not None:
         torch.cuda._sleep(40_000_000)   # some 20 ms of work on the default stream
@@ -33,9 +33,10 @@ def _run(p, stream, change):
         prop.set_variant(change[1]) if change[0] == "variant" else prop.set_option(*change[1:])
     prop.forward(wav, tr, None, s)
     prop.adjoint(resid, adj, s)
+    prop.gradient(wav, resid, g, 4, M.CKPT_FP32, s)
     torch.cuda.synchronize()
     prop.close()
-    return [t.cpu().numpy() for t in (tr, adj)]
+    return [t.cpu().numpy() for t in (tr, adj, g)]
 
 
 @pytest.mark.parametrize("change", CHANGES)

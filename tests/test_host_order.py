@@ -164,3 +164,16 @@ def test_batch_sets_up_its_tiles(rt, mode, variant):
     log = rt.log()
     assert not [e for e in log if e["op"] == "malloc"]
     assert all(e["stream"] != 0 for e in log if "stream" in e)   # the shots' arguments go up on the caller's
+
+
+@pytest.mark.parametrize("scheme,dtype,ckpt", [(M.SCHEME_SEGMENTS, M.CKPT_FP32, 4), (M.SCHEME_SEGMENTS, M.CKPT_FP32, 16),
+                                               (M.SCHEME_SEGMENTS, M.CKPT_BF16, 4), (M.SCHEME_REVOLVE, M.CKPT_FP32, 3)])
+def test_first_gradient_fills_its_work_volumes_on_the_callers_stream(rt, scheme, dtype, ckpt):
+    p = _problem()
+    prop = rt.propagator(p)
+    prop.set_option(M.OPT_CKPT_SCHEME, scheme)
+    wav, resid, grad = (rt.malloc(n) for n in (p.wavelet.size, p.nt * 9, p.vel.size))
+    s = rt.stream()
+    rt.log()
+    prop.gradient(wav, resid, grad, ckpt, dtype, stream=s)
+    assert all(e["stream"] != 0 for e in rt.log() if "stream" in e)
