@@ -319,6 +319,7 @@ MMOD_API mmod_status mmod_batch_create(mmod_handle *const *shots, int nshots, mm
         CKB(cudaStreamCreateWithFlags(&b->sub[k], cudaStreamNonBlocking));
         CKB(cudaEventCreateWithFlags(&b->join[k], cudaEventDisableTiming));
     }
+    CKB(cudaStreamSynchronize(cudaStreamLegacy));   // the tables are in place whatever stream the next call is on
 #undef CKB
     *out = b;
     return MMOD_OK;

@@ -1491,6 +1491,8 @@ MMOD_API mmod_status mmod_vd_create(const mmod_config *cfg, int device, mmod_vd 
     ok = ok && encode_box(&h->maps.k_own, h->kd, c.nx, c.ny, c.nz, h->nxp, t.tx, t.ty);
     cudaGetLastError();
     h->tma_ok = ok;
+    // the tables and cleared volumes are in place whatever stream the next call is on
+    VD_CREATE(cudaStreamSynchronize(cudaStreamLegacy), "tables");
 #undef VD_CREATE
     *out = h;
     return MMOD_OK;

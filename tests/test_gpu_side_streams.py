@@ -1,6 +1,6 @@
 """Handles used on a non-blocking stream while the default stream is busy: a run
 may rely on nothing that the default stream still has to do.  Tile shapes
-selected by variant and option right before the run; the same bits as
+selected by variant, option and batch mode right before the run; the same bits as
 on the default stream."""
 import numpy as np
 import pytest
@@ -47,3 +47,49 @@ def test_side_stream_bitwise(change):
     got = _run(p, torch.cuda.Stream(), change)
     for a, b in zip(got, ref):
         assert np.abs(b).max() > 0 and np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("mode", [M.BATCH_STREAMS, M.BATCH_FUSED, M.BATCH_PERSISTENT])
+def test_batch_on_a_side_stream_bitwise(mode):
+    torch = torch_cuda()
+    shots = [_problem(seed) for seed in (9, 10, 11)]
+    vel = [torch.from_numpy(p.vel).cuda() for p in shots]
+    wav = [torch.from_numpy(p.wavelet).cuda() for p in shots]
+    tr = [torch.empty((p.nt, 5000), device="cuda") for p in shots]
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    torch.cuda._sleep(40_000_000)
+    props = [M.Propagator.from_problem(p) for p in shots]
+    for prop, v in zip(props, vel):
+        prop.set_model(v, s.cuda_stream)
+    b = M.Batch(props)
+    b.set_mode(mode)
+    b.forward(wav, tr, s.cuda_stream)
+    torch.cuda.synchronize()
+    b.close()
+    for p, t in zip(shots, tr):
+        ref = _run(p, None, None)[0]
+        assert np.abs(ref).max() > 0 and np.array_equal(t.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("cpml", [False, True])
+def test_staggered_on_a_side_stream_bitwise(cpml):
+    torch = torch_cuda()
+    p = W.tiny_problem_vd(shape=(40, 100, 130), nt=40, nbl=8, nsrc=4, nrec=5000, seed=9)
+    p.cpml, p.cpml_f0 = cpml, 15.0 if cpml else 0.0
+    out = []
+    for stream in (None, torch.cuda.Stream()):
+        vel, rho, wav = (torch.from_numpy(a).cuda() for a in (p.vel, p.rho, p.wavelet))
+        tr = torch.empty((p.nt, 5000), device="cuda")
+        torch.cuda.synchronize()
+        s = None
+        if stream is not None:
+            s = stream.cuda_stream
+            torch.cuda._sleep(40_000_000)
+        prop = M.StaggeredPropagator.from_problem(p)
+        prop.set_model(vel, rho, s)
+        prop.forward(wav, tr, stream=s)
+        torch.cuda.synchronize()
+        prop.close()
+        out.append(tr.cpu().numpy())
+    assert np.abs(out[0]).max() > 0 and np.array_equal(out[0], out[1])

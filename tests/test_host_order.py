@@ -177,3 +177,24 @@ def test_first_gradient_fills_its_work_volumes_on_the_callers_stream(rt, scheme,
     rt.log()
     prop.gradient(wav, resid, grad, ckpt, dtype, stream=s)
     assert all(e["stream"] != 0 for e in rt.log() if "stream" in e)
+
+
+@pytest.mark.parametrize("make", ["batch", "vd", "vd_cpml"])
+def test_batches_and_staggered_handles_return_with_their_tables_in_place(rt, make):
+    if make == "batch":
+        props = [rt.propagator(_problem(), model=False)]
+        rt.log()
+        rt.batch(props)
+    else:
+        p = W.tiny_problem_vd(shape=(12, 30, 40), nt=16, nbl=4, nsrc=3, nrec=9, seed=3)
+        p.cpml, p.cpml_f0 = make == "vd_cpml", 15.0 if make == "vd_cpml" else 0.0
+        rt.log()
+        rt.open.append(M.StaggeredPropagator.from_problem(p))
+    last = {}
+    log = rt.log()
+    for i, e in enumerate(log):
+        if e["op"] in ("memset", "memcpy"):
+            last[e["stream"]] = i
+    assert last
+    for stream, i in last.items():
+        assert any(e["op"] == "sync" and e["stream"] == stream for e in log[i:]), stream
