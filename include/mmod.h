@@ -420,11 +420,15 @@ mmod_status mmod_batch_destroy(mmod_batch *b);
 mmod_status mmod_batch_forward(mmod_batch *b, const float *const *wavelets, float *const *traces,
                                mmod_stream stream);
 
-/* Select the TMA variant used by the batch (see mmod_tma_variant_count); in
- * streams mode it is set on every handle of the batch. */
+/* Select the TMA variant used by the batch: one with fused kernels, i.e. with
+ * 64 x 16 tiles (0 to 8; ARG otherwise).  In streams mode it is set on every
+ * handle of the batch, except that variant 2, the form which every tile shape is
+ * compiled in, leaves each handle the tile shape of its own grid
+ * (mmod_set_tma_variant -1).  Errors: ARG, OOM, CUDA. */
 mmod_status mmod_batch_set_variant(mmod_batch *b, int v);
 
-/* MMOD_BATCH_STREAMS or MMOD_BATCH_FUSED.  Errors: ARG. */
+/* MMOD_BATCH_STREAMS, MMOD_BATCH_FUSED or MMOD_BATCH_PERSISTENT.  Errors: ARG,
+ * OOM, CUDA. */
 enum { MMOD_BATCH_STREAMS = 0, MMOD_BATCH_FUSED = 1, MMOD_BATCH_PERSISTENT = 2 };
 mmod_status mmod_batch_set_mode(mmod_batch *b, int mode);
 
@@ -436,7 +440,9 @@ const char *mmod_batch_last_error(const mmod_batch *b);
  * Times every compiled TMA variant (points per thread, z-window unroll,
  * ring depths) for `steps` time steps on the handle's (or batch's) own grids
  * and model, without sources, and selects the fastest; *variant_out (may be
- * NULL) receives it.  Synchronises `stream`; overwrites the wavefields.
+ * NULL) receives it.  A batch is tuned over the variants that
+ * mmod_batch_set_variant takes, and what it finds can be set again with that
+ * call.  Synchronises `stream`; overwrites the wavefields.
  * Errors: ARG, STATE (no model), UNSUPPORTED, CUDA. */
 mmod_status mmod_autotune(mmod_handle *h, int steps, mmod_stream stream, int *variant_out);
 mmod_status mmod_batch_autotune(mmod_batch *b, int steps, mmod_stream stream, int *variant_out);

@@ -128,6 +128,16 @@ mmod_status enqueue_batch_steps(mmod_batch *b, int n0, int n1, cudaStream_t s) {
     return MMOD_OK;
 }
 
+// Variant v on every shot's own loop.  The default variant is the form that every
+// tile shape is compiled in, and stands for it in the shape that suits each
+// shot's grid: no single shape was faster for a whole batch.  ms, own shapes /
+// 64 x 16 / the best single shape: 32 uneven shots x 800 steps 603 / 612 / 605, 6 of
+// 160^3 x 200 12.0 / 13.6 / 12.0, 4 uneven of about 130^3 x 200 6.05 / 6.37 / 6.13; 16
+// of 64^3 and 8 of 128^3 equal.
+void set_shot_variants(mmod_batch *b, int v) {
+    for (mmod_handle *h : b->shots) h->variant = v == kTmaDefaultVariant ? -1 : v;
+}
+
 // The maps and arguments of the fused and persistent kernels (64 x 16 tiles).
 mmod_status fill_desc(mmod_batch *b) {
     for (size_t i = 0; i < b->shots.size(); ++i) {
@@ -347,7 +357,7 @@ MMOD_API mmod_status mmod_batch_set_variant(mmod_batch *b, int v) {
         if (mmod_status st = ensure_shape(h, 0)) return bfail(b, st, h->err);
     b->variant = v;
     b->variant_set = true;
-    for (mmod_handle *h : b->shots) h->variant = v;   // streams mode runs each handle's own plan
+    set_shot_variants(b, v);   // streams mode runs each handle's own plan
     return MMOD_OK;
 }
 
@@ -527,7 +537,8 @@ MMOD_API mmod_status mmod_batch_autotune(mmod_batch *b, int steps, mmod_stream s
         float best_ms = 1e30f;
         mmod_status st = MMOD_OK;
         for (int v = 0; v < tma_variant_count() && st == MMOD_OK; ++v) {
-            for (mmod_handle *h : b->shots) h->variant = v;
+            if (!tma_variant_has_batch(v)) continue;   // what mmod_batch_set_variant takes
+            set_shot_variants(b, v);
             float ms = -1.0f;
             for (int rep = 0; rep < 2 && st == MMOD_OK; ++rep) {   // the first repetition warms up
                 if (cudaEventRecord(e0, s) != cudaSuccess) st = MMOD_ERR_CUDA;
@@ -546,9 +557,9 @@ MMOD_API mmod_status mmod_batch_autotune(mmod_batch *b, int steps, mmod_stream s
         }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
-        for (mmod_handle *h : b->shots) h->variant = best;
+        set_shot_variants(b, best);
         if (st != MMOD_OK) return bfail(b, st, "autotuning the batch failed");
-        if (tma_variant_has_batch(best)) b->variant = best;   // the fused mode's kernels: 64 x 16 tiles only
+        b->variant = best;
         b->variant_set = true;
         if (variant_out) *variant_out = best;
         return MMOD_OK;

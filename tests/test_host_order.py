@@ -198,3 +198,29 @@ def test_batches_and_staggered_handles_return_with_their_tables_in_place(rt, mak
     assert last
     for stream, i in last.items():
         assert any(e["op"] == "sync" and e["stream"] == stream for e in log[i:]), stream
+
+
+@pytest.mark.parametrize("mode", [M.BATCH_STREAMS, M.BATCH_FUSED])
+@pytest.mark.parametrize("fast", ["StagedILi48", "StagedILi40", "StagedILi32", "StagedILi64", "5ShapeILi16ELi2ELi1"])
+def test_a_tuned_batch_variant_can_be_set_again(rt, fast, mode):
+    """Whatever kernel turns out fastest, the number that tuning returns is taken by
+    set_variant and selects what tuning left selected."""
+    props = [rt.propagator(_problem(shape=shape)) for shape in ((64, 64, 64), (40, 100, 130))]
+
+    def variants():
+        return [pr.plan()["variant"] for pr in props]
+
+    own = variants()
+    assert own == [2, 9]
+    b = rt.batch(props)
+    b.set_mode(mode)
+    rt.lib.fake_fast_kernel(fast.encode())
+    v = b.autotune(steps=3)
+    tuned = variants()
+    b.set_variant(v)
+    if mode == M.BATCH_STREAMS:   # tuning the fused kernels leaves the shots' own loops alone
+        assert variants() == tuned and (v == 2 or fast != "StagedILi48")
+    b.set_variant(5)
+    assert variants() == [5, 5]
+    b.set_variant(2)   # the default form: each shot in its own tile shape
+    assert variants() == own
