@@ -307,6 +307,7 @@ cudaError_t restore_state(mmod_handle *h, int slot, float *u_prev, float *u_cur,
 mmod_status encode_grad_maps(mmod_handle *h, int shape) {
     auto &gw = h->gw;
     if (gw.shape == shape || !h->tma_ok) return MMOD_OK;
+    gw.shape = -1;   // until every map is one of this shape
     bool ok = true;
     for (int i = 0; i < gw.nwork; ++i) ok = ok && encode_maps(h->cfg, h->nxp, gw.seg[i], shape, &gw.seg_map[i]);
     for (int b = 0; b < 2; ++b) ok = ok && encode_maps(h->cfg, h->nxp, gw.psi[b], shape, &gw.psi_map[b]);

@@ -224,3 +224,35 @@ def test_a_tuned_batch_variant_can_be_set_again(rt, fast, mode):
     assert variants() == [5, 5]
     b.set_variant(2)   # the default form: each shot in its own tile shape
     assert variants() == own
+
+
+@pytest.mark.parametrize("dtype", [M.CKPT_FP32, M.CKPT_BF16])
+@pytest.mark.parametrize("nth", range(1, 9))
+def test_work_volume_maps_after_a_failed_change_of_tiles(rt, nth, dtype):
+    """The work volumes' tensor maps are encoded anew for another tile shape; if that
+    fails half way, a later run in the old shape must not use what was encoded."""
+    prop = rt.propagator(_problem(shape=(40, 100, 130)))
+    wav, resid, grad = (rt.malloc(n) for n in (2 * 16, 16 * 9, 40 * 100 * 130))
+
+    def gradient():
+        prop.gradient(wav, resid, grad, 8, dtype)
+
+    prop.set_variant(9)
+    gradient()
+    prop.set_variant(10)
+    prop.set_variant(9)   # both shapes of the handle's own volumes are set up
+    prop.set_variant(10)
+    rt.lib.fake_fail_encode(0, 0, nth)
+    with pytest.raises(M.MmodError):
+        gradient()
+    rt.lib.fake_fail_encode(0, 0, 0)
+    prop.set_variant(9)
+    rt.log()
+    gradient()
+    boxes = {}
+    for e in rt.log():
+        if e["op"] == "encode":
+            boxes[e["map"]] = tuple(e["box"])
+    # every map overwritten for the 40 x 24 tiles is one of the 48 x 20 tiles again
+    assert len(boxes) >= nth - 1 and set(boxes.values()) <= {(56, 28), (48, 20)}
+    assert {(56, 28), (48, 20)} <= set(boxes.values())
