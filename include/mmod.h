@@ -253,8 +253,8 @@ mmod_status mmod_set_kernel(mmod_handle *h, int kernel);
 /* Compiled variants of the TMA kernel (tile shape, points per thread, z
  * queue handling), for tuning.  mmod_tma_variant_name returns a static
  * description ("" out of range).  mmod_set_tma_variant selects one for the
- * handle (-1 = automatic).  All variants produce the same bits.  Errors:
- * ARG (out of range), UNSUPPORTED (no TMA plan). */
+ * handle (-1 = automatic) and sets its tile shape up.  All variants produce the
+ * same bits.  Errors: ARG (out of range), UNSUPPORTED (no TMA plan), OOM, CUDA. */
 int mmod_tma_variant_count(void);
 /* Resources of variant v on the current device, 14 ints: threads per CTA,
  * dynamic shared bytes, then {registers per thread, local bytes per thread,
@@ -312,7 +312,8 @@ mmod_status mmod_set_tma_variant(mmod_handle *h, int v);
  *                         kernel returns and the call reports MMOD_ERR_TIMEOUT
  *                         (the handle stays in that state; the device and
  *                         other handles stay usable).
- * Errors: ARG (unknown option or value). */
+ * Errors: ARG (unknown option or value); OOM, CUDA where an option needs
+ * another tile shape set up. */
 enum { MMOD_OPT_PDL = 2, MMOD_OPT_CKPT_SCHEME = 3, MMOD_OPT_PERSISTENT = 4, MMOD_OPT_PERSISTENT_CTAS = 5,
        MMOD_OPT_TEST_STALL = 6, MMOD_OPT_ZLEN = 7, MMOD_OPT_CPML_PLANES = 8, MMOD_OPT_CLAIM = 9,
        MMOD_OPT_CPML_TILES = 10 };

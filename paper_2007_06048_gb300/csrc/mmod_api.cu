@@ -417,7 +417,7 @@ mmod_status ensure_shape(mmod_handle *h, int shape) {
     if (h->tma_ok) {
         bool ok = encode_maps(c, h->nxp, h->c, shape, &m.c);
         for (int b = 0; b < 2; ++b) ok = ok && encode_maps(c, h->nxp, h->u[b], shape, &m.u[b]);
-        if (!ok) return fail(h, MMOD_ERR_CUDA, "tensor map encoding failed");
+        if (!ok) return fail(h, MMOD_ERR_UNSUPPORTED, "the tensor maps of this tile shape cannot be encoded");
     }
     const TmaShape &sh = kTmaShapes[shape];
     try {
@@ -764,11 +764,17 @@ MMOD_API mmod_status mmod_create(const mmod_config *cfg, int device, mmod_handle
     if (is_cpml(h)) make_cpml_tiles(cpml_args(h), h->u, &h->cpml_tiles);   // axes it cannot tile keep the march
     h->tma_ok = make_tma_plan(h->cfg, h->plans);
     if (h->tma_ok) h->auto_variant = auto_tma_variant(h->plans);
-    if (ensure_shape(h, active_shape(h)) != MMOD_OK) {   // maps the encoder rejects: the plain kernel
-        h->tma_ok = false;
-        h->latched = cudaSuccess;
-        if (ensure_shape(h, 0) != MMOD_OK) return bail(cudaErrorMemoryAllocation, h->err.c_str());
+    // maps that the encoder rejects: the default tiles, then the plain kernel
+    st = ensure_shape(h, active_shape(h));
+    if (st == MMOD_ERR_UNSUPPORTED) {
+        h->auto_variant = kTmaDefaultVariant;
+        st = ensure_shape(h, active_shape(h));
     }
+    if (st == MMOD_ERR_UNSUPPORTED) {
+        h->tma_ok = false;
+        st = ensure_shape(h, 0);
+    }
+    if (st != MMOD_OK) return bail(st == MMOD_ERR_OOM ? cudaErrorMemoryAllocation : h->latched, "injection tables");
     if (h->tma_ok) {   // counters of the persistent kernel, sized for the plan with the most units
         for (int v = 0; v < tma_variant_count(); ++v)
             h->ncounters = std::max<long long>(h->ncounters, (long long)h->plans[v].tiles_x * h->plans[v].tiles_y *

@@ -256,3 +256,40 @@ def test_work_volume_maps_after_a_failed_change_of_tiles(rt, nth, dtype):
     # every map overwritten for the 40 x 24 tiles is one of the 48 x 20 tiles again
     assert len(boxes) >= nth - 1 and set(boxes.values()) <= {(56, 28), (48, 20)}
     assert {(56, 28), (48, 20)} <= set(boxes.values())
+
+
+def _step_kernels(rt, prop, p):
+    rt.log()
+    prop.forward(rt.malloc(p.wavelet.size), rt.malloc(p.nt * 9))
+    names = {e["name"] for e in rt.log() if e["op"] == "launch"}
+    return {n for n in names if "step_tma_kernel" in n or "step_simple_kernel" in n}
+
+
+@pytest.mark.parametrize("box", [(56, 28), (48, 20)])
+def test_create_falls_back_to_the_default_tiles(rt, box):
+    """Tile shapes whose maps cannot be encoded give way to 64 x 16, not to the plain kernel."""
+    p = _problem(shape=(40, 100, 130))
+    rt.lib.fake_fail_encode(*box, 1)
+    prop = rt.propagator(p)
+    assert prop.plan()["variant"] == 2
+    kernels = _step_kernels(rt, prop, p)
+    assert kernels and all("StagedILi64" in k for k in kernels)
+    with pytest.raises(M.MmodError) as ei:   # the shape itself stays refused, and selecting it changes nothing
+        prop.set_variant(9)
+    assert ei.value.status == -7 and prop.plan()["variant"] == 2
+
+
+def test_create_falls_back_to_the_plain_kernel(rt):
+    p = _problem(shape=(40, 100, 130))
+    rt.lib.fake_fail_encode(0, 0, 1)
+    prop = rt.propagator(p)
+    kernels = _step_kernels(rt, prop, p)
+    assert kernels and all("step_simple_kernel" in k for k in kernels)
+
+
+@pytest.mark.parametrize("entries", [40 * 3 * 5 + 1, 40 * 3 * 7 + 1])   # bucket starts of 48 x 20 and of 64 x 16 tiles
+def test_create_reports_memory_that_is_missing_for_tables(rt, entries):
+    rt.lib.fake_fail_malloc(4 * entries)
+    with pytest.raises(M.MmodError) as ei:
+        rt.propagator(_problem(shape=(40, 100, 130)))
+    assert M.STATUS[ei.value.status].endswith("OOM")
