@@ -147,7 +147,7 @@ mmod_status mmod_adjoint(mmod_handle *h, const float *resid, float *adj_src, mmo
  * plane, rounded to BF16 / FP16 (one FP32 scale per plane).
  * MMOD_CKPT_BFP16: block floating point, one FP32 scale s = max |u| over each
  * block of 32 consecutive x values and round(u * 32767 / s) as int16 per
- * value (error <= s / 65534; 2.125 bytes per value). */
+ * value (error <= s / 65534; 2.125 bytes per value); s is at least 2^-111. */
 enum { MMOD_CKPT_FP32 = 0, MMOD_CKPT_BF16 = 1, MMOD_CKPT_FP16 = 2, MMOD_CKPT_BFP16 = 3 };
 
 /* Gradient of J = 1/2 sum_n |traces^n - d_obs^n|^2 with respect to the

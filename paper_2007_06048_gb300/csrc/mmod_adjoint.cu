@@ -172,12 +172,16 @@ __global__ void __launch_bounds__(256) decompress_kernel(const CkptPair<T> p, lo
 // values of a padded row (rows are padded to 32, so blocks never straddle
 // rows), scale s = max |u| over the block and q = round(u * 32767 / s) as
 // int16; u is restored as q * (s / 32767), within s / 65534 of the stored
-// value.  Four threads per block, eight values each (16-byte accesses).
+// value.  s is at least kBfpMin, 2^15 times the smallest normal number, so that
+// 32767 / s and s / 32767 are finite and normal (below it, the far tail of a wave
+// was stored as +-s).  Four threads per block, eight values each (16-byte
+// accesses).
 constexpr int kBfpBlock = 32;
 constexpr float kBfpMax = 32767.0f;
+constexpr float kBfpMin = 32768.0f * FLT_MIN;
 
-__device__ __forceinline__ short bfp_value(float v, float m) {
-    return m > 0.0f ? (short)max(-32767, min(32767, __float2int_rn(v * (kBfpMax / m)))) : (short)0;
+__device__ __forceinline__ short bfp_value(float v, float s) {
+    return (short)max(-32767, min(32767, __float2int_rn(v * (kBfpMax / s))));
 }
 
 __global__ void __launch_bounds__(256) compress_bfp_kernel(const CkptPair<short> p, long long nblocks) {
@@ -195,6 +199,7 @@ __global__ void __launch_bounds__(256) compress_bfp_kernel(const CkptPair<short>
                         fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fmaxf(fabsf(b.z), fabsf(b.w))));
         m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
         m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        if (m < kBfpMin) m = kBfpMin;   // not a block of NaN
         if (!in) continue;
         out[g] = make_uint4(pack2(bfp_value(a.x, m), bfp_value(a.y, m)), pack2(bfp_value(a.z, m), bfp_value(a.w, m)),
                             pack2(bfp_value(b.x, m), bfp_value(b.y, m)), pack2(bfp_value(b.z, m), bfp_value(b.w, m)));
