@@ -113,11 +113,10 @@ void free_all(mmod_handle *h) {
     if (h->err_host) cudaFreeHost(h->err_host);
 }
 
-// Tables go up on a stream of the handle's own, which the functions below wait
-// for while the host vectors live: whatever stream the next run is on, they are
-// in place.  (On the legacy stream a copy from pageable memory may return before
-// its last transfer has landed, and nothing orders that stream before a
-// non-blocking one.)
+// The functions below wait for the stream that their tables go up on while the
+// host vectors live: whatever stream the next run is on, the tables are in place.
+// (A copy from pageable memory may return before its last transfer has landed,
+// and nothing orders the legacy stream before a non-blocking one.)
 template <class T>
 cudaError_t upload(T **dst, const std::vector<T> &v, cudaStream_t s) {
     const size_t n = std::max<size_t>(v.size(), 1);
@@ -716,8 +715,10 @@ MMOD_API mmod_status mmod_create(const mmod_config *cfg, int device, mmod_handle
     } while (0)
 
     const size_t vbytes = sizeof(float) * (size_t)h->vol;
-    CKC(cudaStreamCreateWithFlags(&h->st_copy, cudaStreamNonBlocking));
-    cudaStream_t up = h->st_copy;
+    // The legacy stream, waited for below.  A stream of the handle's own, made
+    // before the volumes, moved where later allocations land: staggered 176 x 150 x
+    // 123 steps 1.5 % slower, 64^3 ones 0.4 %.
+    cudaStream_t up = cudaStreamLegacy;
     CKC(cudaMalloc(&h->u[0], vbytes));
     CKC(cudaMalloc(&h->u[1], vbytes));
     CKC(cudaMalloc(&h->c, vbytes));
@@ -753,6 +754,7 @@ MMOD_API mmod_status mmod_create(const mmod_config *cfg, int device, mmod_handle
     CKC(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
     CKC(cudaEventCreate(&h->ev_t0));
     CKC(cudaEventCreate(&h->ev_t1));
+    CKC(cudaStreamCreateWithFlags(&h->st_copy, cudaStreamNonBlocking));
     CKC(cudaEventCreateWithFlags(&h->ev_copied, cudaEventDisableTiming));
     for (int i = 0; i < mmod_handle::kTraceChunks; ++i) {
         CKC(cudaEventCreateWithFlags(&h->ev_rows[i], cudaEventDisableTiming));

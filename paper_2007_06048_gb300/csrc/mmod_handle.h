@@ -90,7 +90,7 @@ struct mmod_handle {
     static constexpr int kTraceChunks = 8;
     cudaEvent_t ev_rows[kTraceChunks] = {};
     long long rows_at[kTraceChunks] = {};
-    cudaStream_t st_copy = nullptr;     // also uploads the tables at set-up
+    cudaStream_t st_copy = nullptr;     // also uploads the tables of a tile shape
     cudaEvent_t ev_copied = nullptr;
     mmod::GraphSlot g_fwd, g_adj;
 
