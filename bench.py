@@ -543,7 +543,8 @@ def measure_batched(M, dev, stream, fwd_gpts, reps=3):
             "fused_variant": M.mmod_tma_variant_name(fused_variant),
             "shots": len(shots), "nt": shots[0].nt,
             "points": int(sum(p.npoints for p in shots)), "variant": M.mmod_tma_variant_name(variant),
-            "what": "mmod_batch_forward, streams mode: the shots' graphs overlap on two or four streams; "
+            "what": "mmod_batch_forward, streams mode: the shots' graphs overlap on two or four streams, and "
+                    "variant 2 runs each shot in its own tile shape; "
                     "fused: one launch per step for all shots; persistent: one cooperative launch for every "
                     "shot's whole loop"}
 

@@ -302,7 +302,7 @@ mmod_status mmod_set_tma_variant(mmod_handle *h, int v);
  *   MMOD_OPT_CPML_TILES   0 / 1 (default 1): run the CPML layer pass of an
  *                         axis as tiles of 128 lines loaded whole into shared
  *                         memory by bulk-tensor copies, where the axis allows
- *                         it (layer width 8 or 20, the two layer ranges
+ *                         it (layer width 8, 12, .. 32, the two layer ranges
  *                         apart; along x also nx a multiple of 4); 0: the
  *                         marching passes only.  The same bits either way;
  *   MMOD_OPT_TEST_STALL   1: test hook of the failure path.  The next
@@ -390,7 +390,7 @@ mmod_status mmod_forward_noalloc(const mmod_config *cfg, int device, const float
 
 /* ---- Batched shots ------------------------------------------------------
  * A batch advances several shots (one handle each: any grid sizes, the same
- * nt, the same device) together, in one of two modes (mmod_batch_set_mode):
+ * nt, the same device) together, in one of three modes (mmod_batch_set_mode):
  *   MMOD_BATCH_STREAMS (default): each shot's own time loop (the handle's
  *     graph of one-step kernels) on one of two internal streams (four for
  *     small grids) forked from and joined back to the caller's stream, so the
@@ -402,7 +402,7 @@ mmod_status mmod_forward_noalloc(const mmod_config *cfg, int device, const float
  *     step once the neighbouring units of its shot have finished the
  *     previous one (per-unit counters, waits bounded at 100 ms: a give-up
  *     is reported as MMOD_ERR_TIMEOUT); TMA variants 2 and 5 only.
- * Both give every shot the bits it gets alone.  The batch refers to the
+ * Each gives every shot the bits it gets alone.  The batch refers to the
  * handles (they keep their buffers, models and geometry); destroy the batch
  * before its handles.  Each handle's buffers hold its shot's final state
  * after mmod_batch_forward (mmod_get_state). */

@@ -69,11 +69,11 @@ __global__ void source_scale_kernel(const float *__restrict__ vel, int nx, int n
     scale[t] = (float)(dt * dt * v * v / cell);
 }
 
-// Dense <-> padded copies and the gradient's scaling: one warp per row, so
-// no index divisions, and 16-byte accesses where both sides' rows start on
-// 16-byte boundaries (V = 4: nx a multiple of 4 and an aligned dense array;
-// padded rows always are).  Bound by memory; with one thread per point and two
-// 64-bit divisions, unpacking 240^3 took 35 us (3.2 TB/s).
+// Dense <-> padded copies: one warp per row, so no index divisions, and 16-byte
+// accesses where both sides' rows start on 16-byte boundaries (V = 4: nx a
+// multiple of 4 and an aligned dense array; padded rows always are).  Bound by
+// memory; with one thread per point and two 64-bit divisions, unpacking 240^3
+// took 35 us (3.2 TB/s).
 template <int V>
 struct Vec;
 template <>

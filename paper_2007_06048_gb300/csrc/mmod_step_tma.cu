@@ -2,24 +2,33 @@
 // whole grid (inner region, damping layers, source add) and gathers the
 // receivers of the previous step.
 //
-// Decomposition.  A CTA owns a 64 x TY tile in (x, y) and a range of planes in
-// z, and marches down z.  Each thread owns 2 (x) x RY (y) points: lane l holds
-// columns x0+2l, x0+2l+1, warp w rows y0+RY*w .. y0+RY*w+RY-1.
+// Two forms of the plane pipeline share this file's launches, dependencies and
+// options: the staged form (step_staged.cuh), which every run takes unless a
+// caller selects another variant, in four tile shapes (variants 2 and 9 to 11);
+// and the ring form below (variants 0, 1 and 3 to 8), slower in every
+// measurement since the staged form exists, which a caller may still select and
+// which the tuners time.
 //
-// Data movement.  One elected thread issues cp.async.bulk.tensor loads:
+// Decomposition.  A CTA owns an x-y tile and a range of planes in z, and marches
+// down z.  In the ring form the tile is 64 x TY, and each thread owns 2 (x) x RY
+// (y) points: lane l holds columns x0+2l, x0+2l+1, warp w rows y0+RY*w ..
+// y0+RY*w+RY-1.
+//
+// Data movement.  One elected thread issues cp.async.bulk.tensor loads.  In the
+// ring form:
 //   * u^n planes with a 4-cell x-y halo, (64+8) x (TY+8) floats, into an
 //     S::NSU-slot ring.  The tensor map's zero fill outside the grid is exactly
 //     the u = 0 reading, so no thread tests bounds on loads.
 //   * u^{n-1} and c planes, 64 x TY floats each, into an S::NSC-slot ring.
 // Each slot has an mbarrier (transaction count = box bytes).  A slot is
 // refilled after the block barrier that ends the last step reading it, so
-// several planes per ring are in flight while the CTA computes.
+// several planes per ring are in flight while the CTA computes.  (The staged form
+// has one mbarrier per plane for all three operands.)
 //
 // Stencil.  x and y neighbours come from the centre plane in shared memory
 // (8-byte loads, conflict-free: a warp reads 64 consecutive floats per row);
-// z neighbours come from a register queue of 9 planes per point, either
-// shifted by one plane after every step (compact code) or rotated by
-// unrolling nine steps (no moves).  The two points of a thread share every
+// z neighbours come from a register queue of 8 planes and one group of U steps
+// per point, shifted by U planes after every group.  The two points of a thread share every
 // operation, so the arithmetic runs as packed FP32x2 (__ffma2_rn, __fadd2_rn:
 // per component the same rounding as the scalar intrinsics), except the x
 // offsets 1 and 3 whose operands do not form aligned register pairs.  The

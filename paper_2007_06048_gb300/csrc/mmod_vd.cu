@@ -1261,8 +1261,8 @@ mmod_status vd_loop(mmod_vd *h, const float *wav, float *tr, cudaStream_t s, lon
 // wins, and of those the one with the fewest CTAs; 64 x 16 gives way on equal
 // planes only to 48 x 20 tiles of the same number (40 x 24 ones lost 5 % there:
 // 105 x 45 x 118 15.8 / 16.6 us per step, 110 x 84 x 221 28.5 / 28.6 with everything
-// else 5 % faster).  Measured, 64 x 16 against the
-// choice (us per step, damping): 96^3 15.5 / 13.1 (32 x 32), 144^3 36.9 / 31.9 (48 x
+// else 5 % faster).  That tie rule has thin support: 240^3 is the one measured
+// grid that gains by it.  Measured, 64 x 16 against the choice (us per step, damping): 96^3 15.5 / 13.1 (32 x 32), 144^3 36.9 / 31.9 (48 x
 // 20), 160^3 41.0 / 35.7 (32 x 32), 200^3 96.9 / 88.4 (40 x 24), 240^3 136.3 / 134.3 (48
 // x 20), 77 x 210 x 64 23.0 / 17.2 (40 x 24); on equal planes and other counts it is
 // the better one (112^3 19.8 against 20.7, 100 x 220 x 180 47.7 against 48.2).

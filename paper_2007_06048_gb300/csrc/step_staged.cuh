@@ -35,11 +35,12 @@
 // Bound by DRAM on large grids and by the pipeline's latencies on one-wave
 // grids.  us per step, ring form -> staged: 64^3 4.47 -> 3.83, 128^3 8.68 ->
 // 7.89, 200^3 34.98 -> 32.35, 240^3 41.96 -> 41.20, 512^3 337.0 -> 325.5 (6.60
-// TB/s); 110 registers instead of 120.  Then, with the tensor maps prefetched,
+// TB/s).  Then, with the tensor maps prefetched,
 // u^n requested ahead of the block barrier, and the source and receiver
 // look-ups taken off the critical path (they were dependent loads right after
 // the wait and at the end): 64^3 3.83 -> 3.58, 151 x 117 x 98 7.8 -> 7.4, 240^3 39.4
-// -> 38.8.
+// -> 38.8.  122 registers (123 with g^n, 106 to 108 in the imaging form, 128 in the
+// claiming and persistent kernels), no spills.
 // PITCH, the halo tile's row pitch, is chosen so that a half-warp whose lanes
 // span two row pairs reads 16 different bank pairs: 2 PITCH = TX (mod 32).
 #pragma once
