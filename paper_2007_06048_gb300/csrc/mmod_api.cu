@@ -619,8 +619,10 @@ mmod_status run_loop_graph(mmod_handle *h, GraphSlot &g, const Geometry &geo, co
         return MMOD_OK;
     }
     const int kern = use_tma(h) ? 100 + active_plan(h).variant : MMOD_KERNEL_SIMPLE;
-    const long long opts = h->pdl + 2LL * h->zlen_override + (1LL << 20) * h->claim_planes +
-                           (1LL << 40) * h->cpml_planes;
+    // the options a captured loop depends on, each in bits of its own: 1, 1, 21
+    // (0 .. 2^20), 13 (0 .. 4096), and the z range last
+    const long long opts = h->pdl | h->cpml_tiles_on << 1 | (long long)h->claim_planes << 2 |
+                           (long long)h->cpml_planes << 23 | (long long)std::min(h->zlen_override, h->cfg.nz) << 36;
     // whether the rows are recorded is part of the key: the staging buffer may
     // get the address of device traces that an earlier loop was captured for
     const void *key[4] = {wav, tr, &geo, records_rows(h, geo, tr) ? h->ev_rows : nullptr};

@@ -286,3 +286,22 @@ def test_create_reports_memory_that_is_missing_for_tables(rt, entries):
     with pytest.raises(M.MmodError) as ei:
         rt.propagator(_problem(shape=(40, 100, 130)))
     assert M.STATUS[ei.value.status].endswith("OOM")
+
+
+@pytest.mark.parametrize("first,second", [({M.OPT_CPML_TILES: 1}, {M.OPT_CPML_TILES: 0}),
+                                          ({M.OPT_ZLEN: 1 << 19}, {M.OPT_ZLEN: 0, M.OPT_CLAIM: 1}),
+                                          ({M.OPT_CLAIM: 1 << 20}, {M.OPT_CLAIM: 0, M.OPT_CPML_PLANES: 1}),
+                                          ({M.OPT_PDL: 0}, {M.OPT_PDL: 1}), ({M.OPT_ZLEN: 4}, {M.OPT_ZLEN: 5})])
+def test_an_option_changed_between_runs_takes_effect(rt, first, second):
+    """Every option that the captured loop depends on makes the next run capture anew."""
+    p = _problem()
+    p.cpml, p.cpml_f0, p.nbl = True, 15.0, 4
+    prop = rt.propagator(p)
+    prop.set_variant(2)   # the same kernel throughout
+    wav, tr = rt.malloc(p.wavelet.size), rt.malloc(p.nt * 9)
+    for options, captures in ((first, 1), (first, 0), (second, 1), (second, 0)):
+        for o, v in options.items():
+            prop.set_option(o, v)
+        rt.log()
+        prop.forward(wav, tr)
+        assert len([e for e in rt.log() if e["op"] == "begin_capture"]) == captures
