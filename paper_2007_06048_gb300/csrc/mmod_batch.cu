@@ -614,7 +614,12 @@ MMOD_API mmod_status mmod_autotune(mmod_handle *h, int steps, mmod_stream stream
         float ms = 0.0f;
         for (int rep = 0; rep < 2; ++rep) {   // the first repetition warms up
             MMOD_CK(h, cudaEventRecord(e0, s));
-            if (mmod_status st = enqueue_tune_steps(h, steps, s)) return st;
+            const mmod_status st = enqueue_tune_steps(h, steps, s);
+            if (st == MMOD_ERR_UNSUPPORTED) {   // a tile shape that cannot be set up here
+                ms = best_ms;
+                break;
+            }
+            if (st != MMOD_OK) return st;
             MMOD_CK(h, cudaEventRecord(e1, s));
             MMOD_CK(h, cudaEventSynchronize(e1));
             MMOD_CK(h, cudaEventElapsedTime(&ms, e0, e1));

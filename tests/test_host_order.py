@@ -305,3 +305,14 @@ def test_an_option_changed_between_runs_takes_effect(rt, first, second):
         rt.log()
         prop.forward(wav, tr)
         assert len([e for e in rt.log() if e["op"] == "begin_capture"]) == captures
+
+
+def test_tuning_skips_tiles_that_cannot_be_set_up(rt):
+    """A handle that fell back to the default tiles can still be tuned, and runs afterwards."""
+    p = _problem(shape=(40, 100, 130))
+    rt.lib.fake_fail_encode(48, 20, 1)
+    prop = rt.propagator(p)
+    rt.lib.fake_fast_kernel(b"StagedILi40")
+    assert prop.autotune(steps=3) == 10
+    kernels = _step_kernels(rt, prop, p)
+    assert kernels and all("StagedILi40" in k for k in kernels)
